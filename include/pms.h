@@ -65,7 +65,13 @@ typedef struct {
     size_t count;           /* number of motifs (raw count on PMS_ETOOMANY) */
 } pms_result;
 
-/* Tunables. Zero in any field selects the default (or the tuned value). */
+/* Tunables. Zero in any field selects the default (or the tuned value).
+ * A solve takes one of two forms of the search with the same answer: the tree
+ * over B(x, d) of every seed, or the sieve (every window marks the strings
+ * within d of it in a bit map of all 4^l; l <= 16), whichever is estimated to
+ * be faster for its n, m, l, d and quorum. Setting chunk_work, grab,
+ * count_work, smem_rows, seed_mode, partial_rows or triple_rows selects the
+ * tree form, which these fields describe. */
 typedef struct {
     int ctas_per_sm;       /* resident CTAs of the verification kernel per SM */
     int chunk_work;        /* target work of one queue item, in candidate units */
@@ -306,7 +312,7 @@ int pms_inject_fault(pms_ctx *h, int kind, int after, int count);
  * filter, work per queue item, CTAs per SM, node batch policy; the best is
  * kept in the context
  * for the class (l, d, n and m rounded up to powers of two) and used by every
- * later solve of that class, and copied to *out when out is non-null.
+ * later solve of that class that takes the tree form, and copied to *out when out is non-null.
  * pms_save_tuning / pms_load_tuning write / read the context's table as text
  * (one class per line). Options chunk_work / ctas_per_sm, when set,
  * override the tuned values. */

@@ -51,6 +51,8 @@ struct InstDev {
     uint32_t raw_cap;      // capacity of the raw motif buffer (power of two)
     int triple_rows;       // rows after the first whose occurrences are tested in pairs with the first
                            //   row's (three-string feasibility below a node); 0: no such test
+    int sieve_mid;         // sieve form: middle letters of a block (pms_sieve.cu); its window words (uint32)
+                           //   are then stored in place of the planes. 0: the tree form
 };
 
 // A contiguous range of queue items: chunks [chunk_lo, chunk_hi) of instance
@@ -153,6 +155,53 @@ const void *pack_kernel_fn();
 const void *sort_unique_kernel_fn();
 cudaError_t launch_probe(int kind, int iters, int blocks, unsigned long long *cycles, unsigned long long *sink,
                          cudaStream_t st);
+
+// Launch configuration of a programmatic dependent launch: the kernel may be
+// scheduled before the previous kernel in the stream has completed, and
+// waits for it with griddepcontrol.wait before touching its output. After a
+// copy, a memset or an event the stream orders it as usual.
+inline cudaLaunchConfig_t dependent_launch(cudaLaunchAttribute *attr, int blocks, int threads, size_t smem,
+                                           cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// ---------------------------------------------------------------- the sieve form (pms_sieve.cu)
+
+// The blocks of one instance in a sieve launch, from global item work_lo on.
+struct SieveSeg {
+    long long work_lo;
+    int inst;
+    int pad;
+};
+
+struct SieveParams {
+    const InstDev *inst;
+    const SieveSeg *seg;
+    int nseg;
+    long long total;              // blocks in this launch
+    unsigned long long *head;     // queue head (zeroed before the launch)
+    const uint2 *planes;          // instance plane_off: its window words
+    uint64_t *raw;
+    uint32_t *raw_count;
+    uint32_t *flags;
+};
+
+cudaError_t sieve_init_tables();
+// mid: middle letters of a block (3, 4, 5). planes: bits of the hit counters
+// of the quorum form (5 with mid 4, 7 with mid 3), 0 for q = n. share (q = n):
+// 1 a warp per block; 8 a CTA per block, its warps split every sequence's
+// windows (mid 5); 0 a CTA per block, its warps split the sequences (mid 3, 4).
+cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, int sms, cudaStream_t st);
 
 // ---------------------------------------------------------------- general alphabets (pms_sigma.cu)
 //

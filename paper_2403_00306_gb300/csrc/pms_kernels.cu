@@ -27,6 +27,7 @@
 //     motifs are appended with one atomic per warp, then sorted and
 //     de-duplicated per instance.
 #include "pms_internal.h"
+#include "pms_sieve.cuh"
 
 #include <algorithm>
 
@@ -2383,11 +2384,14 @@ __global__ void __launch_bounds__(256) compat_rows_kernel(const InstDev *__restr
     }
 }
 
-// Window planes for every (instance, sequence, window); flags bytes that are not A/C/G/T.
+// Window planes (sieve form: window words) for every (instance, sequence,
+// window); flags bytes that are not A/C/G/T.
 __global__ void pack_kernel(const InstDev *__restrict__ inst, int ninst, const long long *__restrict__ win_prefix,
                             long long total, const uint8_t *__restrict__ seqs, uint2 *__restrict__ planes,
                             uint32_t *__restrict__ flags)
 {
+    // a sieve kernel that follows may launch now; it waits for this grid
+    asm volatile("griddepcontrol.launch_dependents;");
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
          q += (long long)gridDim.x * blockDim.x) {
         int lo = 0, hi = ninst - 1;
@@ -2411,7 +2415,13 @@ __global__ void pack_kernel(const InstDev *__restrict__ inst, int ninst, const l
             h |= (code >> 1) << k;
             lo_bits |= (code & 1u) << k;
         }
-        planes[in.plane_off + local] = make_uint2(h, lo_bits);
+        if (in.sieve_mid == 0)
+            planes[in.plane_off + local] = make_uint2(h, lo_bits);
+        else
+            reinterpret_cast<uint32_t *>(planes + in.plane_off)[local] =
+                in.sieve_mid == 5   ? sieve_word<5>(h, lo_bits, in.l)
+                : in.sieve_mid == 4 ? sieve_word<4>(h, lo_bits, in.l)
+                                    : sieve_word<3>(h, lo_bits, in.l);
         if (bad)
             atomicOr(&flags[lo], kFlagInvalidByte);
     }
@@ -2659,7 +2669,8 @@ cudaError_t init_tables()
         e = cudaMemcpyToSymbol(c_digit, digit, sizeof(digit));
     if (e != cudaSuccess)
         return e;
-    return cudaMemcpyToSymbol(c_pow3, pow3, sizeof(pow3));
+    e = cudaMemcpyToSymbol(c_pow3, pow3, sizeof(pow3));
+    return e != cudaSuccess ? e : sieve_init_tables();
 }
 
 // Resident CTAs per SM each form's registers are bounded for: with 8-warp
@@ -2697,25 +2708,6 @@ cudaError_t main_occupancy(int *blocks_per_sm, bool count_mode, bool small_rows)
                           : occupancy_of<false, kRowSmemCapSmall, kMinBlocksSmall>(blocks_per_sm, smem);
     return count_mode ? occupancy_of<true, kRowSmemCap, kMinBlocksLarge>(blocks_per_sm, smem)
                       : occupancy_of<false, kRowSmemCap, kMinBlocksLarge>(blocks_per_sm, smem);
-}
-
-// Launch configuration of a programmatic dependent launch: the kernel may be
-// scheduled before the previous kernel in the stream has completed, and
-// waits for it with griddepcontrol.wait before touching its output. After a
-// copy, a memset or an event the stream orders it as usual.
-static cudaLaunchConfig_t dependent_launch(cudaLaunchAttribute *attr, int blocks, int threads, size_t smem,
-                                           cudaStream_t st)
-{
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cfg;
 }
 
 cudaError_t launch_main(const MainParams &p, int blocks, bool count_mode, cudaStream_t st, bool small_rows)

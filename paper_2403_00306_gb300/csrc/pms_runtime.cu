@@ -2,6 +2,7 @@
 // contexts, device-memory budget and arenas, plan building (queue chunks),
 // the plain / device-resident / batched solves and the served scheduler.
 #include "pms_internal.h"
+#include "pms_sieve.cuh"
 #include "../../include/pms.h"
 
 #include <algorithm>
@@ -99,6 +100,15 @@ uint64_t binom(int a, int b)
     return r;
 }
 
+// C(a, b) as a double (n up to 64 sequences).
+double choose(int a, int b)
+{
+    double r = 1;
+    for (int i = 1; i <= b; ++i)
+        r = r * (a - b + i) / i;
+    return r;
+}
+
 uint64_t ball_size(int l, int d)
 {
     uint64_t s = 0, p3 = 1;
@@ -176,6 +186,12 @@ ChunkTable make_chunks_k(int l, int d, int k)
 // ---------------------------------------------------------------------------------- context
 
 struct Served;
+
+// The form an instance is solved in: the sieve (mid > 0: middle letters,
+// counter planes and warps per block, see launch_sieve) or the tree (mid = 0).
+struct SieveForm {
+    int mid = 0, planes = 0, share = 1;
+};
 
 struct pms_ctx {
     int device = 0;
@@ -401,6 +417,10 @@ struct pms_ctx {
         double ms = 0;
     };
     std::map<std::tuple<int, int, int, int>, Tuning> tuned;
+    bool tuning_tree = false;   // the autotuner is timing the tree form
+    // sieve_form's estimates by (n, m, l, d, q, single), at most kMaxForms of them
+    static constexpr size_t kMaxForms = 1024;
+    mutable std::map<std::tuple<int, int, int, int, int, bool>, SieveForm> forms;
     static int bucket(int v)
     {
         int b = 1;
@@ -541,11 +561,20 @@ struct Plan {
     size_t seq_bytes = 0, planes = 0, raw = 0, compat = 0, rowlen = 0;
     int rows_cap = 1;
     uint64_t candidates = 0;
+    // sieve launches: one per (middle letters, counter planes) in use
+    struct SieveLaunch {
+        int mid, planes, share;
+        size_t seg_lo;       // its segments: [seg_lo, seg_lo + nseg) of sieve_seg
+        int nseg;
+        long long total;     // blocks
+    };
+    std::vector<SieveSeg> sieve_seg;
+    std::vector<SieveLaunch> sieve;
 };
 
 // Byte layout of the descriptor block (device d_meta, pinned h_meta).
 struct MetaLayout {
-    size_t inst, seg, win, rowp, seedp, segp, ctab, total;
+    size_t inst, seg, win, rowp, seedp, segp, ctab, sieve, total;
     MetaLayout(const Plan &p)
     {
         size_t o = 0;
@@ -563,20 +592,24 @@ struct MetaLayout {
         o = round_up(o + p.seg_pair.size() * sizeof(Segment), 16);
         ctab = o;
         o = round_up(o + p.ctab.size() * sizeof(int), 16);
+        sieve = o;
+        o = round_up(o + p.sieve_seg.size() * sizeof(SieveSeg), 16);
         total = o;
     }
 };
 
-// Counters block (d_ctr): head, work counters, dense_total, then per instance
+// Counters block (d_ctr): queue heads, work counters, dense_total, then per instance
 // raw_count and flags, then (items > 0) the steal cursor and the nodes claimed
 // of every queue item, for the verification kernel's work sharing.
+constexpr int kMaxSieveLaunches = 5;   // q = n with 3, 4 or 5 middle letters, the quorum form with 3 or 4
 struct CtrLayout {
-    size_t head, head_pair, work, dense_total, raw_count, flags, steal, claim, total;
+    size_t head, head_pair, head_sieve, work, dense_total, raw_count, flags, steal, claim, total;
     CtrLayout(size_t k, size_t items = 0)
     {
         head = 0;
         head_pair = 8;
-        work = 16;
+        head_sieve = 16;
+        work = head_sieve + 8 * kMaxSieveLaunches;
         dense_total = work + kCntNum * 8;
         raw_count = round_up(dense_total + 4, 16);
         flags = round_up(raw_count + 4 * k, 16);
@@ -673,6 +706,107 @@ static double expected_seed_rows(int n, int m, int l, int d)
     return (n - 1) * ((m - l + 1) * p + 3.0);
 }
 
+// The form with the smaller estimated time. Both estimates were fitted to
+// device times on one GB300 (n = 10 and 20, m = 200, 600, 1200, l = 8..16,
+// d = 1..5); they only choose, so what matters is where they cross.
+//   tree: W |B(x, d)| candidates at 250 E^2 ps each, E = expected_near: the more
+//     windows lie near a candidate, the fewer nodes fail. A quorum adds seeds
+//     and keeps nodes with misses. 38 us + 25 ns W for the launches, the masks
+//     and the slowest seeds of a single instance.
+//     Measured and (estimated), us: (15,4) m = 600 118 (136), m = 1000 562 (455);
+//     (14,4) 761 (700); (16,5) 5576 (5200); (13,4) 1704 (3300); (13,3) 54 (60).
+//   sieve: 4^A blocks, W windows and S sequences at 3.2 ps and 0.3 ps per word
+//     a window marks; S = n, or less when a block's strings run out sooner.
+//     A single instance with few blocks is bound by one block's latency.
+//     Measured and (estimated), us: (15,4) m = 600 192 (197), m = 1000 337 (375);
+//     (14,4) 135 (128); (16,5) 1156 (1160); (13,4) 174 (135); (13,3) 67 (63).
+// `single`: the only instance of its launch.
+static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int q, bool single)
+{
+    SieveForm f;
+    f.planes = q == n ? 0 : (n <= 31 && l >= 12 ? 5 : 7);
+    f.mid = q < n ? (f.planes == 5 ? 4 : 3) : (l <= 10 ? 3 : l == 11 || (!single && l == 12) ? 4 : 5);
+    const int A = l - f.mid - kSvSuf;
+    if (n < 2 || A < 0 || A > (f.mid == 5 ? sv_pre<5>() : f.mid == 4 ? sv_pre<4>() : sv_pre<3>()))
+        return SieveForm{};
+    const double W = m - l + 1, E = expected_near(m, l, d), p = 1.0 - std::exp(-E);
+    const double seeds = W * (n - q + 1);
+    // short motifs that most sequences hold: the answer is a good part of all
+    // 4^l strings, and writing it is what takes the time
+    if (l == 8 && E > 1.0)
+        return SieveForm{};
+    const double tree = seeds * (double)ball_size(l, d) * 250e-6 * E * E * (1.0 + 3.0 * (n - q)) +
+                        (single ? 38.0 + 0.025 * W : 0.0);
+    const double strings = std::pow(4.0, f.mid + kSvSuf), blocks = std::pow(4.0, A);
+    // sequences until a block holds fewer than two (quorum: no) strings that may still be motifs
+    int S = 1;
+    for (; S < n; ++S) {
+        double tail = 0;   // a string has S - (n - q) hits of S
+        for (int k = std::max(0, S - (n - q)); k <= S; ++k)
+            tail += choose(S, k) * std::pow(p, k) * std::pow(1.0 - p, S - k);
+        if (strings * tail < (q == n ? 2.0 : 0.5))
+            break;
+    }
+    const double words = (double)ball_size(l - kSvSuf, d) / (blocks * std::pow(4.0, f.mid));
+    const bool wide = q == n && single && l <= 13;   // few blocks: a CTA each
+    f.share = !wide ? 1 : (f.mid == 5 ? 8 : 0);
+    const double slots = 16.0 * h->num_sms;
+    const double rounded = single && !wide ? std::ceil(blocks / slots) * slots : blocks;
+    const double marks = rounded * W * S * (3.2 + 0.3 * words) * 1e-6;
+    double motifs = 0;
+    for (int k = q; k <= n; ++k)
+        motifs += choose(n, k) * std::pow(p, k) * std::pow(1.0 - p, n - k);
+    motifs *= std::pow(4.0, l);
+    // every motif is looked up in the seed sequences, by as many warps as have blocks
+    const double lookups = motifs * seeds * 14e-6 * (wide ? 1.0 : std::max(1.0, slots / blocks));
+    const double latency = !single ? 0.0 : f.share == 8 ? 12.0 + 0.085 * W : f.share == 0 ? 14.0 + 0.04 * W : 35.0;
+    const double sieve = (f.share == 8 ? std::max(latency, 25.0 + marks) : latency + marks) + lookups;
+    return sieve < tree ? f : SieveForm{};
+}
+
+// The form of one instance under the context's options: those that shape the
+// tree search, its work counters and its tuning keep the tree form. The
+// estimates are kept (they take about a microsecond, quorums ten).
+static SieveForm sieve_form(const pms_ctx *h, int n, int m, int l, int d, bool single)
+{
+    const pms_options &o = h->opt;
+    if (o.count_work || o.seed_mode || o.grab || o.smem_rows || o.partial_rows || o.triple_rows || o.chunk_work ||
+        h->tuning_tree)
+        return SieveForm{};
+    const int q = o.quorum > 0 && o.quorum < n ? o.quorum : n;
+    const auto key = std::make_tuple(n, m, l, d, q, single);
+    const auto it = h->forms.find(key);
+    if (it != h->forms.end())
+        return it->second;
+    if (h->forms.size() >= pms_ctx::kMaxForms)
+        h->forms.clear();
+    return h->forms[key] = estimate_form(h, n, m, l, d, q, single);
+}
+
+// Adds the sieve launches of the instances in sieve form.
+static void plan_sieve(Plan &P, const std::vector<SieveForm> &form)
+{
+    static const int forms[kMaxSieveLaunches][2] = {{5, 0}, {4, 0}, {3, 0}, {4, 5}, {3, 7}};
+    for (const auto &f : forms) {
+        std::vector<int> list;
+        for (size_t k = 0; k < P.inst.size(); ++k)
+            if (form[k].mid == f[0] && form[k].planes == f[1])
+                list.push_back((int)k);
+        if (list.empty())
+            continue;
+        // the costliest blocks first
+        std::stable_sort(list.begin(), list.end(), [&](int a, int b) {
+            return (long long)P.inst[a].n * P.inst[a].W > (long long)P.inst[b].n * P.inst[b].W;
+        });
+        Plan::SieveLaunch L{f[0], f[1], form[list[0]].share, P.sieve_seg.size(), (int)list.size(), 0};
+        for (int k : list) {
+            P.sieve_seg.push_back(SieveSeg{L.total, k, 0});
+            L.total += 1ll << (2 * (P.inst[k].l - f[0] - kSvSuf));
+        }
+        P.sieve.push_back(L);
+    }
+}
+
 static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
 {
     Plan P;
@@ -680,9 +814,12 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
     // their rows in its shared memory (seeds with more, such as those near the
     // planted copies, read their rows from the CTA's global scratch)
     P.small_rows = h->occ_small[0] > h->occ[0];
-    for (const InstSpec &s : specs)
-        if (expected_seed_rows(s.n, s.m, s.l, s.d) > kSmallFormRows)
+    std::vector<SieveForm> form;
+    for (const InstSpec &s : specs) {
+        form.push_back(sieve_form(h, s.n, s.m, s.l, s.d, specs.size() == 1));
+        if (form.back().mid == 0 && expected_seed_rows(s.n, s.m, s.l, s.d) > kSmallFormRows)
             P.small_rows = false;
+    }
     long long work = 0;
     const int adaptive = kDefaultChunkWork;   // untuned classes: about 2^20 candidate units per queue item
     bool quorum_used = false;
@@ -697,6 +834,8 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
         in.NW = (in.W + 31) / 32;
         in.q = (h->opt.quorum > 0 && h->opt.quorum < s.n) ? h->opt.quorum : s.n;
         in.nseed = s.n - in.q + 1;
+        in.sieve_mid = form[k].mid;
+        const bool tree = in.sieve_mid == 0;
         const long long seeds = (long long)in.nseed * in.W;
         const int cw = h->chunk_work_for(s.n, s.m, s.l, s.d);
         const ChunkTable &ct = h->chunks(s.l, s.d, cw > 0 ? cw : adaptive);
@@ -715,19 +854,25 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
         in.raw_cap = default_cap(h, s, specs.size() == 1);
         P.raw += in.raw_cap;
         in.compat_off = (long long)P.compat;
-        P.compat += (size_t)seeds * (s.n - 1) * in.NW;
+        P.compat += tree ? (size_t)seeds * (s.n - 1) * in.NW : 0;
         in.rlen_off = (long long)P.rowlen;
-        P.rowlen += (size_t)seeds * (s.n - 1);
+        P.rowlen += tree ? (size_t)seeds * (s.n - 1) : 0;
         P.win_prefix.push_back(P.total_windows);
         P.total_windows += (long long)s.n * in.W;
         P.row_prefix.push_back(P.total_rows);
-        P.total_rows += seeds * (s.n - 1);
+        P.total_rows += tree ? seeds * (s.n - 1) : 0;
         in.seed_off = P.total_seeds;
         P.seed_prefix.push_back(P.total_seeds);
         P.total_seeds += in.W;
         in.cps_b = (in.W + 63) / 64;
         P.seg_pair.push_back(Segment{P.total_pair_items, (int)k, 0, in.W * in.cps_b, 0});
         P.total_pair_items += (long long)in.W * in.cps_b;
+        P.candidates += (uint64_t)seeds * ball_size(s.l, s.d);
+        if (in.q < in.n)
+            quorum_used = true;
+        P.inst.push_back(in);
+        if (!tree)
+            continue;
         P.rows_cap = std::max(P.rows_cap, (int)round_up((size_t)(s.n - 1) * (in.W + 3), 4));
         const int chunks = (int)(seeds * in.cps);
         // one instance of whole-seed items whose last round would occupy only r
@@ -750,11 +895,8 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
             P.seg.push_back(Segment{work, (int)k, 0, chunks, 0, 0, 0});
             work += chunks;
         }
-        P.candidates += (uint64_t)seeds * ball_size(s.l, s.d);
-        if (in.q < in.n)
-            quorum_used = true;
-        P.inst.push_back(in);
     }
+    plan_sieve(P, form);
     P.total_items = work;
     P.pair_mode = h->opt.seed_mode == 1 && !quorum_used;   // pair seeds are for q = n
     return P;
@@ -779,9 +921,14 @@ static void record_event(const pms_ctx *h, cudaEvent_t ev, cudaStream_t st, bool
 // have the most unclaimed tree nodes).
 static int plan_blocks(const pms_ctx *h, const Plan &P, bool count_mode)
 {
-    const int occ = P.inst.empty()
-                        ? std::max(1, h->occ[count_mode ? 1 : 0])
-                        : plan_occ(h, P.inst[0].n, P.inst[0].m, P.inst[0].l, P.inst[0].d, count_mode, P.small_rows);
+    const InstDev *first = nullptr;
+    for (const InstDev &in : P.inst)
+        if (in.sieve_mid == 0) {
+            first = &in;
+            break;
+        }
+    const int occ = !first ? std::max(1, h->occ[count_mode ? 1 : 0])
+                           : plan_occ(h, first->n, first->m, first->l, first->d, count_mode, P.small_rows);
     return (int)std::min<long long>((long long)h->num_sms * occ, std::max<long long>(2 * P.total_items, 1));
 }
 
@@ -795,6 +942,7 @@ static void fill_meta(const Plan &P, const MetaLayout &ml, char *hm)
     std::memcpy(hm + ml.seedp, P.seed_prefix.data(), P.seed_prefix.size() * sizeof(long long));
     std::memcpy(hm + ml.segp, P.seg_pair.data(), P.seg_pair.size() * sizeof(Segment));
     std::memcpy(hm + ml.ctab, P.ctab.data(), P.ctab.size() * sizeof(int));
+    std::memcpy(hm + ml.sieve, P.sieve_seg.data(), P.sieve_seg.size() * sizeof(SieveSeg));
 }
 
 // Enqueues the whole pipeline of a plan on h->stream. d_seq_src: device
@@ -889,6 +1037,21 @@ static int enqueue_plan(pms_ctx *h, const Plan &P, const uint8_t *d_seq_src, Sta
     record_event(h, h->evm0, st, meta_dev != nullptr);
     if (P.total_items > 0 && (e = launch_main(mp, blocks, count_mode, st, P.small_rows)) != cudaSuccess)
         return h->cuda_fail(e, "verification kernel");
+    for (size_t j = 0; j < P.sieve.size(); ++j) {
+        const Plan::SieveLaunch &L = P.sieve[j];
+        SieveParams sp{};
+        sp.inst = d_inst;
+        sp.seg = (const SieveSeg *)(dm + ml.sieve) + L.seg_lo;
+        sp.nseg = L.nseg;
+        sp.total = L.total;
+        sp.head = (unsigned long long *)(dc + cl.head_sieve) + j;
+        sp.planes = mp.planes;
+        sp.raw = mp.raw;
+        sp.raw_count = d_rawcnt;
+        sp.flags = d_flags;
+        if ((e = launch_sieve(sp, L.mid, L.planes, L.share, h->num_sms, st)) != cudaSuccess)
+            return h->cuda_fail(e, "sieve kernel");
+    }
     if (P.pair_mode && P.total_pair_items > 0) {
         MainParams pp = mp;
         pp.item_claim = nullptr;   // the pair kernel claims pairs within its own CTA
@@ -1355,6 +1518,7 @@ static int autotune_class(pms_ctx *h, int n, int m, int l, int d, pms_ctx::Tunin
     h->opt.count_work = 0;
     h->opt.grab = 0;
     h->opt.partial_rows = 0;
+    h->tuning_tree = true;   // what is tuned is the tree form's schedule
     h->opt.graph = -1;   // every trial timed by its own events, never a graph replay
     std::vector<InstSpec> specs{InstSpec{n, m, l, d, seqs.data()}};
     auto run = [&](const pms_ctx::Tuning &t, double &ms) -> int {
@@ -1420,6 +1584,7 @@ static int autotune_class(pms_ctx *h, int n, int m, int l, int d, pms_ctx::Tunin
         }
     }
     h->opt = saved;
+    h->tuning_tree = false;
     if (rc) {
         h->tuned.erase(key);
         return rc;

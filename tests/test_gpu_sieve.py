@@ -1,0 +1,63 @@
+"""The sieve form against the oracle, bit-exact, at the edges of its blocks, words and windows,
+and against the tree form (which an explicit node filter selects) on larger instances."""
+import numpy as np
+import pytest
+
+import planted_inputs as pi
+import paper_2403_00306_gb300 as pms
+
+pytestmark = pytest.mark.gpu
+
+# l = 8..10: 3 middle letters (8 and 9: almost no prefix); 11: 4; 12, 13: 5, a CTA per block;
+# 14..16: 5, a warp per block (16: the longest prefix); W around 32 and one window per sequence;
+# more sequences than a CTA has warps; more changes than middle letters
+SMALL = [(2, 9, 9, 2), (2, 40, 8, 1), (3, 39, 8, 1), (9, 40, 9, 2), (17, 41, 9, 1), (5, 64, 10, 3), (64, 42, 10, 4),
+         (8, 43, 11, 3), (6, 11, 11, 5), (9, 75, 12, 4), (20, 96, 13, 4), (12, 45, 13, 6), (7, 46, 14, 5),
+         (10, 60, 15, 5), (5, 16, 16, 4), (12, 50, 16, 6)]
+# 5 counter planes up to 31 sequences and l >= 12, else 7
+QUORUM = [(5, 60, 9, 1, 3), (12, 64, 10, 2, 10), (31, 50, 12, 3, 28), (32, 50, 12, 3, 29), (64, 40, 11, 3, 60),
+          (8, 50, 13, 4, 7), (6, 40, 15, 4, 5), (10, 48, 16, 5, 9), (4, 30, 9, 2, 1)]
+
+
+@pytest.mark.parametrize("case", SMALL, ids=str)
+def test_sieve_matches_oracle(oracle_, case):
+    n, m, l, d = case
+    for seqs in (pi.planted_instance(n, m, l, d, 7).seqs, pi.random_sequences(n, m, 70)):
+        want = oracle_.solve_packed(seqs, l, d)
+        with pms.Context(0) as c:
+            assert np.array_equal(c.solve(seqs, l, d), want)
+            for got in c.solve_batch([(seqs, l, d)] * 3):   # a warp per block for every l
+                assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("case", QUORUM, ids=str)
+def test_sieve_quorum_matches_oracle(oracle_, case):
+    n, m, l, d, q = case
+    seqs = pi.planted_instance(n, m, l, d, 11).seqs
+    with pms.Context(0) as c:
+        c.set_options(quorum=q)
+        assert np.array_equal(c.solve(seqs, l, d), oracle_.solve_quorum(seqs, l, d, q, cap=1 << 24))
+
+
+@pytest.mark.parametrize("case", [(9, 2, 20, 600, 0), (11, 3, 17, 733, 0), (12, 3, 25, 1000, 0), (13, 4, 20, 600, 0),
+                                  (14, 4, 13, 999, 0), (15, 4, 20, 1100, 0), (15, 5, 20, 301, 0), (16, 5, 20, 250, 0),
+                                  (13, 4, 20, 300, 18), (15, 4, 15, 200, 12), (12, 3, 40, 400, 37)], ids=str)
+def test_sieve_and_tree_form_agree(case):
+    """Whole motif sets and, on the device entry point, raw counts (a motif once per seed window near it)."""
+    import torch
+    l, d, n, m, q = case
+    seqs = pi.planted_instance(n, m, l, d, 3).seqs
+    d_in = torch.from_numpy(seqs.copy()).cuda()
+    outs = []
+    for opts in ({}, {"grab": 1}):
+        with pms.Context(0) as c:
+            c.set_options(quorum=q, **opts)
+            out = torch.zeros(1 << 16, dtype=torch.int64, device="cuda")
+            st = torch.zeros(4, dtype=torch.int32, device="cuda")
+            torch.cuda.synchronize()
+            for _ in range(3):   # kernel by kernel, captured, replayed
+                c.solve_device(d_in, n, m, l, d, out, 1 << 16, st)
+            torch.cuda.synchronize()
+            outs.append((out.cpu().numpy(), st.cpu().numpy(), c.solve(seqs, l, d)))
+    assert np.array_equal(outs[0][1], outs[1][1]) and np.array_equal(outs[0][0], outs[1][0])
+    assert np.array_equal(outs[0][2], outs[1][2]) and len(outs[0][2]) > 0
