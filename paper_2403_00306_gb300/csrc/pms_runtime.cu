@@ -191,6 +191,7 @@ struct Served;
 // counter planes and warps per block, see launch_sieve) or the tree (mid = 0).
 struct SieveForm {
     int mid = 0, planes = 0, share = 1;
+    double us = 0;   // estimated time
 };
 
 struct pms_ctx {
@@ -761,6 +762,7 @@ static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int
     const double lookups = motifs * seeds * 14e-6 * (wide ? 1.0 : std::max(1.0, slots / blocks));
     const double latency = !single ? 0.0 : f.share == 8 ? 12.0 + 0.085 * W : f.share == 0 ? 14.0 + 0.04 * W : 35.0;
     const double sieve = (f.share == 8 ? std::max(latency, 25.0 + marks) : latency + marks) + lookups;
+    f.us = sieve;
     return sieve < tree ? f : SieveForm{};
 }
 
@@ -1635,6 +1637,7 @@ struct Request {
     size_t dense_rel = 0, status_rel = 0;   // offsets in the arena
     long long chunks_total = 0, chunks_next = 0;
     double units_per_chunk = 1.0;
+    SieveForm form;                // mid > 0: sieve form, run whole by one wave
     cudaEvent_t done_ev = nullptr;
     int status = PMS_OK;
     std::vector<uint64_t> codes;
@@ -1686,7 +1689,7 @@ struct PoolAlloc {
 // A request's arena in the pool (offsets relative to the arena start).
 struct ReqLayout {
     size_t seqs, planes, compat, rowlen, raw, tmp, dense, status, ctab, total;
-    ReqLayout(int n, int m, int W, uint32_t raw_cap, size_t ctab_ints)
+    ReqLayout(int n, int m, int W, uint32_t raw_cap, size_t ctab_ints, bool tree)
     {
         size_t o = 0;
         auto take = [&](size_t b) {
@@ -1696,8 +1699,8 @@ struct ReqLayout {
         };
         seqs = take((size_t)n * m);
         planes = take((size_t)n * W * sizeof(uint2));
-        compat = take((size_t)W * (n - 1) * ((W + 31) / 32) * sizeof(uint32_t));
-        rowlen = take((size_t)W * (n - 1) * sizeof(int));
+        compat = take(tree ? (size_t)W * (n - 1) * ((W + 31) / 32) * sizeof(uint32_t) : 0);
+        rowlen = take(tree ? (size_t)W * (n - 1) * sizeof(int) : 0);
         raw = take((size_t)raw_cap * 8);
         tmp = take((size_t)raw_cap * 8);   // directly after raw: the sort's twin buffer
         dense = take((size_t)raw_cap * 8);
@@ -1731,7 +1734,11 @@ struct Served {
     int *h_ctab = nullptr;           // pinned [slots][kCtabMax]
     static constexpr int kCtabMax = 8192;
     static constexpr int kRing = 4;
-    char *d_ring = nullptr;          // per wave: head + segments
+    // per wave: queue heads (the verification kernel's, then one per sieve
+    // launch: 3, 4 and 5 middle letters), the segments of the verification
+    // queue [slots], the sieve launches' segments [slots]
+    static constexpr size_t kRingSegs = 32;
+    char *d_ring = nullptr;
     char *h_ring = nullptr;          // pinned
     size_t ring_stride = 0;
     cudaEvent_t ring_ev[kRing] = {};
@@ -1779,7 +1786,7 @@ static int served_start(pms_ctx *h)
     S->pool = (char *)h->dev_alloc(pool);
     S->d_inst = (InstDev *)h->dev_alloc(S->slots * sizeof(InstDev));
     S->d_cnt = (uint32_t *)h->dev_alloc(cnt_words * 4);
-    S->ring_stride = round_up(8 + (size_t)S->slots * sizeof(Segment), 256);
+    S->ring_stride = round_up(Served::kRingSegs + (size_t)S->slots * (sizeof(Segment) + sizeof(SieveSeg)), 256);
     S->d_ring = (char *)h->dev_alloc(S->ring_stride * Served::kRing);
     bool ok = S->pool && S->d_inst && S->d_cnt && S->d_ring;
     if (ok)
@@ -1860,6 +1867,10 @@ static void served_stop(pms_ctx *h)
     h->served = nullptr;
 }
 
+// Candidate units of a wave's budget that a microsecond of the sieve stands for
+// (a wave of the default 6.4e9 units of tree work runs for about 10 ms).
+constexpr double kUnitsPerUs = 6.4e5;
+
 // Admission: a slot and an arena must be free. Uploads the request, packs
 // its windows and builds its compatibility masks (stream order).
 static bool served_admit(Served *S, Request *r)
@@ -1880,7 +1891,12 @@ static bool served_admit(Served *S, Request *r)
     }
     InstSpec spec{r->n, r->m, r->l, r->d, nullptr};
     r->raw_cap = default_cap(h, spec, true);
-    ReqLayout L(r->n, r->m, r->W, r->raw_cap, ct.tab.size());
+    // the stream's requests share the device, so the form is the one for a launch of many
+    r->form = sieve_form(h, r->n, r->m, r->l, r->d, false);
+    if (r->form.planes != 0)
+        r->form = SieveForm{};   // the served form solves q = n
+    const bool tree = r->form.mid == 0;
+    ReqLayout L(r->n, r->m, r->W, r->raw_cap, ct.tab.size(), tree);
     if (L.total > S->pool_bytes) {
         r->status = PMS_ENOMEM;   // can never fit
         return true;
@@ -1900,6 +1916,10 @@ static bool served_admit(Served *S, Request *r)
     for (int i = 0; i <= r->d; ++i)
         units += (double)binom(r->l, i) * (std::pow(3.0, i) + kNodeUnits);
     r->units_per_chunk = std::max(1.0, units / ct.cps);
+    if (!tree) {
+        r->chunks_total = 1;
+        r->units_per_chunk = r->form.us * kUnitsPerUs;
+    }
     InstDev &in = S->h_inst[r->slot];
     in = InstDev{};
     in.n = r->n;
@@ -1915,6 +1935,7 @@ static bool served_admit(Served *S, Request *r)
     in.triple_rows = h->triple_rows_for(r->n, r->m, r->l, r->d);
     in.q = r->n;
     in.nseed = 1;
+    in.sieve_mid = r->form.mid;
     in.seq_off = (long long)(off + L.seqs);
     in.plane_off = (long long)((off + L.planes) / sizeof(uint2));
     in.raw_off = (long long)((off + L.raw) / 8);
@@ -1935,7 +1956,7 @@ static bool served_admit(Served *S, Request *r)
     launch_pack(S->d_inst + r->slot, 1, srv_zero(S), windows, (const uint8_t *)S->pool, (uint2 *)S->pool,
                 srv_flags(S) + r->slot, (int)std::max<long long>(1, std::min<long long>((windows + 255) / 256, h->num_sms * 8)),
                 st);
-    const long long rows = (long long)r->W * (r->n - 1);
+    const long long rows = tree ? (long long)r->W * (r->n - 1) : 0;
     if (rows > 0)
         launch_compat(S->d_inst + r->slot, 1, srv_zero(S), rows, (const uint2 *)S->pool, (uint32_t *)S->pool,
                       (int *)S->pool,
@@ -2012,6 +2033,9 @@ static void served_loop(Served *S)
             S->wave_ev.erase(S->wave_ev.begin());
         }
         std::vector<Segment> segs;
+        std::vector<SieveSeg> sieve_segs[3];   // by middle letters - 3
+        long long sieve_blocks[3] = {0, 0, 0};
+        size_t reqs = 0;
         std::vector<Request *> finishing;
         if (S->wave_ev.size() < 2) {
             long long items = 0;
@@ -2020,8 +2044,18 @@ static void served_loop(Served *S)
             for (Request *r : S->active) {
                 if (r->state != 1 || r->chunks_next >= r->chunks_total)
                     continue;
-                if (units >= wave_units || (int)segs.size() >= S->slots)
+                if (units >= wave_units || (int)reqs >= S->slots)
                     break;
+                ++reqs;
+                if (r->form.mid > 0) {
+                    const int j = r->form.mid - 3;
+                    sieve_segs[j].push_back(SieveSeg{sieve_blocks[j], r->slot, 0});
+                    sieve_blocks[j] += 1ll << (2 * (r->l - r->form.mid - kSvSuf));
+                    r->chunks_next = r->chunks_total;
+                    units += r->units_per_chunk;
+                    finishing.push_back(r);
+                    continue;
+                }
                 long long take = (long long)std::ceil((wave_units - units) / r->units_per_chunk);
                 take = std::max<long long>(1, std::min(take, r->chunks_total - r->chunks_next));
                 segs.push_back(Segment{items, r->slot, (int)r->chunks_next, (int)(r->chunks_next + take), 0});
@@ -2032,7 +2066,7 @@ static void served_loop(Served *S)
                 if (r->chunks_next >= r->chunks_total)
                     finishing.push_back(r);
             }
-            if (!segs.empty()) {
+            if (reqs > 0) {
                 cudaError_t e = cudaSuccess;
                 if (need_rows > S->rows_cap) {
                     std::lock_guard<std::recursive_mutex> hg(h->mu);
@@ -2060,13 +2094,18 @@ static void served_loop(Served *S)
                 cudaEventSynchronize(S->ring_ev[rp]);
                 char *hr = S->h_ring + rp * S->ring_stride;
                 char *dr = S->d_ring + rp * S->ring_stride;
-                const unsigned long long zero = 0;
-                std::memcpy(hr, &zero, 8);
-                std::memcpy(hr + 8, segs.data(), segs.size() * sizeof(Segment));
-                e = cudaMemcpyAsync(dr, hr, 8 + segs.size() * sizeof(Segment), cudaMemcpyHostToDevice, S->st);
+                std::memset(hr, 0, Served::kRingSegs);
+                std::memcpy(hr + Served::kRingSegs, segs.data(), segs.size() * sizeof(Segment));
+                size_t sieve_off[3], ring_bytes = Served::kRingSegs + segs.size() * sizeof(Segment);
+                for (int j = 0; j < 3; ++j) {
+                    sieve_off[j] = ring_bytes;
+                    std::memcpy(hr + ring_bytes, sieve_segs[j].data(), sieve_segs[j].size() * sizeof(SieveSeg));
+                    ring_bytes += sieve_segs[j].size() * sizeof(SieveSeg);
+                }
+                e = cudaMemcpyAsync(dr, hr, ring_bytes, cudaMemcpyHostToDevice, S->st);
                 MainParams mp{};
                 mp.inst = S->d_inst;
-                mp.seg = (const Segment *)(dr + 8);
+                mp.seg = (const Segment *)(dr + Served::kRingSegs);
                 mp.nseg = (int)segs.size();
                 mp.total = items;
                 mp.head = (unsigned long long *)dr;
@@ -2081,8 +2120,25 @@ static void served_loop(Served *S)
                 mp.rows_cap = (int)S->rows_cap;
                 mp.smem_rows_cap = h->opt.smem_rows > 0 ? std::min(h->opt.smem_rows, kRowSmemCap) : kRowSmemCap;
                 mp.counters = nullptr;
-                if (e == cudaSuccess)
+                if (e == cudaSuccess && items > 0)
                     e = launch_main(mp, (int)std::min<long long>(S->blocks, items), false, S->st);
+                for (int j = 0; j < 3 && e == cudaSuccess; ++j) {
+                    if (sieve_segs[j].empty())
+                        continue;
+                    SieveParams sp{};
+                    sp.inst = S->d_inst;
+                    sp.seg = (const SieveSeg *)(dr + sieve_off[j]);
+                    sp.nseg = (int)sieve_segs[j].size();
+                    sp.total = sieve_blocks[j];
+                    sp.head = (unsigned long long *)dr + 1 + j;
+                    sp.planes = mp.planes;
+                    sp.raw = mp.raw;
+                    sp.raw_count = mp.raw_count;
+                    sp.flags = mp.flags;
+                    // a launch with few blocks gives each a CTA
+                    const bool few = sp.total < 16ll * h->num_sms;
+                    e = launch_sieve(sp, j + 3, 0, !few ? 1 : j == 2 ? 8 : 0, h->num_sms, S->st);
+                }
                 cudaEventRecord(S->ring_ev[rp], S->st);
                 for (Request *r : finishing) {
                     char *base = S->pool + r->arena_off;
@@ -2108,8 +2164,8 @@ static void served_loop(Served *S)
                 cudaEventRecord(wev, S->st);
                 S->wave_ev.push_back(wev);
                 S->waves += 1;
-                S->max_reqs_per_wave = std::max<long long>(S->max_reqs_per_wave, (long long)segs.size());
-                if (segs.size() > 1)
+                S->max_reqs_per_wave = std::max<long long>(S->max_reqs_per_wave, (long long)reqs);
+                if (reqs > 1)
                     S->overlapped_waves += 1;
                 if (e != cudaSuccess) {
                     cudaGetLastError();
