@@ -68,7 +68,7 @@ typedef struct {
 /* Tunables. Zero in any field selects the default (or the tuned value).
  * A solve takes one of two forms of the search with the same answer: the tree
  * over B(x, d) of every seed, or the sieve (every window marks the strings
- * within d of it in a bit map of all 4^l; l <= 16), whichever is estimated to
+ * within d of it in a bit map of all 4^l), whichever is estimated to
  * be faster for its n, m, l, d and quorum. Setting chunk_work, grab,
  * count_work, smem_rows, seed_mode, partial_rows or triple_rows selects the
  * tree form, which these fields describe. */

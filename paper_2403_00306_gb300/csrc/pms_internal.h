@@ -51,8 +51,8 @@ struct InstDev {
     uint32_t raw_cap;      // capacity of the raw motif buffer (power of two)
     int triple_rows;       // rows after the first whose occurrences are tested in pairs with the first
                            //   row's (three-string feasibility below a node); 0: no such test
-    int sieve_mid;         // sieve form: middle letters of a block (pms_sieve.cu); its window words (uint32)
-                           //   are then stored in place of the planes. 0: the tree form
+    int sieve_mid;         // sieve form: middle letters of a block (pms_sieve.cu); its window words are
+                           //   then stored in place of the planes. 0: the tree form
 };
 
 // A contiguous range of queue items: chunks [chunk_lo, chunk_hi) of instance
@@ -197,10 +197,10 @@ struct SieveParams {
 };
 
 cudaError_t sieve_init_tables();
-// mid: middle letters of a block (3, 4, 5). planes: bits of the hit counters
-// of the quorum form (5 with mid 4, 7 with mid 3), 0 for q = n. share (q = n):
+// mid: middle letters of a block (3 to 6). planes: bits of the hit counters of
+// the quorum form (5 with mid 4 or 5, 7 with mid 3), 0 for q = n. share (q = n):
 // 1 a warp per block; 8 a CTA per block, its warps split every sequence's
-// windows (mid 5); 0 a CTA per block, its warps split the sequences (mid 3, 4).
+// windows (mid 5, 6); 0 a CTA per block, its warps split the sequences (mid 3, 4).
 cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, int sms, cudaStream_t st);
 
 // ---------------------------------------------------------------- general alphabets (pms_sigma.cu)

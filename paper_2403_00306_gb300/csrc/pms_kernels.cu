@@ -2415,13 +2415,11 @@ __global__ void pack_kernel(const InstDev *__restrict__ inst, int ninst, const l
             h |= (code >> 1) << k;
             lo_bits |= (code & 1u) << k;
         }
-        if (in.sieve_mid == 0)
-            planes[in.plane_off + local] = make_uint2(h, lo_bits);
-        else
-            reinterpret_cast<uint32_t *>(planes + in.plane_off)[local] =
-                in.sieve_mid == 5   ? sieve_word<5>(h, lo_bits, in.l)
-                : in.sieve_mid == 4 ? sieve_word<4>(h, lo_bits, in.l)
-                                    : sieve_word<3>(h, lo_bits, in.l);
+        planes[in.plane_off + local] = in.sieve_mid == 0   ? make_uint2(h, lo_bits)
+                                       : in.sieve_mid == 6 ? sieve_word<6>(h, lo_bits, in.l)
+                                       : in.sieve_mid == 5 ? sieve_word<5>(h, lo_bits, in.l)
+                                       : in.sieve_mid == 4 ? sieve_word<4>(h, lo_bits, in.l)
+                                                           : sieve_word<3>(h, lo_bits, in.l);
         if (bad)
             atomicOr(&flags[lo], kFlagInvalidByte);
     }

@@ -602,7 +602,7 @@ struct MetaLayout {
 // Counters block (d_ctr): queue heads, work counters, dense_total, then per instance
 // raw_count and flags, then (items > 0) the steal cursor and the nodes claimed
 // of every queue item, for the verification kernel's work sharing.
-constexpr int kMaxSieveLaunches = 5;   // q = n with 3, 4 or 5 middle letters, the quorum form with 3 or 4
+constexpr int kMaxSieveLaunches = 7;   // q = n with 3 to 6 middle letters, the quorum form with 3 to 5
 struct CtrLayout {
     size_t head, head_pair, head_sieve, work, dense_total, raw_count, flags, steal, claim, total;
     CtrLayout(size_t k, size_t items = 0)
@@ -707,63 +707,86 @@ static double expected_seed_rows(int n, int m, int l, int d)
     return (n - 1) * ((m - l + 1) * p + 3.0);
 }
 
-// The form with the smaller estimated time. Both estimates were fitted to
-// device times on one GB300 (n = 10 and 20, m = 200, 600, 1200, l = 8..16,
-// d = 1..5); they only choose, so what matters is where they cross.
-//   tree: W |B(x, d)| candidates at 250 E^2 ps each, E = expected_near: the more
-//     windows lie near a candidate, the fewer nodes fail. A quorum adds seeds
-//     and keeps nodes with misses. 38 us + 25 ns W for the launches, the masks
-//     and the slowest seeds of a single instance.
-//     Measured and (estimated), us: (15,4) m = 600 118 (136), m = 1000 562 (455);
-//     (14,4) 761 (700); (16,5) 5576 (5200); (13,4) 1704 (3300); (13,3) 54 (60).
-//   sieve: 4^A blocks, W windows and S sequences at 3.2 ps and 0.3 ps per word
-//     a window marks; S = n, or less when a block's strings run out sooner.
-//     A single instance with few blocks is bound by one block's latency.
-//     Measured and (estimated), us: (15,4) m = 600 192 (197), m = 1000 337 (375);
-//     (14,4) 135 (128); (16,5) 1156 (1160); (13,4) 174 (135); (13,3) 67 (63).
+// The form with the smallest estimated time. The estimates were fitted to
+// device times on one GB300 (n = 10 and 20, m = 200, 600, 1200, l = 8..19,
+// d = 1..6); they only choose, so what matters is where they cross.
+//   tree: W |B(x, d)| candidates at 390 E^3 / (E + 0.02) ps each, E =
+//     expected_near: the more windows lie near a candidate, the fewer nodes
+//     fail. A quorum adds seeds and keeps nodes with misses. A single instance
+//     takes 38 us + 25 ns W for the launches, the masks and the slowest seeds.
+//     Measured (estimated), us: (15,4) m = 600 118 (154), m = 1000 562 (515),
+//     m = 1200 1050 (1003); (14,4) m = 600 761 (800); (13,3) m = 1200 141 (151);
+//     (17,5) m = 600 1050 (1030), m = 900 4300 (4060), m = 1200 11080 (9500).
+//   sieve: 4^A blocks, W windows and S sequences at a + b words ps, words = the
+//     words of a block that a window marks on average; S = n, or less where a
+//     block's strings run out sooner. With few blocks, one block's latency counts.
+//     Measured (estimated), us, by middle letters:
+//     5: (15,4) m = 600 199 (184), m = 1000 337 (349); (13,4) m = 600 174 (151);
+//        (17,5) m = 1200 5429 (5470); (16,5) m = 600 1183 (1130)
+//     6: (17,5) m = 1200 4326 (4990); (15,4) m = 1200 392 (377); (16,4) 655 (690);
+//        (19,6) m = 1200 58900 (58000, the tree 110800)
 // `single`: the only instance of its launch.
 static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int q, bool single)
 {
-    SieveForm f;
-    f.planes = q == n ? 0 : (n <= 31 && l >= 12 ? 5 : 7);
-    f.mid = q < n ? (f.planes == 5 ? 4 : 3) : (l <= 10 ? 3 : l == 11 || (!single && l == 12) ? 4 : 5);
-    const int A = l - f.mid - kSvSuf;
-    if (n < 2 || A < 0 || A > (f.mid == 5 ? sv_pre<5>() : f.mid == 4 ? sv_pre<4>() : sv_pre<3>()))
-        return SieveForm{};
     const double W = m - l + 1, E = expected_near(m, l, d), p = 1.0 - std::exp(-E);
     const double seeds = W * (n - q + 1);
     // short motifs that most sequences hold: the answer is a good part of all
     // 4^l strings, and writing it is what takes the time
-    if (l == 8 && E > 1.0)
+    if (n < 2 || (l == 8 && E > 1.0))
         return SieveForm{};
-    const double tree = seeds * (double)ball_size(l, d) * 250e-6 * E * E * (1.0 + 3.0 * (n - q)) +
-                        (single ? 38.0 + 0.025 * W : 0.0);
-    const double strings = std::pow(4.0, f.mid + kSvSuf), blocks = std::pow(4.0, A);
-    // sequences until a block holds fewer than two (quorum: no) strings that may still be motifs
-    int S = 1;
-    for (; S < n; ++S) {
-        double tail = 0;   // a string has S - (n - q) hits of S
-        for (int k = std::max(0, S - (n - q)); k <= S; ++k)
-            tail += choose(S, k) * std::pow(p, k) * std::pow(1.0 - p, S - k);
-        if (strings * tail < (q == n ? 2.0 : 0.5))
-            break;
-    }
-    const double words = (double)ball_size(l - kSvSuf, d) / (blocks * std::pow(4.0, f.mid));
-    const bool wide = q == n && single && l <= 13;   // few blocks: a CTA each
-    f.share = !wide ? 1 : (f.mid == 5 ? 8 : 0);
-    const double slots = 16.0 * h->num_sms;
-    const double rounded = single && !wide ? std::ceil(blocks / slots) * slots : blocks;
-    const double marks = rounded * W * S * (3.2 + 0.3 * words) * 1e-6;
+    double best = seeds * (double)ball_size(l, d) * 390e-6 * E * E * E / (E + 0.02) * (1.0 + 3.0 * (n - q)) +
+                  (single ? 38.0 + 0.025 * W : 0.0);
     double motifs = 0;
     for (int k = q; k <= n; ++k)
         motifs += choose(n, k) * std::pow(p, k) * std::pow(1.0 - p, n - k);
     motifs *= std::pow(4.0, l);
-    // every motif is looked up in the seed sequences, by as many warps as have blocks
-    const double lookups = motifs * seeds * 14e-6 * (wide ? 1.0 : std::max(1.0, slots / blocks));
-    const double latency = !single ? 0.0 : f.share == 8 ? 12.0 + 0.085 * W : f.share == 0 ? 14.0 + 0.04 * W : 35.0;
-    const double sieve = (f.share == 8 ? std::max(latency, 25.0 + marks) : latency + marks) + lookups;
-    f.us = sieve;
-    return sieve < tree ? f : SieveForm{};
+    struct Option {
+        int mid, planes, share;
+        bool use;
+        double a, b;   // ps per block, window and sequence, and per word marked
+    };
+    const bool all = q == n;
+    const Option options[] = {
+        {3, 0, single ? 0 : 1, all && l <= 10, 2.8, 0.33},
+        {4, 0, single ? 0 : 1, all && (l == 11 || (!single && l == 12)), 2.8, 0.33},
+        {5, 0, single && l <= 13 ? 8 : 1, all && l >= (single ? 12 : 13), 2.8, 0.33},
+        {6, 0, 8, all && l >= 14, 6.0, 0.45},
+        {5, 5, 8, !all && l >= 13 && n <= 31, 5.2, 0.45},
+        {4, 5, 1, !all && l >= 12 && n <= 31, 2.8, 0.33},
+        {3, 7, 1, !all && (l < 12 || n > 31), 2.8, 0.33},
+    };
+    const double slots = 16.0 * h->num_sms;   // warps, of a form with a warp per block
+    SieveForm form;
+    for (const Option &o : options) {
+        const int A = l - o.mid - kSvSuf;
+        if (!o.use || A < 0 || A > kSvPre)
+            continue;
+        const double strings = std::pow(4.0, o.mid + kSvSuf), blocks = std::pow(4.0, A);
+        // sequences until a block holds fewer than two (quorum: no) strings that may still be motifs
+        int S = 1;
+        for (; S < n; ++S) {
+            double tail = 0;   // a string has S - (n - q) hits of S
+            for (int k = std::max(0, S - (n - q)); k <= S; ++k)
+                tail += choose(S, k) * std::pow(p, k) * std::pow(1.0 - p, S - k);
+            if (strings * tail < (all ? 2.0 : 0.5))
+                break;
+        }
+        const double words = (double)ball_size(l - kSvSuf, d) / std::pow(4.0, l - kSvSuf) * std::pow(4.0, o.mid);
+        // the last round of blocks, and a CTA's last round of 32 windows a warp
+        const bool wide = all && single && l <= 13;   // few blocks: a CTA each
+        const double rounds = single && !wide && o.share == 1 ? std::ceil(blocks / slots) * slots : blocks;
+        const double windows = o.share == 8 && !wide ? std::ceil(W / 256.0) * 256.0 : W;
+        const double marks = rounds * windows * S * (o.a + o.b * words) * 1e-6;
+        // every motif is looked up in the seed sequences, by as many warps as have blocks
+        const double lookups = motifs * seeds * 14e-6 * (o.share != 1 ? 1.0 : std::max(1.0, slots / blocks));
+        const double latency = !single ? 0.0 : !wide ? 35.0 : o.share == 8 ? 12.0 + 0.085 * W : 14.0 + 0.04 * W;
+        const double us = (wide && o.share == 8 ? std::max(latency, 25.0 + marks) : latency + marks) + lookups;
+        if (us < best) {
+            best = us;
+            form = SieveForm{o.mid, o.planes, o.share, us};
+        }
+    }
+    return form;
 }
 
 // The form of one instance under the context's options: those that shape the
@@ -788,7 +811,7 @@ static SieveForm sieve_form(const pms_ctx *h, int n, int m, int l, int d, bool s
 // Adds the sieve launches of the instances in sieve form.
 static void plan_sieve(Plan &P, const std::vector<SieveForm> &form)
 {
-    static const int forms[kMaxSieveLaunches][2] = {{5, 0}, {4, 0}, {3, 0}, {4, 5}, {3, 7}};
+    static const int forms[kMaxSieveLaunches][2] = {{6, 0}, {5, 0}, {4, 0}, {3, 0}, {5, 5}, {4, 5}, {3, 7}};
     for (const auto &f : forms) {
         std::vector<int> list;
         for (size_t k = 0; k < P.inst.size(); ++k)
@@ -1735,9 +1758,9 @@ struct Served {
     static constexpr int kCtabMax = 8192;
     static constexpr int kRing = 4;
     // per wave: queue heads (the verification kernel's, then one per sieve
-    // launch: 3, 4 and 5 middle letters), the segments of the verification
+    // launch: 3 to 6 middle letters), the segments of the verification
     // queue [slots], the sieve launches' segments [slots]
-    static constexpr size_t kRingSegs = 32;
+    static constexpr size_t kRingSegs = 48;
     char *d_ring = nullptr;
     char *h_ring = nullptr;          // pinned
     size_t ring_stride = 0;
@@ -2033,8 +2056,8 @@ static void served_loop(Served *S)
             S->wave_ev.erase(S->wave_ev.begin());
         }
         std::vector<Segment> segs;
-        std::vector<SieveSeg> sieve_segs[3];   // by middle letters - 3
-        long long sieve_blocks[3] = {0, 0, 0};
+        std::vector<SieveSeg> sieve_segs[4];   // by middle letters - 3
+        long long sieve_blocks[4] = {0, 0, 0, 0};
         size_t reqs = 0;
         std::vector<Request *> finishing;
         if (S->wave_ev.size() < 2) {
@@ -2096,8 +2119,8 @@ static void served_loop(Served *S)
                 char *dr = S->d_ring + rp * S->ring_stride;
                 std::memset(hr, 0, Served::kRingSegs);
                 std::memcpy(hr + Served::kRingSegs, segs.data(), segs.size() * sizeof(Segment));
-                size_t sieve_off[3], ring_bytes = Served::kRingSegs + segs.size() * sizeof(Segment);
-                for (int j = 0; j < 3; ++j) {
+                size_t sieve_off[4], ring_bytes = Served::kRingSegs + segs.size() * sizeof(Segment);
+                for (int j = 0; j < 4; ++j) {
                     sieve_off[j] = ring_bytes;
                     std::memcpy(hr + ring_bytes, sieve_segs[j].data(), sieve_segs[j].size() * sizeof(SieveSeg));
                     ring_bytes += sieve_segs[j].size() * sizeof(SieveSeg);
@@ -2122,7 +2145,7 @@ static void served_loop(Served *S)
                 mp.counters = nullptr;
                 if (e == cudaSuccess && items > 0)
                     e = launch_main(mp, (int)std::min<long long>(S->blocks, items), false, S->st);
-                for (int j = 0; j < 3 && e == cudaSuccess; ++j) {
+                for (int j = 0; j < 4 && e == cudaSuccess; ++j) {
                     if (sieve_segs[j].empty())
                         continue;
                     SieveParams sp{};
@@ -2137,7 +2160,7 @@ static void served_loop(Served *S)
                     sp.flags = mp.flags;
                     // a launch with few blocks gives each a CTA
                     const bool few = sp.total < 16ll * h->num_sms;
-                    e = launch_sieve(sp, j + 3, 0, !few ? 1 : j == 2 ? 8 : 0, h->num_sms, S->st);
+                    e = launch_sieve(sp, j + 3, 0, !few ? 1 : j >= 2 ? 8 : 0, h->num_sms, S->st);
                 }
                 cudaEventRecord(S->ring_ev[rp], S->st);
                 for (Request *r : finishing) {

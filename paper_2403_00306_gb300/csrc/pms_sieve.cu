@@ -8,7 +8,7 @@
 // 3-5 with q = n), or that at least q sequences mark (the quorum form). Its
 // cost depends on n, W and |B(l, d)| only, not on how many strings survive.
 //
-// The map is cut into blocks that live in shared memory and registers. A
+// The map is cut into blocks (of 2^12 to 2^18 strings) that live in shared memory and registers. A
 // string is split into a prefix of A letters, kMid middle letters and three
 // last letters. A block is one prefix; its words are the 4^kMid middles; the
 // 64 bits of a word are the last three letters. A window at prefix distance t
@@ -32,12 +32,18 @@
 // with a window's index keeps banks distinct). Windows with one change left
 // touch 16 words: they are listed, and 32 of them worked on at once, a lane each.
 //
-// What bounds it: instruction issue and the marks. One GB300, n = 20:
-// (13,4) m = 1000 (20 sequences x 988 windows x 1024 blocks, 20.7 words marked
-// per window and block) 316 us, 190 M warp instructions, 16.8 M mark operations,
-// 2.3 instructions a cycle; 64 registers and 25 warps per SM. The same search in
-// the tree form takes 7409 us. Load-or-stores in place of the atomics, a warp
-// per block: 587 us, 325 M instructions.
+// What bounds it. Where windows mark many words of a block: instruction issue
+// and the marks; (13,4), n = 20, m = 1000 (20 sequences x 988 windows x 1024
+// blocks, 20.7 words marked per window and block) 316 us, 190 M warp
+// instructions, 17 M mark operations, 2.3 instructions a cycle. The tree form
+// takes 7409 us there; load-or-stores in place of the atomics, a warp per
+// block, took 587 us and 325 M instructions. Where they mark few: the 50 or so
+// instructions that sort 32 windows by the changes they have left; larger
+// blocks pay them less often. (17,5), n = 20, m = 1200: 5 middle letters and a
+// warp per block 5429 us, 6 letters and a CTA per block 4326 us (the tree
+// 11089 us); (15,4) 449 and 392 us (1046 us). With six letters 32 KB of marks
+// serve a CTA of eight warps, and what is lost is their wait for the slowest
+// (5.8 of 14 cycles per instruction), so few windows favour the warp per block.
 #include "pms_sieve.cuh"
 
 #include <algorithm>
@@ -50,7 +56,7 @@ namespace {
 constexpr uint32_t kFull = 0xffffffffu;
 constexpr int kSvWarps = 8;
 constexpr int kSvThreads = kSvWarps * 32;
-constexpr int kSvMaxShell = 5;             // changed middle letters, at most kMid
+constexpr int kSvMaxShell = 6;             // changed middle letters, at most kMid
 // Lanes that still hold strings, at or below which a block looks its strings up
 // in the remaining sequences instead of marking them.
 constexpr int kSvLookupLanes = 2;
@@ -67,13 +73,18 @@ __host__ __device__ constexpr uint32_t sv_single(int e)
 
 // Changes of t >= 2 middle letters, in groups of 32 with different banks where
 // that is possible; the last group repeats changes in its unused places.
-constexpr int kSvGroupsMax = 40;
+constexpr int kSvGroupsMax = 132;
+template <int kMid>
+__host__ __device__ constexpr int sv_groups()
+{
+    return kMid == 6 ? 129 : kMid == 5 ? 33 : kMid == 4 ? 10 : 2;
+}
 struct SvTable {
     uint16_t change[kSvGroupsMax * 32];    // byte offsets of word indexes
     int first[kSvMaxShell + 2];            // first group of the shell of t changes; [t + 1] is its end
 };
 
-__device__ SvTable g_sv_table[3];          // kMid = 3, 4, 5
+__device__ SvTable g_sv_table[4];          // kMid = 3, 4, 5, 6
 // bits of the ball of radius v around last letters s, one half of the 64: [v][s][half]
 __device__ uint32_t g_sv_ball[4][64][2];
 
@@ -81,17 +92,19 @@ __device__ uint32_t g_sv_ball[4][64][2];
 template <int kMid>
 __host__ __device__ constexpr int sv_groups2()
 {
-    return kMid == 5 ? 3 : kMid == 4 ? 2 : 1;
+    return kMid == 6 ? 5 : kMid == 5 ? 3 : kMid == 4 ? 2 : 1;
 }
 
-// Shared memory of a CTA besides its teams' marks.
+// Shared memory of a CTA besides its marks, which it precedes: the marks are
+// aligned to one half of a buffer.
+template <int kMid>
 struct SvSmem {
     uint32_t ball[4 * 64 * 2];             // g_sv_ball
-    uint16_t change[kSvGroupsMax * 32];
+    uint16_t change[sv_groups<kMid>() * 32];
     uint32_t list[kSvWarps][64];           // windows with one change left, until 32 are there
     int first[kSvMaxShell + 2];
-    long long item[kSvWarps];              // per team
-    int alive[kSvWarps][3];                // per team: lanes that hold strings alive after sequence i, at i % 3
+    long long item;                        // of the CTA, when its warps share a block
+    int alive[3];                          // lanes that hold strings alive after sequence i, at i % 3
 };
 
 template <int kMid>
@@ -101,101 +114,126 @@ struct SvMarks {
     static constexpr uint32_t kBytes = 2 * kHalf;
 };
 
+// Marks: an atomic OR on shared memory without a result. No memory clobber: the
+// barriers around a sequence's marks order them against the plain accesses.
 __device__ __forceinline__ void red_or(uint32_t addr, uint32_t v)
 {
-    asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+    asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(addr), "r"(v));
+}
+__device__ __forceinline__ void red_or_if(bool on, uint32_t addr, uint32_t v)
+{
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p red.shared.or.b32 [%1], %2; }" ::"r"((uint32_t)on), "r"(addr),
+                 "r"(v));
 }
 
 // The distance of two strings as sieve words (see sieve_word), prefix included.
 template <int kMid>
-__device__ __forceinline__ int sv_distance(uint32_t a, uint32_t b)
+__device__ __forceinline__ int sv_distance(uint2 a, uint2 b)
 {
-    constexpr uint32_t kMask = (1u << kMid) - 1u;
-    const uint32_t x = a ^ b;
-    const uint32_t hi = (x >> (6 + kMid)) & kMask;
-    const uint32_t lo = ((x >> 6) & kMask) ^ sv_fold<kMid>(hi);
-    const uint32_t mid = hi | lo, suf = (x | (x >> 3)) & 7u;
-    const uint32_t pre = kMid == 5   ? ((x >> 24) | (x >> 16)) & 0xffu
-                         : kMid == 4 ? ((x >> 23) | (x >> 14)) & 0x1ffu
-                                     : ((x >> 22) | (x >> 12)) & 0x3ffu;
-    return __popc((pre << 16) | (mid << 8) | suf);
+    const uint32_t x = a.x ^ b.x, y = a.y ^ b.y;
+    const uint32_t mid = (x >> (6 + kMid)) | sv_lo<kMid>(x >> 6), suf = (x | (x >> 3)) & 7u;
+    return __popc(((y | (y >> 16)) & 0xffffu) | (mid << 16) | (suf << 22));
 }
 
-// The windows of one sequence mark the block's words; the team's warps take
-// 32 windows in turn. marks: shared address, aligned to kBytes, so that a word
-// address is an exclusive-or away from another.
+// What a lane changes in the words of a window, as offsets from the window's
+// own word: at most one letter (with up to 16 such changes, half a warp for
+// each half of the words) and two letters. The lanes left over repeat a change.
+template <int kMid>
+struct SvLane {
+    static constexpr bool kBoth = 1 + 3 * kMid <= 16;
+    uint32_t single;                    // and, with kBoth, the half
+    uint32_t pair[sv_groups2<kMid>()];
+    int t;                              // letters `single` changes
+    int half;                           // the half of the words `single` works on first
+    __device__ __forceinline__ SvLane(const SvSmem<kMid> &sm, int lane)
+    {
+        const int e0 = kBoth ? (lane & 15) : lane < 1 + 3 * kMid ? lane : lane - 16;
+        half = kBoth ? lane >> 4 : 0;
+        single = 0;
+#pragma unroll
+        for (int e = 1; e <= 3 * kMid; ++e)
+            single = e0 == e ? sv_single<kMid>(e) << 2 : single;
+        t = e0 >= 1 && e0 <= 3 * kMid ? 1 : 0;
+        single += (uint32_t)half * SvMarks<kMid>::kHalf;
+#pragma unroll
+        for (int k = 0; k < sv_groups2<kMid>(); ++k)
+            pair[k] = sm.change[(sm.first[2] + k) * 32 + lane];
+    }
+};
+
+// The windows of one sequence mark the block's words; kShare warps take 32
+// windows in turn. marks: shared address, aligned to kHalf, so that within a
+// half a word address is an exclusive-or away from another. prefix: the
+// block's, as in a window's word.
 template <int kMid, int kShare>
-__device__ __forceinline__ void sv_mark(const uint32_t *__restrict__ win, int W, int d, uint32_t block, uint32_t marks,
-                                        uint32_t *list, const SvSmem &sm, uint32_t slot0,
-                                        const uint32_t (&d2)[sv_groups2<kMid>()], int g, int lane)
+__device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, int d, uint32_t prefix, uint32_t marks,
+                                        uint32_t *list, const SvSmem<kMid> &sm, const SvLane<kMid> &my, int g, int lane)
 {
     using M = SvMarks<kMid>;
-    constexpr int kPre = sv_pre<kMid>();
-    constexpr uint32_t kCode = (1u << (6 + 2 * kMid)) - 1u;
-    constexpr uint32_t kPreMask = ((1u << kPre) - 1u) << (6 + 2 * kMid);
-    constexpr uint32_t kWordMask = (4u << (2 * kMid)) - 4u;
     constexpr int kStep = 32 * kShare;
-    const bool edge = (lane & 15) < 1 + 3 * kMid;
-    const uint32_t *ball2 = sm.ball + (2 - ((lane & 15) != 0)) * 128 + (lane >> 4);
+    constexpr bool kBoth = SvLane<kMid>::kBoth;
     const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t single0 = marks + my.single;
+    const uint32_t *ball2 = sm.ball + (2 - my.t) * 128 + my.half;   // radius 2 or 1 of the last letters
     int n1 = 0;
     int w0 = 32 * g;
-    uint32_t next = w0 + lane < W ? __ldg(win + w0 + lane) : 0u;
+    uint2 next = w0 + lane < W ? __ldg(win + w0 + lane) : make_uint2(0u, 0u);
     for (; w0 < W; w0 += kStep) {
-        const uint32_t x = next ^ block;
+        const uint32_t y = next.y ^ prefix, code = next.x;
         const bool in = w0 + lane < W;
         if (w0 + kStep + lane < W)
             next = __ldg(win + w0 + kStep + lane);
-        const int r = in ? d - __popc((x | (x >> kPre)) & kPreMask) : -1;
-        const uint32_t code = x & kCode;
-        // the window's own word: byte address in the half that holds its last three letters
-        const uint32_t own = marks ^ ((code >> 6) << 2) ^ ((code & 32u) ? M::kHalf : 0u);
-        if (r == 0)
-            red_or(own, 1u << (code & 31u));
+        const int r = in ? d - __popc((y | (y >> 16)) & 0xffffu) : -1;
+        // word offset in a half's marks; the last three letters choose half and bit
+        const uint32_t off = (code >> 6) << 2;
+        red_or_if(r == 0, (marks + (code & 32u) * (M::kHalf / 32u)) ^ off, 1u << (code & 31u));
         const uint32_t one = __ballot_sync(kFull, r == 1);
         if (r == 1)
             list[n1 + __popc(one & lt)] = code;
         n1 += __popc(one);
-        uint32_t wide = __ballot_sync(kFull, r >= 2);
-        const uint32_t packed = ((code >> 4) & kWordMask) | ((code & 63u) << 16) | ((uint32_t)r << 24);
-        while (wide) {
-            const int src = __ffs(wide) - 1;
-            wide &= wide - 1u;
-            const uint32_t v = __shfl_sync(kFull, packed, src);
-            const uint32_t wa = marks ^ (v & kWordMask);   // the word in the lower half's marks
-            const uint32_t suf = (v >> 16) & 63u;
-            const uint32_t wh = wa ^ ((v & (32u << 16)) ? M::kHalf : 0u);
-            const uint32_t bit = 1u << (suf & 31u);
-            if ((v >> 24) == 2u) {
-                // no change and one change: half a warp per half of the words
-                // (slot0: the lane's change and half; ball2: its table column)
-                if (edge)
-                    red_or(wa ^ slot0, ball2[2 * suf]);
+        uint32_t two = __ballot_sync(kFull, r == 2);
+        const uint32_t packed = off | (code << 16);   // bits 16..21: the last letters; above them what is not used
+        while (two) {
+            const uint32_t v = __shfl_sync(kFull, packed, __ffs(two) - 1);
+            two &= two - 1u;
+            const uint32_t o = v & 0xffffu, suf = (v >> 16) & 63u;
+            red_or(single0 ^ o, ball2[2 * suf]);
+            if (!kBoth)
+                red_or((single0 + M::kHalf) ^ o, ball2[2 * suf + 1]);
+            const uint32_t wh = (marks + (suf >> 5) * M::kHalf) ^ o, bit = 1u << (suf & 31u);
 #pragma unroll
-                for (int t = 0; t < sv_groups2<kMid>(); ++t)
-                    red_or(wh ^ d2[t], bit);
-            } else {
-                const int rr = (int)(v >> 24);
-                const uint32_t *ball = sm.ball + 2 * suf;
-                if (edge)
-                    red_or(wa ^ slot0, ball[min(rr - ((lane & 15) != 0), 3) * 128 + (lane >> 4)]);
-                const int tmax = min(rr, kMid);
-                const uint16_t *ch = sm.change + lane;
-                for (int t = 2; t <= tmax; ++t) {
-                    const int q1 = sm.first[t + 1];
-                    if (t == rr) {
-#pragma unroll 3
-                        for (int q = sm.first[t]; q < q1; ++q)
-                            red_or(wh ^ ch[q * 32], bit);
-                    } else {
-                        const int rad = min(rr - t, 3);
-                        const uint32_t b0 = ball[rad * 128], b1 = ball[rad * 128 + 1];
-#pragma unroll 3
-                        for (int q = sm.first[t]; q < q1; ++q) {
-                            const uint32_t wc = wa ^ ch[q * 32];
-                            red_or(wc, b0);
-                            red_or(wc ^ M::kHalf, b1);
-                        }
+            for (int t = 0; t < sv_groups2<kMid>(); ++t)
+                red_or(wh ^ my.pair[t], bit);
+        }
+        uint32_t more = __ballot_sync(kFull, r > 2);
+        while (more) {
+            const int src = __ffs(more) - 1;
+            more &= more - 1u;
+            const uint32_t v = __shfl_sync(kFull, packed, src);
+            const int rr = __shfl_sync(kFull, r, src);
+            const uint32_t o = v & 0xffffu, suf = (v >> 16) & 63u;
+            const uint32_t *ball = sm.ball + 2 * suf;
+            red_or(single0 ^ o, ball[min(rr - my.t, 3) * 128 + my.half]);
+            if (!kBoth)
+                red_or((single0 + M::kHalf) ^ o, ball[min(rr - my.t, 3) * 128 + 1]);
+            const int tmax = min(rr, kMid);
+            const uint16_t *ch = sm.change + lane;
+            for (int t = 2; t <= tmax; ++t) {
+                const int q1 = sm.first[t + 1];
+                if (t == rr) {
+                    const uint32_t wh = (marks + (suf >> 5) * M::kHalf) ^ o, bit = 1u << (suf & 31u);
+#pragma unroll 4
+                    for (int q = sm.first[t]; q < q1; ++q)
+                        red_or(wh ^ ch[q * 32], bit);
+                } else {
+                    const uint32_t wa = marks ^ o;
+                    const int rad = min(rr - t, 3);
+                    const uint32_t b0 = ball[rad * 128], b1 = ball[rad * 128 + 1];
+#pragma unroll 4
+                    for (int q = sm.first[t]; q < q1; ++q) {
+                        const uint32_t wc = wa ^ ch[q * 32];
+                        red_or(wc, b0);
+                        red_or(wc + M::kHalf, b1);
                     }
                 }
             }
@@ -206,12 +244,10 @@ __device__ __forceinline__ void sv_mark(const uint32_t *__restrict__ win, int W,
             __syncwarp();
             const uint32_t v = list[lane], up = list[32 + lane];
             if (lane < n1) {
-                const uint32_t suf = v & 63u;
-                const uint32_t wa = marks ^ ((v & ~63u) >> 4);
-                red_or(wa, sm.ball[128 + 2 * suf]);
-                red_or(wa ^ M::kHalf, sm.ball[128 + 2 * suf + 1]);
-                const uint32_t wh = wa ^ ((suf & 32u) ? M::kHalf : 0u);
-                const uint32_t bit = 1u << (suf & 31u);
+                const uint32_t suf = v & 63u, o = (v >> 6) << 2;
+                red_or(marks ^ o, sm.ball[128 + 2 * suf]);
+                red_or((marks + M::kHalf) ^ o, sm.ball[128 + 2 * suf + 1]);
+                const uint32_t wh = (marks + (suf >> 5) * M::kHalf) ^ o, bit = 1u << (suf & 31u);
 #pragma unroll
                 for (int e = 1; e <= 3 * kMid; ++e)
                     red_or(wh ^ (sv_single<kMid>(e) << 2), bit);
@@ -226,7 +262,7 @@ __device__ __forceinline__ void sv_mark(const uint32_t *__restrict__ win, int W,
 
 // Does a window of the sequence lie within d of the string c? Warp-uniform.
 template <int kMid>
-__device__ __forceinline__ bool sv_occurs(const uint32_t *__restrict__ win, int W, int d, uint32_t c, int lane)
+__device__ __forceinline__ bool sv_occurs(const uint2 *__restrict__ win, int W, int d, uint2 c, int lane)
 {
     for (int w0 = 0; w0 < W; w0 += 32) {
         const int w = w0 + lane;
@@ -242,7 +278,7 @@ __device__ __forceinline__ bool sv_occurs(const uint32_t *__restrict__ win, int 
 // sequences within d, as the tree form finds them.
 template <int kMid>
 __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, uint64_t *raw, uint32_t *raw_count, uint32_t *flags,
-                                     const uint32_t *__restrict__ win, bool has, uint32_t c, int first, int lane)
+                                     const uint2 *__restrict__ win, bool has, uint2 c, int first, int lane)
 {
     const int n = inst->n, W = inst->W, d = inst->d, l = inst->l;
     uint32_t todo = __ballot_sync(kFull, has);
@@ -250,7 +286,7 @@ __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, uint64_t 
     while (todo) {
         const int src = __ffs(todo) - 1;
         todo &= todo - 1u;
-        const uint32_t cc = __shfl_sync(kFull, c, src);
+        const uint2 cc = make_uint2(__shfl_sync(kFull, c.x, src), __shfl_sync(kFull, c.y, src));
         bool ok = true;
         for (int i = first; ok && i < n; ++i)
             ok = sv_occurs<kMid>(win + (size_t)i * W, W, d, cc, lane);
@@ -279,13 +315,10 @@ __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, uint64_t 
         base = atomicAdd(raw_count, (uint32_t)all);
     base = __shfl_sync(kFull, base, 0) + (uint32_t)(incl - copies);
     if (copies > 0) {
-        constexpr uint32_t kMask = (1u << kMid) - 1u;
-        constexpr int kPre = sv_pre<kMid>();
         const int A = l - kMid - kSvSuf;
-        const uint32_t mh = (c >> (6 + kMid)) & kMask, ml = ((c >> 6) & kMask) ^ sv_fold<kMid>(mh);
-        const uint32_t pre_l = (c >> (6 + 2 * kMid)) & ((1u << kPre) - 1u), pre_h = c >> (6 + 2 * kMid + kPre);
-        const uint32_t h = pre_h | (mh << A) | (((c >> 3) & 7u) << (A + kMid));
-        const uint32_t lo = pre_l | (ml << A) | ((c & 7u) << (A + kMid));
+        const uint32_t mid = c.x >> 6;
+        const uint32_t h = (c.y >> 16) | ((mid >> kMid) << A) | (((c.x >> 3) & 7u) << (A + kMid));
+        const uint32_t lo = (c.y & 0xffffu) | (sv_lo<kMid>(mid) << A) | ((c.x & 7u) << (A + kMid));
         uint64_t key = 0;
         for (int k = 0; k < l; ++k)
             key = (key << 2) | (uint64_t)((((h >> k) & 1u) << 1) | ((lo >> k) & 1u));
@@ -301,10 +334,10 @@ __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, uint64_t 
 
 // The string of bit `bit` of mark word `at` ([half][word]) of a block.
 template <int kMid>
-__device__ __forceinline__ uint32_t sv_string(uint32_t block, int at, int bit)
+__device__ __forceinline__ uint2 sv_string(uint32_t prefix, int at, int bit)
 {
     constexpr int kWords = SvMarks<kMid>::kWords;
-    return block | ((uint32_t)(at & (kWords - 1)) << 6) | ((uint32_t)(at / kWords) << 5) | (uint32_t)bit;
+    return make_uint2(((uint32_t)(at & (kWords - 1)) << 6) | ((uint32_t)(at / kWords) << 5) | (uint32_t)bit, prefix);
 }
 
 // Bits of piece k whose counter exceeds v: the planes compared with v, low plane first.
@@ -319,59 +352,62 @@ __device__ __forceinline__ uint32_t sv_above(const uint32_t (&cnt)[kPlanes][kPie
 }
 
 template <int kShare>
-__device__ __forceinline__ void team_sync(int team)
+__device__ __forceinline__ void share_sync()
 {
     if (kShare == 1)
         __syncwarp();
     else
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(kShare * 32) : "memory");
+        __syncthreads();
 }
 
-// Copies the tables to shared memory (the caller synchronises) and places the
-// CTA's mark buffers, aligned to their size, before them.
+// Shared memory: the tables, then the buffers of marks at the next multiple of
+// kHalf of the shared address space, in which dynamic shared memory starts
+// after what the system reserves (`reserved`: 1 KB).
 template <int kMid>
-__device__ __forceinline__ SvSmem &sv_setup(unsigned char *raw, int buffers, unsigned char *&marks_ptr, uint32_t &marks0)
+__host__ __device__ constexpr uint32_t sv_marks_at(uint32_t reserved)
 {
     using M = SvMarks<kMid>;
+    return (reserved + (uint32_t)sizeof(SvSmem<kMid>) + M::kHalf - 1) / M::kHalf * M::kHalf;
+}
+template <int kMid>
+size_t sv_smem_bytes(int reserved, int buffers)
+{
+    return sv_marks_at<kMid>((uint32_t)reserved) - reserved + (size_t)buffers * SvMarks<kMid>::kBytes;
+}
+
+// Copies the tables to shared memory and clears the marks; returns the shared
+// address of the first buffer.
+template <int kMid>
+__device__ __forceinline__ uint32_t sv_setup(unsigned char *raw, int buffers)
+{
+    using M = SvMarks<kMid>;
+    SvSmem<kMid> &sm = *reinterpret_cast<SvSmem<kMid> *>(raw);
     const uint32_t raw0 = (uint32_t)__cvta_generic_to_shared(raw);
-    marks0 = (raw0 + M::kBytes - 1) & ~(M::kBytes - 1);
-    marks_ptr = raw + (marks0 - raw0);
-    SvSmem &sm = *reinterpret_cast<SvSmem *>(marks_ptr + buffers * M::kBytes);
+    const uint32_t marks0 = sv_marks_at<kMid>(raw0);
     const SvTable &tab = g_sv_table[kMid - 3];
-    for (int i = threadIdx.x; i < kSvGroupsMax * 32; i += kSvThreads)
+    for (int i = threadIdx.x; i < sv_groups<kMid>() * 32; i += kSvThreads)
         sm.change[i] = tab.change[i];
     for (int i = threadIdx.x; i < 4 * 64 * 2; i += kSvThreads)
         sm.ball[i] = (&g_sv_ball[0][0][0])[i];
     if (threadIdx.x < kSvMaxShell + 2)
         sm.first[threadIdx.x] = tab.first[threadIdx.x];
-    return sm;
-}
-
-// A lane's change of at most one letter (half a warp per half of the words) and of two.
-template <int kMid>
-__device__ __forceinline__ void sv_lane_changes(const SvSmem &sm, int lane, uint32_t &slot0,
-                                                uint32_t (&d2)[sv_groups2<kMid>()])
-{
-    slot0 = 0;
-#pragma unroll
-    for (int e = 0; e <= 3 * kMid; ++e)
-        slot0 = (lane & 15) == e ? sv_single<kMid>(e) << 2 : slot0;
-    slot0 ^= lane >= 16 ? SvMarks<kMid>::kHalf : 0u;
-#pragma unroll
-    for (int t = 0; t < sv_groups2<kMid>(); ++t)
-        d2[t] = sm.change[(sm.first[2] + t) * 32 + lane];
+    if (threadIdx.x < 3)
+        sm.alive[threadIdx.x] = 0;
+    uint4 *m4 = reinterpret_cast<uint4 *>(raw + (marks0 - raw0));
+    for (int i = threadIdx.x; i < buffers * (int)(M::kBytes / 16); i += kSvThreads)
+        m4[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    return marks0;
 }
 
 // Item it of a launch: its instance and block.
-template <int kMid>
 struct SvBlock {
     int I;
     InstDev in;
-    uint32_t block;        // the block's prefix, as in a window's word
-    const uint32_t *win;   // the instance's window words
-    __device__ __forceinline__ SvBlock(const SieveParams &p, long long it)
+    uint32_t prefix;     // the block's, as in a window's word
+    const uint2 *win;    // the instance's windows
+    __device__ __forceinline__ SvBlock(const SieveParams &p, long long it, int mid_letters)
     {
-        constexpr int kPre = sv_pre<kMid>();
         int lo = 0, hi = p.nseg - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -383,53 +419,47 @@ struct SvBlock {
         I = p.seg[lo].inst;
         in = p.inst[I];
         const uint32_t b = (uint32_t)(it - p.seg[lo].work_lo);   // the prefix letters' planes, hi above lo
-        const int A = in.l - kMid - kSvSuf;
-        block = ((b & ((1u << A) - 1u)) << (6 + 2 * kMid)) | ((b >> A) << (6 + 2 * kMid + kPre));
-        win = reinterpret_cast<const uint32_t *>(p.planes + in.plane_off);
+        const int A = in.l - mid_letters - kSvSuf;
+        prefix = (b & ((1u << A) - 1u)) | ((b >> A) << 16);
+        win = p.planes + in.plane_off;
     }
 };
 
-// Buffers of marks in a CTA: one per team of one warp, else two.
-template <int kShare>
+// Buffers of marks in a CTA: one per warp that works alone. A CTA that shares
+// a block marks sequence i in buffer i % 2, so that one barrier a sequence is
+// enough, where two buffers leave room for as many CTAs.
+template <int kMid, int kPlanes, int kShare>
 __host__ __device__ constexpr int sv_buffers()
 {
-    return kShare == 1 ? kSvWarps : 2 * kSvWarps / kShare;
+    return kShare == 1 ? kSvWarps : (kPlanes == 0 && kMid <= 5 ? 2 : 1);
 }
 
-// Items are blocks; a team of kShare warps of a CTA takes one at a time and
-// its warps split the windows of every sequence. kPlanes = 0: q = n, a thread
-// keeps its share of the strings alive in registers, and a block ends once
-// none is alive or the last few have been looked up window by window.
-// kPlanes > 0: the quorum form, kPlanes bit-sliced hit counters (kShare = 1).
+// Items are blocks; kShare warps take one at a time (1, or all of the CTA) and
+// split the windows of every sequence. kPlanes = 0: q = n, a thread keeps its
+// share of the strings alive in registers, and a block ends once none is alive
+// or the last few have been looked up window by window. kPlanes > 0: the quorum
+// form, kPlanes bit-sliced hit counters.
 template <int kMid, int kPlanes, int kShare, int kMinBlocks>
 __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SieveParams p)
 {
     extern __shared__ __align__(16) unsigned char sv_raw[];
     using M = SvMarks<kMid>;
+    static_assert(kShare == 1 || kShare == kSvWarps, "a warp or the CTA works on a block");
     constexpr int kPieces = 2 * M::kWords / (32 * kShare);   // mark words of a thread
     constexpr int kVec = kPieces % 4 == 0 ? 4 : 1;           // of them in one access
-    constexpr int kPre = sv_pre<kMid>();
+    constexpr int kAll = sv_buffers<kMid, kPlanes, kShare>();
+    constexpr int kBuf = kShare == 1 ? 1 : kAll;             // buffers a block uses
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int team = warp / kShare, g = warp % kShare;
-    unsigned char *marks_ptr;
-    uint32_t marks0;
-    SvSmem &sm = sv_setup<kMid>(sv_raw, sv_buffers<kShare>(), marks_ptr, marks0);
-    if (threadIdx.x < 3 * kSvWarps)
-        (&sm.alive[0][0])[threadIdx.x] = 0;
-    // a team of several warps marks sequence i in buffer i % 2, so that one
-    // barrier a sequence is enough
-    constexpr int kBuf = kShare > 1 ? 2 : 1;
-    const uint32_t marks = marks0 + team * kBuf * M::kBytes;
-    uint32_t *mw = reinterpret_cast<uint32_t *>(marks_ptr + team * kBuf * M::kBytes);
-    // piece k of this thread: mark word sv_at(k)
+    const int g = kShare == 1 ? 0 : warp, own = kShare == 1 ? warp : 0;
+    SvSmem<kMid> &sm = *reinterpret_cast<SvSmem<kMid> *>(sv_raw);
+    const uint32_t marks0 = sv_setup<kMid>(sv_raw, kAll);
+    const uint32_t marks = marks0 + own * M::kBytes;
+    uint32_t *mw =
+        reinterpret_cast<uint32_t *>(sv_raw + (marks - (uint32_t)__cvta_generic_to_shared(sv_raw)));
+    // piece k of this thread
     const int tid = g * 32 + lane;
     auto at_of = [&](int k) { return (k / kVec) * (32 * kShare * kVec) + tid * kVec + k % kVec; };
-#pragma unroll
-    for (int k = 0; k < kPieces * kBuf; ++k)
-        mw[at_of(k)] = 0u;
-    __syncthreads();
-    uint32_t slot0, d2[sv_groups2<kMid>()];
-    sv_lane_changes<kMid>(sm, lane, slot0, d2);
+    const SvLane<kMid> my(sm, lane);
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the packed windows are complete and visible
     for (;;) {
         long long it = 0;
@@ -439,18 +469,18 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
             it = __shfl_sync(kFull, it, 0);
         }
         if (kShare > 1) {
-            if (g == 0 && lane == 0)
-                sm.item[team] = it;
-            team_sync<kShare>(team);
-            it = sm.item[team];
-            team_sync<kShare>(team);
+            __syncthreads();   // the last item has been read, the counters of its block too
+            if (threadIdx.x == 0)
+                sm.item = it;
+            if (threadIdx.x < 3)
+                sm.alive[threadIdx.x] = 0;
+            __syncthreads();
+            it = sm.item;
         }
         if (it >= p.total)
             break;
-        SvBlock<kMid> blk(p, it);
+        SvBlock blk(p, it, kMid);
         const InstDev &in = blk.in;
-        const uint32_t block = blk.block;
-        const uint32_t *win = blk.win;
         // what is left of the block's strings goes back to its marks
         uint32_t left = 0;   // != 0: this thread holds some
         int i = 0;
@@ -460,16 +490,16 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
             for (int k = 0; k < kPieces; ++k)
                 cur[k] = kFull;
             while (i < in.n) {
-                const uint32_t buf = kShare > 1 ? (uint32_t)(i & 1) : 0u;
+                const uint32_t buf = kBuf > 1 ? (uint32_t)(i & 1) : 0u;
                 uint32_t *mb = mw + buf * (2 * M::kWords);
-                sv_mark<kMid, kShare>(win + (size_t)i * in.W, in.W, in.d, block, marks + buf * M::kBytes, sm.list[warp],
-                                      sm, slot0, d2, g, lane);
-                team_sync<kShare>(team);
+                sv_mark<kMid, kShare>(blk.win + (size_t)i * in.W, in.W, in.d, blk.prefix, marks + buf * M::kBytes,
+                                      sm.list[warp], sm, my, g, lane);
+                share_sync<kShare>();
                 int lanes = 32 * kShare;
-                if (kShare > 1 && i > 0) {   // after the sequence before
-                    lanes = *(volatile int *)&sm.alive[team][(i - 1) % 3];
-                    if (g == 0 && lane == 0)
-                        *(volatile int *)&sm.alive[team][(i + 1) % 3] = 0;
+                if (kBuf > 1 && i > 0) {   // after the sequence before
+                    lanes = *(volatile int *)&sm.alive[(i - 1) % 3];
+                    if (threadIdx.x == 0)
+                        *(volatile int *)&sm.alive[(i + 1) % 3] = 0;
                 }
                 left = 0;
 #pragma unroll
@@ -490,22 +520,26 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                     }
                 }
                 const int mine = __popc(__ballot_sync(kFull, left != 0u));
-                if (kShare > 1) {
-                    if (lane == 0)
-                        atomicAdd(&sm.alive[team][i % 3], mine);
-                } else {
+                if (kShare == 1) {
                     __syncwarp();
                     lanes = mine;
+                } else if (lane == 0) {
+                    atomicAdd(&sm.alive[i % 3], mine);
+                }
+                if (kShare > 1 && kBuf == 1) {
+                    // everybody has added, and the marks are clear; the slot read
+                    // here is cleared two sequences later at the earliest
+                    __syncthreads();
+                    lanes = *(volatile int *)&sm.alive[i % 3];
+                    if (threadIdx.x == 0)
+                        *(volatile int *)&sm.alive[(i + 1) % 3] = 0;
                 }
                 ++i;
                 if (lanes <= kSvLookupLanes)
                     break;
             }
-            if (kShare > 1) {   // the counters are zero again before the next block
-                team_sync<kShare>(team);
-                if (g == 0 && lane < 3)
-                    sm.alive[team][lane] = 0;
-            }
+            if (kBuf > 1)
+                __syncthreads();   // a buffer's marks are all taken before strings are put into it
             if (__any_sync(kFull, left != 0u)) {
 #pragma unroll
                 for (int k = 0; k < kPieces; ++k)
@@ -519,8 +553,8 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                 for (int k = 0; k < kPieces; ++k)
                     cnt[s][k] = 0u;
             while (i < in.n) {
-                sv_mark<kMid, 1>(win + (size_t)i * in.W, in.W, in.d, block, marks, sm.list[warp], sm, slot0, d2, 0, lane);
-                __syncwarp();
+                sv_mark<kMid, kShare>(blk.win + (size_t)i * in.W, in.W, in.d, blk.prefix, marks, sm.list[warp], sm, my, g, lane);
+                share_sync<kShare>();
 #pragma unroll
                 for (int k = 0; k < kPieces; ++k) {
                     uint32_t m = mw[at_of(k)];
@@ -532,18 +566,22 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                         m &= c;
                     }
                 }
-                __syncwarp();
                 ++i;
                 // a string needs q - (n - i) hits by now; the block ends once none has them
                 const int need1 = in.q - (in.n - i) - 1;
-                if (need1 < 0)
-                    continue;
                 left = 0;
+                if (need1 >= 0) {
 #pragma unroll
-                for (int k = 0; k < kPieces; ++k)
-                    left |= sv_above<kPlanes, kPieces>(cnt, k, need1);
-                if (!__any_sync(kFull, left != 0u))
+                    for (int k = 0; k < kPieces; ++k)
+                        left |= sv_above<kPlanes, kPieces>(cnt, k, need1);
+                }
+                if (kShare == 1) {
+                    __syncwarp();
+                    if (!__any_sync(kFull, need1 < 0 || left != 0u))
+                        break;
+                } else if (!__syncthreads_or(need1 < 0 || left != 0u)) {
                     break;
+                }
             }
             if (__any_sync(kFull, left != 0u)) {
 #pragma unroll
@@ -566,8 +604,8 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                         const bool has = v != 0u;
                         const int bit = has ? __ffs(v) - 1 : 0;
                         v &= v - 1u;
-                        sv_emit<kMid>(p.inst + blk.I, p.raw, p.raw_count + blk.I, p.flags + blk.I, win, has,
-                                      sv_string<kMid>(block, at, bit), i, lane);
+                        sv_emit<kMid>(p.inst + blk.I, p.raw, p.raw_count + blk.I, p.flags + blk.I, blk.win, has,
+                                      sv_string<kMid>(blk.prefix, at, bit), i, lane);
                     }
                 }
             }
@@ -591,32 +629,26 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_split_kernel(Sie
     using M = SvMarks<kMid>;
     constexpr int kPieces = 2 * M::kWords / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned char *marks_ptr;
-    uint32_t marks0;
-    SvSmem &sm = sv_setup<kMid>(sv_raw, kSvWarps, marks_ptr, marks0);
+    SvSmem<kMid> &sm = *reinterpret_cast<SvSmem<kMid> *>(sv_raw);
+    const uint32_t marks0 = sv_setup<kMid>(sv_raw, kSvWarps);
     const uint32_t marks = marks0 + warp * M::kBytes;
-    uint32_t *all = reinterpret_cast<uint32_t *>(marks_ptr);
+    uint32_t *all = reinterpret_cast<uint32_t *>(sv_raw + (marks0 - (uint32_t)__cvta_generic_to_shared(sv_raw)));
     uint32_t *mw = all + warp * (2 * M::kWords);
-    int *dead = &sm.alive[0][0];
-#pragma unroll
-    for (int k = 0; k < kPieces; ++k)
-        mw[k * 32 + lane] = 0u;
-    __syncthreads();
-    uint32_t slot0, d2[sv_groups2<kMid>()];
-    sv_lane_changes<kMid>(sm, lane, slot0, d2);
+    int *dead = &sm.alive[0];
+    const SvLane<kMid> my(sm, lane);
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the packed windows are complete and visible
     for (long long it = blockIdx.x; it < p.total; it += gridDim.x) {
         if (threadIdx.x == 0)
             *dead = 0;
         __syncthreads();
-        SvBlock<kMid> blk(p, it);
+        SvBlock blk(p, it, kMid);
         const InstDev &in = blk.in;
         uint32_t cur[kPieces];
 #pragma unroll
         for (int k = 0; k < kPieces; ++k)
             cur[k] = kFull;
         for (int i = warp; i < in.n && !*(volatile int *)dead; i += kSvWarps) {
-            sv_mark<kMid, 1>(blk.win + (size_t)i * in.W, in.W, in.d, blk.block, marks, sm.list[warp], sm, slot0, d2, 0,
+            sv_mark<kMid, 1>(blk.win + (size_t)i * in.W, in.W, in.d, blk.prefix, marks, sm.list[warp], sm, my, 0,
                              lane);
             __syncwarp();
             uint32_t left = 0;
@@ -646,7 +678,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_split_kernel(Sie
                     const int bit = has ? __ffs(v) - 1 : 0;
                     v &= v - 1u;
                     sv_emit<kMid>(p.inst + blk.I, p.raw, p.raw_count + blk.I, p.flags + blk.I, blk.win, has,
-                                  sv_string<kMid>(blk.block, at, bit), in.n, lane);
+                                  sv_string<kMid>(blk.prefix, at, bit), in.n, lane);
                 }
             }
         }
@@ -668,7 +700,7 @@ void fill_table(SvTable &t)
         t.first[shell] = group;
         if (shell <= kMid) {
             // every change of `shell` middle letters, by bank
-            uint16_t bank[32][256];
+            uint16_t bank[32][128];
             int nb[32] = {}, total = 0;
             for (uint32_t hi = 0; hi < (1u << kMid); ++hi)
                 for (uint32_t lo = 0; lo < (1u << kMid); ++lo) {
@@ -720,30 +752,30 @@ cudaError_t launch_kernel(void (*kernel)(SieveParams), const SieveParams &p, lon
 }
 
 template <int kMid, int kPlanes, int kShare, int kMinBlocks>
-cudaError_t launch(const SieveParams &p, int sms, cudaStream_t st)
+cudaError_t launch(const SieveParams &p, int sms, int reserved, cudaStream_t st)
 {
-    const size_t smem = (sv_buffers<kShare>() + 1) * (size_t)SvMarks<kMid>::kBytes + sizeof(SvSmem);
     const long long teams = kSvWarps / kShare;
     return launch_kernel(sieve_kernel<kMid, kPlanes, kShare, kMinBlocks>, p,
-                         std::min<long long>((long long)sms * kMinBlocks, (p.total + teams - 1) / teams), smem, st);
+                         std::min<long long>((long long)sms * kMinBlocks, (p.total + teams - 1) / teams),
+                         sv_smem_bytes<kMid>(reserved, sv_buffers<kMid, kPlanes, kShare>()), st);
 }
 
 template <int kMid, int kMinBlocks>
-cudaError_t launch_split(const SieveParams &p, int sms, cudaStream_t st)
+cudaError_t launch_split(const SieveParams &p, int sms, int reserved, cudaStream_t st)
 {
-    const size_t smem = (kSvWarps + 1) * (size_t)SvMarks<kMid>::kBytes + sizeof(SvSmem);
-    return launch_kernel(sieve_split_kernel<kMid, kMinBlocks>, p,
-                         std::min<long long>((long long)sms * kMinBlocks, p.total), smem, st);
+    return launch_kernel(sieve_split_kernel<kMid, kMinBlocks>, p, std::min<long long>((long long)sms * kMinBlocks, p.total),
+                         sv_smem_bytes<kMid>(reserved, kSvWarps), st);
 }
 
 }  // namespace
 
 cudaError_t sieve_init_tables()
 {
-    static SvTable t[3];
+    static SvTable t[4];
     fill_table<3>(t[0]);
     fill_table<4>(t[1]);
     fill_table<5>(t[2]);
+    fill_table<6>(t[3]);
     uint32_t ball[4][64][2] = {};
     for (int v = 0; v < 4; ++v)
         for (int s = 0; s < 64; ++s)
@@ -760,13 +792,23 @@ cudaError_t sieve_init_tables()
 
 cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, int sms, cudaStream_t st)
 {
+    int dev = 0, reserved = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (e != cudaSuccess)
+        return e;
     if (planes > 0)
-        return mid == 4 ? launch<4, 5, 1, 2>(p, sms, st) : launch<3, 7, 1, 3>(p, sms, st);
+        return mid == 5   ? launch<5, 5, 8, 3>(p, sms, reserved, st)
+               : mid == 4 ? launch<4, 5, 1, 2>(p, sms, reserved, st)
+                          : launch<3, 7, 1, 3>(p, sms, reserved, st);
+    if (mid == 6)
+        return launch<6, 0, 8, 4>(p, sms, reserved, st);
     if (mid == 5)
-        return share == 1 ? launch<5, 0, 1, 2>(p, sms, st) : launch<5, 0, 8, 4>(p, sms, st);
+        return share == 1 ? launch<5, 0, 1, 2>(p, sms, reserved, st) : launch<5, 0, 8, 4>(p, sms, reserved, st);
     if (mid == 4)
-        return share == 1 ? launch<4, 0, 1, 4>(p, sms, st) : launch_split<4, 5>(p, sms, st);
-    return share == 1 ? launch<3, 0, 1, 5>(p, sms, st) : launch_split<3, 5>(p, sms, st);
+        return share == 1 ? launch<4, 0, 1, 4>(p, sms, reserved, st) : launch_split<4, 5>(p, sms, reserved, st);
+    return share == 1 ? launch<3, 0, 1, 5>(p, sms, reserved, st) : launch_split<3, 5>(p, sms, reserved, st);
 }
 
 }  // namespace pms

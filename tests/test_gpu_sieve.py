@@ -9,14 +9,14 @@ import paper_2403_00306_gb300 as pms
 pytestmark = pytest.mark.gpu
 
 # l = 8..10: 3 middle letters (8 and 9: almost no prefix); 11: 4; 12, 13: 5, a CTA per block;
-# 14..16: 5, a warp per block (16: the longest prefix); W around 32 and one window per sequence;
+# 14 and more: 5, a warp per block, or 6, a CTA per block; W around 32 and one window per sequence;
 # more sequences than a CTA has warps; more changes than middle letters
 SMALL = [(2, 9, 9, 2), (2, 40, 8, 1), (3, 39, 8, 1), (9, 40, 9, 2), (17, 41, 9, 1), (5, 64, 10, 3), (64, 42, 10, 4),
          (8, 43, 11, 3), (6, 11, 11, 5), (9, 75, 12, 4), (20, 96, 13, 4), (12, 45, 13, 6), (7, 46, 14, 5),
-         (10, 60, 15, 5), (5, 16, 16, 4), (12, 50, 16, 6)]
+         (10, 60, 15, 5), (5, 16, 16, 4), (12, 50, 16, 6), (4, 300, 14, 4), (10, 290, 15, 5), (20, 80, 16, 6)]
 # 5 counter planes up to 31 sequences and l >= 12, else 7
 QUORUM = [(5, 60, 9, 1, 3), (12, 64, 10, 2, 10), (31, 50, 12, 3, 28), (32, 50, 12, 3, 29), (64, 40, 11, 3, 60),
-          (8, 50, 13, 4, 7), (6, 40, 15, 4, 5), (10, 48, 16, 5, 9), (4, 30, 9, 2, 1)]
+          (8, 50, 13, 4, 7), (6, 40, 15, 4, 5), (31, 300, 13, 4, 29), (10, 48, 16, 5, 9), (4, 30, 9, 2, 1)]
 
 
 @pytest.mark.parametrize("case", SMALL, ids=str)
@@ -41,6 +41,7 @@ def test_sieve_quorum_matches_oracle(oracle_, case):
 
 @pytest.mark.parametrize("case", [(9, 2, 20, 600, 0), (11, 3, 17, 733, 0), (12, 3, 25, 1000, 0), (13, 4, 20, 600, 0),
                                   (14, 4, 13, 999, 0), (15, 4, 20, 1100, 0), (15, 5, 20, 301, 0), (16, 5, 20, 250, 0),
+                                  (17, 5, 20, 1150, 0), (18, 6, 20, 400, 0),
                                   (13, 4, 20, 300, 18), (15, 4, 15, 200, 12), (12, 3, 40, 400, 37)], ids=str)
 def test_sieve_and_tree_form_agree(case):
     """Whole motif sets and, on the device entry point, raw counts (a motif once per seed window near it)."""
