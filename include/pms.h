@@ -167,7 +167,8 @@ typedef struct {
  * pms_solve_batch / pms_solve_sigma). For the DNA solves the comparison
  * counters are filled only when pms_options.count_work was set for that
  * solve; pms_solve_sigma always fills them (subsets = tree nodes visited,
- * candidates_tested = checks of full candidates, cmp_rows / cmp_reduce /
+ * candidates_tested = checks of full candidates (with q = n and d <= 4: those
+ * left by the first sequences' marks), cmp_rows / cmp_reduce /
  * cmp_verify = window, node-bound and candidate-versus-row comparisons). */
 typedef struct {
     uint64_t candidates;        /* size of the searched space: sum over seeds of |B(x,d)| */

@@ -19,7 +19,7 @@ LIB = os.path.join(OUT_DIR, "libpms.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "-diag-suppress", "550", "-I", os.path.join(ROOT, "include")]
-UNITS = ["pms_kernels.cu", "pms_runtime.cu", "pms_sieve.cu", "pms_sigma.cu"]
+UNITS = ["pms_kernels.cu", "pms_runtime.cu", "pms_sieve.cu", "pms_sigma.cu", "pms_sigma_sieve.cu"]
 
 
 def _nvcc() -> str:

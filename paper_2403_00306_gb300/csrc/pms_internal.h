@@ -258,13 +258,29 @@ struct SigmaParams {
     int list_cap;
 };
 
+// The sieve form of a node's letters (pms_sigma_sieve.cu): q = n, d <= 4.
+struct SigmaSieve {
+    const unsigned long long *letters;   // window (i, j): letter p in bits b p .. b p + b - 1, at i * W + j
+    int parts;          // items a seed's nodes are split into
+    int warp_words;     // map words of a warp
+    int map_words;      // map words of a CTA
+    int row_bytes;      // shared or scratch bytes of a row
+};
+constexpr int kSsMaskWords = 2048;             // row masks of one seed kept in shared memory
+constexpr int kSsSmemMax = 200 * 1024;         // dynamic shared memory of a CTA at most
+bool sigma_sieve_plan(int n, int l, int d, int b, int sigma, SigmaSieve *q);
+size_t sigma_sieve_smem(const SigmaSieve &q, int rows);
+cudaError_t sigma_sieve_init();
+cudaError_t sigma_sieve_occupancy(const SigmaSieve &q, int rows, int *blocks_per_sm);
+cudaError_t launch_sigma_sieve(const SigmaParams &p, const SigmaSieve &q, int blocks, cudaStream_t st);
+
 int sigma_planes(int sigma);
 size_t sigma_row_bytes(int b, int l);   // shared or scratch bytes of one seed row
 int sigma_smem_rows(int b, int l, bool large);
 cudaError_t sigma_init_tables();
 cudaError_t sigma_main_occupancy(int b, int l, bool large, int *blocks_per_sm);
 cudaError_t launch_sigma_pack(const uint8_t *seqs, int n, int m, int l, int b, const SigmaMap &map, uint32_t *planes,
-                              uint32_t *flags, cudaStream_t st);
+                              unsigned long long *letters, uint32_t *flags, cudaStream_t st);
 cudaError_t launch_sigma_main(const SigmaParams &p, int blocks, cudaStream_t st);
 // Device state of the sort/unique kernel's CTAs (one grid, all CTAs resident):
 // hist holds sigma_sort_hist_words(ctas) words (per-CTA digit counts, digit

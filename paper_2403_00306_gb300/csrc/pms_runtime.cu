@@ -219,7 +219,7 @@ struct pms_ctx {
     };
     DBuf d_seqs, d_planes, d_raw, d_tmp, d_compat, d_rowlen, d_mode, d_meta, d_ctr, d_scratch, d_result;
     // general-alphabet solves (pms_solve_sigma)
-    DBuf d_sg_seqs, d_sg_planes, d_sg_ctr, d_sg_raw, d_sg_out, d_sg_scratch, d_sg_lists, d_sg_hist;
+    DBuf d_sg_seqs, d_sg_planes, d_sg_ctr, d_sg_raw, d_sg_out, d_sg_scratch, d_sg_lists, d_sg_hist, d_sg_letters;
     bool sigma_ready = false;   // binomial table and kernel attributes loaded on the device
     int sg_sort_ctas = 1;       // CTAs of the sort/unique grid
     void *h_sg = nullptr;       // pinned, mapped: counters block, then the input letters
@@ -2738,7 +2738,8 @@ int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_
     cudaSetDevice(h->device);
     cudaError_t e;
     if (!h->sigma_ready) {
-        if ((e = sigma_init_tables()) != cudaSuccess || (e = sigma_sort_ctas(&h->sg_sort_ctas)) != cudaSuccess)
+        if ((e = sigma_init_tables()) != cudaSuccess || (e = sigma_sieve_init()) != cudaSuccess ||
+            (e = sigma_sort_ctas(&h->sg_sort_ctas)) != cudaSuccess)
             return h->cuda_fail(e, "general-alphabet tables");
         h->sigma_ready = true;
     }
@@ -2759,13 +2760,34 @@ int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_
             p_row += (double)binom(l, j) * std::pow(pm, j) * std::pow(1.0 - pm, l - j);
     }
     const bool large = p_row * max_rows > 0.8 * sigma_smem_rows(b, l, false);
+    // the sieve form of a node's letters, and room for about every seed's rows
+    SigmaSieve sieve{};
+    const bool sieved = qe == n && sigma_sieve_plan(n, l, d, b, sigma, &sieve);
+    int smem_rows = sigma_smem_rows(b, l, large);
+    if (sieved) {
+        const int most = (int)((kSsSmemMax - sigma_sieve_smem(sieve, 0)) / sieve.row_bytes);
+        smem_rows = (int)std::min<double>({1.1 * p_row * max_rows + 256.0, (double)max_rows, (double)most}) & ~1;
+        if (h->opt.smem_rows > 0)
+            smem_rows = std::min(smem_rows, h->opt.smem_rows & ~1);
+        smem_rows = std::max(smem_rows, 2);
+    }
     int occ = 0;
-    if ((e = sigma_main_occupancy(b, l, large, &occ)) != cudaSuccess)
+    if ((e = sieved ? sigma_sieve_occupancy(sieve, smem_rows, &occ)
+                    : sigma_main_occupancy(b, l, large, &occ)) != cudaSuccess)
         return h->cuda_fail(e, "occupancy");
     occ = std::max(occ, 1);
     const int per_sm = h->opt.ctas_per_sm > 0 ? std::min(h->opt.ctas_per_sm, occ) : occ;
     int blocks = (int)std::max(1LL, std::min<long long>((long long)h->num_sms * per_sm, nseeds));
-    const int smem_rows = sigma_smem_rows(b, l, large);
+    if (sieved) {
+        // seeds with many nodes in two items each, few seeds in more, so that the
+        // last round of CTAs costs little (protein (9,4), m = 600: 3.30 -> 2.84 ms;
+        // (9,3), whose nodes take no longer than a seed's rows, 148 us whole, 171 us in two)
+        const int slots = h->num_sms * per_sm;
+        sieve.parts = d == 4 ? 2 : 1;
+        while (sieve.parts < 8 && nseeds * sieve.parts < slots / 2)
+            sieve.parts *= 2;
+        blocks = (int)std::min<long long>(slots, (long long)nseeds * sieve.parts);
+    }
     const int scratch_rows = (max_rows + 1) & ~1;   // even: packed rows are 8-byte words
     if (max_rows > smem_rows) {
         // every CTA may need global scratch for a seed's rows: keep it within 2 GiB
@@ -2795,7 +2817,12 @@ int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_
     // per warp: the row lists of the search's depths (nodes whose lists would not fit keep the
     // search without them; without room for the buffer within the budget, every node does)
     int list_cap = kSigListCap;
-    if (h->ensure(h->d_sg_lists, (size_t)4 * blocks * (kSigThreads / 32) * list_cap) != PMS_OK) {
+    if (sieved) {
+        list_cap = 0;
+        if ((rc = h->ensure(h->d_sg_letters, 8 * NW)))
+            return rc;
+        sieve.letters = (const unsigned long long *)h->d_sg_letters.p;
+    } else if (h->ensure(h->d_sg_lists, (size_t)4 * blocks * (kSigThreads / 32) * list_cap) != PMS_OK) {
         list_cap = 0;
         h->err.clear();
     }
@@ -2854,8 +2881,10 @@ int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_
              (e = cudaMemcpyAsync(h->d_sg_seqs.p, h_ctr + 256, nm, cudaMemcpyHostToDevice, st)) != cudaSuccess) ||
             (e = cudaMemsetAsync(c, 0, ctr_bytes, st)) != cudaSuccess || (e = cudaEventRecord(h->ev0, st)) != cudaSuccess ||
             (e = launch_sigma_pack(seq_src, n, m, l, b, map, (uint32_t *)h->d_sg_planes.p,
-                                   (uint32_t *)(c + 24), st)) != cudaSuccess ||
-            (e = cudaEventRecord(h->evm0, st)) != cudaSuccess || (e = launch_sigma_main(p, blocks, st)) != cudaSuccess ||
+                                   sieved ? (unsigned long long *)h->d_sg_letters.p : nullptr, (uint32_t *)(c + 24),
+                                   st)) != cudaSuccess ||
+            (e = cudaEventRecord(h->evm0, st)) != cudaSuccess ||
+            (e = sieved ? launch_sigma_sieve(p, sieve, blocks, st) : launch_sigma_main(p, blocks, st)) != cudaSuccess ||
             (e = cudaEventRecord(h->evm1, st)) != cudaSuccess ||
             (e = launch_sigma_sort_unique(p.raw, p.raw + 3 * cap, p.raw_count, cap, l, b, letters,
                                           out_ptr, (unsigned long long *)(c + 16),
@@ -2932,7 +2961,7 @@ void pms_destroy(pms_ctx *h)
         cudaStreamDestroy(h->cap_stream);
     pms_ctx::DBuf *bufs[] = {&h->d_seqs, &h->d_planes, &h->d_raw, &h->d_tmp, &h->d_compat, &h->d_rowlen, &h->d_mode, &h->d_meta, &h->d_ctr, &h->d_scratch, &h->d_result,
                              &h->d_sg_seqs, &h->d_sg_planes, &h->d_sg_ctr, &h->d_sg_raw, &h->d_sg_out, &h->d_sg_scratch,
-                             &h->d_sg_lists, &h->d_sg_hist};
+                             &h->d_sg_lists, &h->d_sg_hist, &h->d_sg_letters};
     for (auto *b : bufs)
         h->dev_free(b->p, b->cap);
     if (h->h_result)

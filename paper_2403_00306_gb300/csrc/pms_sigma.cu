@@ -781,10 +781,12 @@ struct SgDeviceSink {
     }
 };
 
-// One thread per window: letter indices into b bit-planes; a byte outside the
+// One thread per window: letter indices into b bit-planes and, for the sieve
+// form (letters, b l <= 64), side by side in one word; a byte outside the
 // alphabet sets flags[0] bit 0.
 __global__ void sigma_pack_kernel(const uint8_t *__restrict__ seqs, int n, int m, int l, int b, SigmaMap map,
-                                  uint32_t *__restrict__ planes, uint32_t *__restrict__ flags)
+                                  uint32_t *__restrict__ planes, unsigned long long *__restrict__ letters,
+                                  uint32_t *__restrict__ flags)
 {
     const int W = m - l + 1;
     const long long NW = (long long)n * W;
@@ -794,6 +796,7 @@ __global__ void sigma_pack_kernel(const uint8_t *__restrict__ seqs, int n, int m
         const int j = (int)(w - (long long)i * W);
         const uint8_t *s = seqs + (size_t)i * m + j;
         uint32_t pl[kSigMaxPlanes] = {0u, 0u, 0u, 0u, 0u};
+        unsigned long long packed = 0;
         bool bad = false;
         for (int k = 0; k < l; ++k) {
             const unsigned a = map.v[s[k]];
@@ -803,7 +806,11 @@ __global__ void sigma_pack_kernel(const uint8_t *__restrict__ seqs, int n, int m
             }
             for (int g = 0; g < kSigMaxPlanes; ++g)
                 pl[g] |= ((a >> g) & 1u) << k;
+            if (letters)
+                packed |= (unsigned long long)a << (b * k);
         }
+        if (letters)
+            letters[w] = packed;
         if (bad)
             atomicOr(flags, 1u);
         for (int g = 0; g < b; ++g)
@@ -1304,12 +1311,12 @@ cudaError_t sigma_main_occupancy(int b, int l, bool large, int *blocks_per_sm)
 }
 
 cudaError_t launch_sigma_pack(const uint8_t *seqs, int n, int m, int l, int b, const SigmaMap &map, uint32_t *planes,
-                              uint32_t *flags, cudaStream_t st)
+                              unsigned long long *letters, uint32_t *flags, cudaStream_t st)
 {
     const long long NW = (long long)n * (m - l + 1);
     const int threads = 256;
     const int blocks = (int)((NW + threads - 1) / threads);
-    sigma_pack_kernel<<<blocks, threads, 0, st>>>(seqs, n, m, l, b, map, planes, flags);
+    sigma_pack_kernel<<<blocks, threads, 0, st>>>(seqs, n, m, l, b, map, planes, letters, flags);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,32 @@
+"""The general-alphabet search with d <= 4 and q = n (tuples of a node's letters in a bit map) against
+the oracle, at its edges: nodes of 0 to 4 letters, alphabets of 3 to 32, maps of one and two sizes,
+rows whose masks share a word with their letters or not, more rows than a list, a sequence or shared
+memory holds, more row masks than are kept."""
+import numpy as np
+import pytest
+
+import planted_inputs as pi
+import paper_2403_00306_gb300 as pms
+
+pytestmark = pytest.mark.gpu
+
+ALPHABET = b"ACDEFGHIKLMNPQRSTVWYBJOUXZabcdef"
+
+# (sigma, l, d, n, m)
+CASES = [(3, 6, 4, 9, 40), (3, 16, 4, 6, 60), (4, 5, 4, 3, 20), (4, 8, 3, 12, 70), (5, 7, 4, 10, 33), (8, 6, 4, 8, 50),
+         (20, 5, 4, 20, 7), (20, 6, 4, 6, 18), (20, 9, 0, 3, 40), (20, 7, 1, 4, 50), (20, 8, 2, 5, 60), (20, 9, 3, 6, 50),
+         (20, 12, 3, 4, 60), (22, 5, 3, 5, 24), (23, 5, 3, 5, 24), (32, 5, 3, 4, 20), (32, 5, 4, 10, 6), (32, 12, 2, 3, 40),
+         (4, 5, 3, 64, 60), (4, 32, 4, 3, 40), (4, 6, 4, 6, 450), (20, 9, 1, 64, 1100), (20, 4, 3, 3, 9)]
+
+
+@pytest.mark.parametrize("case", CASES, ids=str)
+def test_matches_oracle(oracle_, case):
+    sigma, l, d, n, m = case
+    alphabet = ALPHABET[:sigma]
+    inst = pi.planted_instance_sigma(n, m, l, min(d, l), 5, alphabet)
+    want = oracle_.sigma_solve(inst.seqs, l, d, alphabet)
+    with pms.Context(0) as c:
+        got = c.solve_sigma(inst.seqs, l, d, alphabet)
+        assert np.array_equal(got, want), (len(got), len(want))
+        c.set_options(ctas_per_sm=1, smem_rows=8)    # few CTAs, rows in global scratch
+        assert np.array_equal(c.solve_sigma(inst.seqs, l, d, alphabet), want)
