@@ -432,23 +432,31 @@ __global__ void __launch_bounds__(kSsThreads, kMinBlocks) sigma_sieve_kernel(Sig
         for (int g = 0; g < kSigMaxPlanes; ++g)
             x[g] = g < p.b ? p.planes[(size_t)g * NW + seed] : 0u;   // a window of s_1
         auto differs = [&](int i, int w) {
+            const uint32_t *at = p.planes + (i * p.W + w);   // n W < 2^22
             uint32_t mm = 0;
 #pragma unroll
             for (int g = 0; g < kSigMaxPlanes; ++g)
                 if (g < p.b)
-                    mm |= x[g] ^ __ldg(p.planes + (size_t)g * NW + (size_t)i * p.W + w);
+                    mm |= x[g] ^ __ldg(at + g * NW);
             return mm;
         };
         for (int i = warp; i < p.n; i += kSsWarps) {
             int cnt = 0;
             if (i != 0)
-                for (int c = 0; c < NWm; ++c) {
-                    const int w = 32 * c + lane;
-                    const uint32_t bal =
-                        __ballot_sync(kFull, w < p.W && __popc(differs(i, min(w, p.W - 1))) <= 2 * p.d);
-                    if (masks && lane == 0)
-                        s_mask[i * NWm + c] = bal;
-                    cnt += __popc(bal);
+                for (int c0 = 0; c0 < NWm; c0 += 4) {
+                    // four groups of 32 windows, their loads in flight together
+                    uint32_t mm[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        mm[u] = differs(i, min(32 * (c0 + u) + lane, p.W - 1));
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t bal =
+                            __ballot_sync(kFull, 32 * (c0 + u) + lane < p.W && __popc(mm[u]) <= 2 * p.d);
+                        if (masks && lane == 0 && c0 + u < NWm)
+                            s_mask[i * NWm + c0 + u] = bal;
+                        cnt += __popc(bal);
+                    }
                 }
             if (lane == 0)
                 s_cnt[i] = cnt;
@@ -489,6 +497,7 @@ __global__ void __launch_bounds__(kSsThreads, kMinBlocks) sigma_sieve_kernel(Sig
             }
             for (int i = 1 + warp; i < p.n; i += kSsWarps) {
                 int e = s_off[i];
+#pragma unroll 2
                 for (int c = 0; c < NWm; ++c) {
                     const int w = 32 * c + lane;
                     uint32_t bal;
