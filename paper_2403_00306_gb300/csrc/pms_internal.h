@@ -51,6 +51,9 @@ struct InstDev {
     uint32_t raw_cap;      // capacity of the raw motif buffer (power of two)
     int triple_rows;       // rows after the first whose occurrences are tested in pairs with the first
                            //   row's (three-string feasibility below a node); 0: no such test
+    int words;             // offset (ints, even) in the chunk arena of this instance's table of node words: words, first
+                           //   word of the second and third group, 0, then (U, mask) pairs; queue chunks are then
+                           //   ranges of words. -1: ranges of nodes
     int sieve_mid;         // sieve form: middle letters of a block (pms_sieve.cu); its window words are
                            //   then stored in place of the planes. 0: the tree form
 };

@@ -66,7 +66,13 @@ struct __align__(16) WarpSmem {
 };
 
 struct __align__(16) CtaSmem {
-    uint32_t binom[kLMax + 1][kLMax + 1];
+    // binomials (node numbers to nodes), or the word filter's table: [D][t] =
+    // the 5-position sets L with popc(D ^ L) <= d - t
+    union {
+        uint32_t binom[kLMax + 1][kLMax + 1];
+        uint32_t near[32][32];
+    };
+    int table;               // which: 0 the binomials, d + 1 the filter's
     int row_len[kNMax];      // indexed by sequence
     int row_off[kNMax];      // indexed by sequence: first entry of its row (multiple of 4)
     int row_order[kNMax];    // sequences 1..n-1, smallest row first
@@ -81,7 +87,6 @@ struct __align__(16) CtaSmem {
     int next;                // next subset index of the chunk to claim
     int ctab;                // chunk table of the current item
     int stolen;              // the current item was joined after the queue ran out
-    int pad;
 };
 
 // Colex unranking of the rank-th k-subset of {0..l-1} (combinatorial number
@@ -859,6 +864,7 @@ __device__ __forceinline__ int filter_subsets(const WarpCtx &c, int N)
     return N;
 }
 
+// The walk of single nodes, for trees of too many nodes for a word table.
 // Lane-asynchronous node filter of a chunk: every lane holds one tree node P
 // and its position in the rows (row rank r, entry quad e4); each step a lane
 // tests the next 4 * kWalkQuads entries of its own row with the bound popc(D_w ^ P) <= d.
@@ -882,6 +888,7 @@ __device__ __forceinline__ void walk_init(const WarpCtx &c)
     uint32_t *st = c.ws->u.stash;
     st[c.lane] = 0u;
     st[32 + c.lane] = 0u;
+    c.ws->subs[c.lane] = 0u;
     if (c.lane < 4)
         st[64 + c.lane] = 0u;
     __syncwarp();
@@ -1052,6 +1059,304 @@ __device__ __forceinline__ int walk_run(const WarpCtx &c, const int *tab, int g0
     }
     __syncwarp();
     return qn;
+}
+
+// The node filter on words of up to 32 nodes (the default; see make_words in
+// pms_runtime.cu for the table). A node P is a set U of changed positions outside
+// a group of five and a set L inside it; an occurrence w meets the node's bound
+// popc(D_w ^ P) <= d iff popc(D_w in the group ^ L) <= d - t with t = popc((D_w ^
+// U) outside the group), so one look-up in a table by (D_w in the group, t) gives
+// all L at once. A lane holds a word; the warp reads a row's entries together
+// (broadcast loads; the table's 32 entries of one D_w lie in different banks),
+// ORs what they allow, and drops the word's nodes that no entry of the row
+// meets. With at most 16 (8) words the halves (quarters) of the warp share the
+// row. Once few nodes are left 4 or 8 lanes share a node's row.
+//
+// What bounds it: instruction issue, about 7 per entry and word of 14 nodes on
+// average. The walk of single nodes above takes about 77 instructions for 16
+// entries of one node per lane: (15,4), n = 20, m = 600, 1.14 M nodes, 84 M of
+// its comparisons, verification kernel 100 us; with words 78 us.
+//
+// Returns up to 32 nodes that passed, in queue (subs[64..]); the words' nodes
+// not returned yet are parked: stash[0..32) U, stash[32..64) nodes left, subs[0..32)
+// the group's first position.
+
+// Nodes of a warp's words at or below which a lane takes a node, and the fewest
+// words a warp claims. (15,4) and (17,5), us: 32 nodes and claims of half a
+// warp's share 92 and 720; 16 90 and 644; 8 88 and 636; 8 with claims of an
+// eighth of a share 83 and 609; claims of 4 words 97 and 650.
+constexpr unsigned int kLaneNodes = 8;
+constexpr int kMinWords = 8;
+
+// Appends each lane's nodes (bits of `alive` around U) to q[0..32) in lane order
+// until it is full; returns how many there are in all. `alive` keeps the rest.
+__device__ __forceinline__ int queue_nodes(uint32_t *q, uint32_t U, int sh, uint32_t &alive, int lane)
+{
+    const int cnt = __popc(alive);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o)
+            incl += y;
+    }
+    for (int at = incl - cnt; alive != 0u && at < 32; ++at) {
+        q[at] = U | ((uint32_t)(__ffs(alive) - 1) << sh);
+        alive &= alive - 1u;
+    }
+    __syncwarp();
+    return __shfl_sync(kFull, incl, 31);
+}
+
+template <bool kCount>
+__device__ __forceinline__ int word_run(const WarpCtx &c, const int *wtab, int g0, int g1, CtaSmem &cs, int *claim_ctr,
+                                        int claim_base, unsigned int *items_out, bool &finished)
+{
+    const InstDev &in = c.in;
+    const int d = in.d;
+    const int nrows = min(in.prune_rows, in.n - 1);
+    uint32_t *queue = c.ws->subs + 64;
+    volatile uint32_t *st = c.ws->u.stash;
+    volatile uint32_t *gs = c.ws->subs;
+    uint32_t U = st[c.lane], alive = st[32 + c.lane];
+    int sh = (int)gs[c.lane];
+    finished = false;
+    while (!__any_sync(kFull, alive != 0u)) {
+        // claims of an eighth of a warp's share, so that the item's warps end together
+        const int nw = (int)(blockDim.x >> 5);
+        const int want = min(32, max(kMinWords, (g1 - g0 + 8 * nw - 1) / (8 * nw)));
+        int start = 0;
+        if (c.lane == 0) {
+            start = claim_base + atomicAdd(claim_ctr, want);
+            if (items_out) {
+                claim_ctr[1] = max(0, g1 - (start + want));
+                if (start < g1 && start + want >= g1)
+                    atomicAdd(items_out, 1u);
+            }
+        }
+        start = __shfl_sync(kFull, start, 0);
+        const int N = min(want, g1 - start);
+        if (N <= 0) {
+            finished = true;
+            return 0;
+        }
+        // lane groups that share the rows: 1, 2 or 4 of 32, 16 or 8 words
+        const int lw = N <= 8 ? 3 : N <= 16 ? 4 : 5;   // log2 of the words' lanes
+        const int step = 32 >> lw, part = c.lane >> lw, mine = c.lane & ((1 << lw) - 1), idx = start + mine;
+        U = 0u;
+        alive = 0u;
+        sh = 0;
+        if (mine < N) {
+            const int2 w = *reinterpret_cast<const int2 *>(wtab + 4 + 2 * idx);
+            U = (uint32_t)w.x;
+            alive = (uint32_t)w.y;
+            sh = idx < wtab[1] ? 0 : idx < wtab[2] ? 5 : 10;
+        }
+        if (kCount && part == 0)
+            c.cnt[kCntSubsets] += __popc(alive);
+        if (kCount && part == 0)
+            c.cnt[kCntPruned] += __popc(alive);   // minus those that pass, below
+        const uint32_t out = ~(31u << sh);
+        int r = 0;
+        for (; r < nrows; ++r) {
+            const uint4 *D4 = reinterpret_cast<const uint4 *>(c.rows.D) + cs.rank_off4[r];
+            const int len4 = cs.rank_len4[r];
+            uint32_t acc = 0u;
+#pragma unroll 2
+            for (int e4 = part; e4 < len4; e4 += step) {
+                const uint4 v = D4[e4];
+                acc |= cs.near[(v.x >> sh) & 31u][__popc((v.x ^ U) & out)];
+                acc |= cs.near[(v.y >> sh) & 31u][__popc((v.y ^ U) & out)];
+                acc |= cs.near[(v.z >> sh) & 31u][__popc((v.z ^ U) & out)];
+                acc |= cs.near[(v.w >> sh) & 31u][__popc((v.w ^ U) & out)];
+                if (kCount && mine < N)
+                    c.cnt[kCntCmpReduce] += 4;
+            }
+            __syncwarp();
+            if (step >= 2)
+                acc |= __shfl_xor_sync(kFull, acc, 16);
+            if (step == 4)
+                acc |= __shfl_xor_sync(kFull, acc, 8);
+            alive &= acc;
+            if (__reduce_add_sync(kFull, part == 0 ? (unsigned int)__popc(alive) : 0u) <= kLaneNodes)
+                break;
+        }
+        if (part != 0)
+            alive = 0u;   // the same words as part 0's
+        if (r < nrows) {
+            // node by node: lanes j, j + 2^ln, ... share the rows of queue[j]
+            int n = queue_nodes(queue, U, sh, alive, c.lane);
+            uint32_t P = 0u;
+            int ln = 0;   // log2 of the nodes' lanes
+            for (++r; n > 0 && r < nrows; ++r) {
+                const int fit = n <= 4 ? 2 : n <= 8 ? 3 : n <= 16 ? 4 : 5;
+                const int who = c.lane & ((1 << fit) - 1);
+                if (fit != ln) {
+                    ln = fit;
+                    P = who < n ? queue[who] : 0u;
+                }
+                const uint4 *D4 = reinterpret_cast<const uint4 *>(c.rows.D) + cs.rank_off4[r];
+                const int len4 = cs.rank_len4[r];
+                int mn = 64;
+                for (int e4 = c.lane >> ln; e4 < len4; e4 += 32 >> ln) {
+                    const uint4 v = D4[e4];
+                    mn = min(mn, min(min(__popc(v.x ^ P), __popc(v.y ^ P)), min(__popc(v.z ^ P), __popc(v.w ^ P))));
+                    if (kCount && who < n)
+                        c.cnt[kCntCmpReduce] += 4;
+                }
+                uint32_t bal = __ballot_sync(kFull, mn <= d);
+                bal |= ln <= 4 ? bal >> 16 : 0u;
+                bal |= ln <= 3 ? bal >> 8 : 0u;
+                bal |= ln <= 2 ? bal >> 4 : 0u;
+                bal &= n == 32 ? kFull : (1u << n) - 1u;
+                if (__popc(bal) < n) {
+                    if (c.lane < n && ((bal >> c.lane) & 1u))
+                        queue[__popc(bal & c.lt)] = P;
+                    __syncwarp();
+                    n = __popc(bal);
+                    P = who < n ? queue[who] : 0u;
+                    __syncwarp();
+                }
+            }
+            if (kCount && c.lane == 0)
+                c.cnt[kCntPruned] -= n;
+            if (n > 0) {
+                st[32 + c.lane] = 0u;
+                __syncwarp();
+                return n;
+            }
+            continue;   // alive is 0 in every lane
+        }
+        if (kCount)
+            c.cnt[kCntPruned] -= __popc(alive);
+    }
+    const int n = queue_nodes(queue, U, sh, alive, c.lane);
+    st[c.lane] = U;
+    st[32 + c.lane] = alive;
+    gs[c.lane] = (uint32_t)sh;
+    __syncwarp();
+    return min(n, 32);
+}
+
+// The three-string test of triple_filter for up to 32 nodes at once, a lane per
+// node: the lane lists the occurrences u of row 0 that meet its node's bound and,
+// row after row, those w of the next rows (at most kPairList each), and keeps the
+// u that some w of every row leaves a string of the node with. A node without
+// u left is dropped; one with a longer list passes untested. Stops once few
+// nodes are left. Returns how many remain, in queue.
+//
+// triple_filter spends a warp on one node, about 280 instructions for the two rows
+// that most nodes need ((17,5), n = 20, m = 600: 956 k nodes reach it, 1.3 rows
+// each, 18 k leaves are left). Solves, us, words with triple_filter alone and with
+// this: (17,5) 907 and 641, (19,6) 9427 and 6155.
+constexpr int kPairList = 8;
+constexpr int kPairMin = 8;    // nodes for which the lane form is taken
+constexpr int kPairFew = 4;
+
+// Entries of row r that meet the bound of the lane's node: their numbers in the
+// row, 16 bits each, the last found first. Returns how many there are, more than
+// kPairList included.
+template <bool kCount>
+__device__ __forceinline__ int list_row(const WarpCtx &c, int r, uint32_t P, bool live, unsigned long long &lo,
+                                        unsigned long long &hi)
+{
+    const int d = c.in.d;
+    const int ri = c.cs->row_order[r];
+    const uint4 *D4 = reinterpret_cast<const uint4 *>(c.rows.D + c.cs->row_off[ri]);
+    const int len = c.cs->row_len[ri];
+    int k = 0;
+    lo = hi = 0;
+    for (int e = 0; e < len; e += 4) {
+        const uint4 v = D4[e >> 2];
+        const int p0 = __popc(v.x ^ P), p1 = __popc(v.y ^ P), p2 = __popc(v.z ^ P), p3 = __popc(v.w ^ P);
+        if (live && min(min(p0, p1), min(p2, p3)) <= d) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if ((u == 0 ? p0 : u == 1 ? p1 : u == 2 ? p2 : p3) <= d && e + u < len) {
+                    hi = (hi << 16) | (lo >> 48);
+                    lo = (lo << 16) | (unsigned long long)(e + u);
+                    ++k;
+                }
+        }
+        if (kCount && live)
+            c.cnt[kCntCmpReduce] += min(4, len - e);
+    }
+    return k;
+}
+
+template <bool kCount>
+__device__ __forceinline__ int pair_filter(const WarpCtx &c, uint32_t *queue, int qn)
+{
+    const InstDev &in = c.in;
+    const int d = in.d;
+    const int R = min(in.triple_rows + 1, in.n - 1);
+    const uint32_t P = c.lane < qn ? queue[c.lane] : 0u;
+    bool live = c.lane < qn;
+    unsigned long long ulo, uhi;
+    const int off0 = c.cs->row_off[c.cs->row_order[0]];
+    const int ku = list_row<kCount>(c, 0, P, live, ulo, uhi);
+    const bool tested = live && ku <= kPairList;   // a longer list: the node passes
+    uint32_t us = tested ? (1u << ku) - 1u : 1u;   // the u still possible
+    for (int r = 1; r < R; ++r) {
+        const uint32_t left = __ballot_sync(kFull, live);
+        if (__popc(left) <= kPairFew)
+            break;
+        unsigned long long wlo, whi;
+        const int offr = c.cs->row_off[c.cs->row_order[r]];
+        const int kw = list_row<kCount>(c, r, P, tested && live, wlo, whi);
+        if (tested && live && kw <= kPairList) {
+            uint32_t ok = 0u;
+            for (uint32_t todo = us; todo; todo &= todo - 1u) {
+                const int i = __ffs(todo) - 1;
+                const int eu = off0 + (int)((i < 4 ? ulo >> (16 * i) : uhi >> (16 * (i - 4))) & 0xffffu);
+                const uint2 u = c.rows.HL[eu];
+                const uint32_t Du = c.rows.D[eu];
+                const int room = 2 * d - __popc(Du ^ P);
+                bool any = false;
+                for (int j = 0; !any && j < kw; ++j) {
+                    const int ew = offr + (int)((j < 4 ? wlo >> (16 * j) : whi >> (16 * (j - 4))) & 0xffffu);
+                    const uint2 w = c.rows.HL[ew];
+                    const uint32_t Dw = c.rows.D[ew];
+                    any = __popc(Dw ^ P) + __popc(Du & Dw & ((u.x ^ w.x) | (u.y ^ w.y)) & P) <= room;
+                    if (kCount)
+                        c.cnt[kCntCmpVerify] += 1;
+                }
+                ok |= any ? 1u << i : 0u;
+            }
+            us = ok;
+            live = us != 0u;
+        }
+        __syncwarp();
+    }
+    const uint32_t bal = __ballot_sync(kFull, live);
+    __syncwarp();
+    if (live)
+        queue[__popc(bal & c.lt)] = P;
+    __syncwarp();
+    return __popc(bal);
+}
+
+// Loads the shared table that an item needs: the binomials, or the word
+// filter's for d changes.
+__device__ __forceinline__ void load_table(CtaSmem &cs, int want, int d)
+{
+    if (want == 0) {
+        for (int i = threadIdx.x; i < (kLMax + 1) * (kLMax + 1); i += blockDim.x)
+            (&cs.binom[0][0])[i] = (&c_binom[0][0])[i];
+        return;
+    }
+    for (int i = threadIdx.x; i < 32 * 32; i += blockDim.x) {
+        const int D = i >> 5, rad = d - (i & 31);
+        // the sets of at most rad positions, their index exclusive-ored with D
+        uint32_t m = rad < 0 ? 0u : rad == 0 ? 0x00000001u : rad == 1 ? 0x00010117u : rad == 2 ? 0x0117177fu
+                   : rad == 3 ? 0x177f7fffu : rad == 4 ? 0x7fffffffu : 0xffffffffu;
+        m = (D & 1) ? ((m & 0x55555555u) << 1) | ((m >> 1) & 0x55555555u) : m;
+        m = (D & 2) ? ((m & 0x33333333u) << 2) | ((m >> 2) & 0x33333333u) : m;
+        m = (D & 4) ? ((m & 0x0f0f0f0fu) << 4) | ((m >> 4) & 0x0f0f0f0fu) : m;
+        m = (D & 8) ? ((m & 0x00ff00ffu) << 8) | ((m >> 8) & 0x00ff00ffu) : m;
+        m = (D & 16) ? (m << 16) | (m >> 16) : m;
+        cs.near[D][i & 31] = m;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1257,7 +1562,7 @@ __device__ __forceinline__ ItemRef decode_item(const MainParams &p, long long g)
 
 // Fewest unclaimed nodes an item must have for a CTA whose queue ran out to
 // join it, and the rounds such a CTA looks for one before it stops.
-constexpr int kStealMinNodes = 64;
+constexpr int kStealMinNodes = 64;   // or words of nodes
 constexpr int kStealTries = 16;
 
 // Warp-cooperative choice of an item to join once the queue has run out: in
@@ -1517,9 +1822,8 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
         cs.cached_inst = -1;
         cs.cached_seed = -1;
         cs.feasible = 0;
+        cs.table = -1;
     }
-    for (int i = threadIdx.x; i < (kLMax + 1) * (kLMax + 1); i += blockDim.x)
-        (&cs.binom[0][0])[i] = (&c_binom[0][0])[i];
     // launched as a programmatic dependent of the previous kernel: nothing
     // above reads its output; wait here until it has completed and its
     // writes are visible (without the launch attribute this returns at once)
@@ -1574,6 +1878,10 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
             continue;
         }
         const bool rebuild = (I != cs.cached_inst) || (seed != cs.cached_seed);
+        const int table = in.words >= 0 ? in.d + 1 : 0;
+        const bool reload = cs.table != table;
+        if (reload)
+            load_table(cs, table, in.d);
         if (rebuild) {
             build_rows(p, in, seed, cs, smem_D, smem_HL, glob_D, glob_HL, warp, lane, kCount ? cnt : nullptr,
                        reinterpret_cast<uint32_t *>(smem_raw));
@@ -1582,7 +1890,9 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
                 cs.cached_seed = seed;
             }
         }
+        __syncthreads();   // every thread has compared cs.table
         if (threadIdx.x == 0) {
+            cs.table = table;
             cs.next = g0;
             // no node of an infeasible seed is searched: nothing for other CTAs to join
             if (p.item_claim && !cs.feasible)
@@ -1652,8 +1962,12 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
                 walk_init(c);
                 for (;;) {
                     bool fin;
-                    const int qn = walk_run<kCount>(c, tab, g0, g1, cs, ctr, base, exh, fin);
-                    const uint32_t *queue = wsm[warp].subs + 64;
+                    int qn = in.words >= 0
+                                       ? word_run<kCount>(c, p.ctab + in.words, g0, g1, cs, ctr, base, exh, fin)
+                                       : walk_run<kCount>(c, tab, g0, g1, cs, ctr, base, exh, fin);
+                    uint32_t *queue = wsm[warp].subs + 64;
+                    if (in.triple_rows > 0 && qn >= kPairMin && in.n > 2)
+                        qn = pair_filter<kCount>(c, queue, qn);
                     for (int i = 0; i < qn; ++i)
                         expand_subset<kCount>(c, queue[i]);
                     __syncwarp();

@@ -129,6 +129,89 @@ struct ChunkTable {
     int cps = 0;
 };
 
+// The tree nodes of (l, d) as words of up to 32 nodes, as the verification
+// kernel's word filter reads them: a word is a set U of changed positions
+// outside a group of up to five neighbouring positions, and a bit per set of
+// changed positions inside it (the mask says which of those are nodes). A node
+// belongs to the group that holds most of its changes, the first of equals, so
+// that words are full: (15,4) 1941 nodes in 138 words of the three groups, 386
+// with one group; (19,6) 43796 in 2948 (6476).
+struct WordTable {
+    std::vector<int> tab;        // words, first word of groups 1 and 2, 0; then (U, mask) pairs, by group
+    std::vector<double> cost;    // per word, in candidate units
+    int words = 0;
+};
+constexpr int kMaxWords = 1 << 14;
+constexpr uint64_t kMaxWordNodes = 1u << 18;
+
+WordTable make_words(int l, int d)
+{
+    WordTable wt;
+    uint64_t nodes = 0;
+    for (int k = 0; k <= d; ++k)
+        nodes += binom(l, k);
+    if (nodes > kMaxWordNodes)
+        return wt;
+    const int groups = std::max(1, std::min(3, l / 5));
+    std::map<uint32_t, std::pair<uint32_t, double>> words[3];
+    for (int k = 0; k <= d; ++k) {
+        const double c = std::pow(3.0, k) + kNodeUnits;
+        uint64_t P = (1ull << k) - 1;
+        while (P < (1ull << l)) {
+            int best = 0, most = -1;
+            for (int g = 0; g < groups; ++g) {
+                const int in = __builtin_popcount((uint32_t)(P >> (5 * g)) & 31u);
+                if (in > most) {
+                    most = in;
+                    best = g;
+                }
+            }
+            auto &w = words[best][(uint32_t)P & ~(31u << (5 * best))];
+            w.first |= 1u << ((uint32_t)(P >> (5 * best)) & 31u);
+            w.second += c;
+            if (k == 0)
+                break;
+            const uint64_t low = P & (0 - P), up = P + low;   // the next integer with k bits set
+            P = up | (((P ^ up) >> 2) / low);
+        }
+    }
+    const int n0 = (int)words[0].size(), n1 = (int)words[1].size(), n2 = (int)words[2].size();
+    if (n0 + n1 + n2 > kMaxWords)
+        return wt;
+    wt.words = n0 + n1 + n2;
+    wt.tab = {wt.words, n0, n0 + n1, 0};
+    for (const auto &group : words)
+        for (const auto &w : group) {
+            wt.tab.push_back((int)w.first);
+            wt.tab.push_back((int)w.second.first);
+            wt.cost.push_back(w.second.second);
+        }
+    return wt;
+}
+
+// The queue chunks of one seed as ranges of words of equal cost (cf. make_chunks).
+ChunkTable make_word_chunks(const WordTable &wt, int d, int work)
+{
+    ChunkTable ct;
+    double total = 0;
+    for (double c : wt.cost)
+        total += c;
+    const int k = std::max(1, std::min(wt.words, (int)std::lround(total / std::max(1, work))));
+    ct.tab.assign(d + 2, 0);
+    double acc = 0;
+    int start = 0;
+    for (int w = 0; w < wt.words; ++w) {
+        acc += wt.cost[w];
+        if (w + 1 == wt.words || (ct.cps + 1 < k && acc >= total * (ct.cps + 1) / k)) {
+            ct.tab.push_back(start);
+            ct.tab.push_back(w + 1);
+            start = w + 1;
+            ++ct.cps;
+        }
+    }
+    return ct;
+}
+
 ChunkTable make_chunks(int l, int d, int work)
 {
     ChunkTable ct;
@@ -172,13 +255,15 @@ ChunkTable make_chunks(int l, int d, int work)
 }
 
 
-// The chunks of one seed cut into k ranges of equal cost (as make_chunks).
-ChunkTable make_chunks_k(int l, int d, int k)
+// The chunks of one seed cut into k ranges of equal cost (as make_chunks; of
+// words where wt has any).
+ChunkTable make_chunks_k(int l, int d, int k, const WordTable &wt)
 {
     double total = 0;
     for (int i = 0; i <= d; ++i)
         total += (double)binom(l, i) * (std::pow(3.0, i) + kNodeUnits);
-    return make_chunks(l, d, (int)std::max(1.0, std::floor(total / k)));
+    const int work = (int)std::max(1.0, std::floor(total / k));
+    return wt.words > 0 ? make_word_chunks(wt, d, work) : make_chunks(l, d, work);
 }
 
 }  // namespace
@@ -211,7 +296,8 @@ struct pms_ctx {
     int occ_small[2] = {0, 0};  // same for its small-rows form
     int occ_pair[2] = {0, 0};  // same for the pair-form kernel
     pms_stats stats{};
-    std::map<std::tuple<int, int, int>, ChunkTable> ctab_cache;
+    std::map<std::tuple<int, int, int>, ChunkTable> ctab_cache, wtab_cache;
+    std::map<std::pair<int, int>, WordTable> word_cache;
 
     struct DBuf {
         void *p = nullptr;
@@ -477,6 +563,27 @@ struct pms_ctx {
         return t && t->prune_rows > 0 ? std::min(t->prune_rows, n - 1) : n - 1;
     }
 
+    // The word table of (l, d), without words where the node walk is taken:
+    // by other node filters, quorums and trees of more than kMaxWordNodes nodes.
+    const WordTable &words(int l, int d, bool walk)
+    {
+        static const WordTable none;
+        if (!walk)
+            return none;
+        const auto key = std::make_pair(l, d);
+        auto it = word_cache.find(key);
+        if (it == word_cache.end())
+            it = word_cache.emplace(key, make_words(l, d)).first;
+        return it->second;
+    }
+    const ChunkTable &word_chunks(int l, int d, int work)
+    {
+        const auto key = std::make_tuple(l, d, work);
+        auto it = wtab_cache.find(key);
+        if (it == wtab_cache.end())
+            it = wtab_cache.emplace(key, make_word_chunks(words(l, d, true), d, work)).first;
+        return it->second;
+    }
     const ChunkTable &chunks(int l, int d, int work = 0)
     {
         if (work <= 0)
@@ -710,13 +817,15 @@ static double expected_seed_rows(int n, int m, int l, int d)
 // The form with the smallest estimated time. The estimates were fitted to
 // device times on one GB300 (n = 10 and 20, m = 200, 600, 1200, l = 8..19,
 // d = 1..6); they only choose, so what matters is where they cross.
-//   tree: W |B(x, d)| candidates at 390 E^3 / (E + 0.02) ps each, E =
+//   tree: W |B(x, d)| candidates at 4000 E^3 / (1 + E / 0.15) ps each, E =
 //     expected_near: the more windows lie near a candidate, the fewer nodes
-//     fail. A quorum adds seeds and keeps nodes with misses. A single instance
-//     takes 38 us + 25 ns W for the launches, the masks and the slowest seeds.
-//     Measured (estimated), us: (15,4) m = 600 118 (154), m = 1000 562 (515),
-//     m = 1200 1050 (1003); (14,4) m = 600 761 (800); (13,3) m = 1200 141 (151);
-//     (17,5) m = 600 1050 (1030), m = 900 4300 (4060), m = 1200 11080 (9500).
+//     fail. A quorum, filtered node by node, 390 E^3 / (E + 0.02) ps, more for
+//     the nodes kept with misses. 32 us + 25 ns W for the launches, the masks and
+//     the slowest seeds of a single instance.
+//     Measured (estimated), us: (15,4) m = 600 86 (109), m = 800 200 (233),
+//     m = 1000 356 (465), m = 1200 717 (855); (14,4) m = 400 231 (217); (13,3)
+//     m = 1200 119 (136); (17,5) m = 600 586 (610), m = 1000 4062 (3950),
+//     m = 1200 7959 (7500); (19,6) m = 600 6109 (4700), m = 1200 106700 (62800).
 //   sieve: 4^A blocks, W windows and S sequences at a + b words ps, words = the
 //     words of a block that a window marks on average; S = n, or less where a
 //     block's strings run out sooner. With few blocks, one block's latency counts.
@@ -734,8 +843,9 @@ static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int
     // 4^l strings, and writing it is what takes the time
     if (n < 2 || (l == 8 && E > 1.0))
         return SieveForm{};
-    double best = seeds * (double)ball_size(l, d) * 390e-6 * E * E * E / (E + 0.02) * (1.0 + 3.0 * (n - q)) +
-                  (single ? 38.0 + 0.025 * W : 0.0);
+    const double per_candidate =
+        q == n ? 4000e-6 * E * E * E / (1.0 + E / 0.15) : 390e-6 * E * E * E / (E + 0.02) * (1.0 + 3.0 * (n - q));
+    double best = seeds * (double)ball_size(l, d) * per_candidate + (single ? 32.0 + 0.025 * W : 0.0);
     double motifs = 0;
     for (int k = q; k <= n; ++k)
         motifs += choose(n, k) * std::pow(p, k) * std::pow(1.0 - p, n - k);
@@ -779,7 +889,11 @@ static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int
         const double marks = rounds * windows * S * (o.a + o.b * words) * 1e-6;
         // every motif is looked up in the seed sequences, by as many warps as have blocks
         const double lookups = motifs * seeds * 14e-6 * (o.share != 1 ? 1.0 : std::max(1.0, slots / blocks));
-        const double latency = !single ? 0.0 : !wide ? 35.0 : o.share == 8 ? 12.0 + 0.085 * W : 14.0 + 0.04 * W;
+        const double latency = !single          ? 0.0
+                               : !wide          ? 35.0
+                               : o.share == 8   ? 12.0 + 0.085 * W
+                               : l == 11        ? 10.0 + 0.052 * W
+                                                : 14.0 + 0.03 * W;
         const double us = (wide && o.share == 8 ? std::max(latency, 25.0 + marks) : latency + marks) + lookups;
         if (us < best) {
             best = us;
@@ -846,6 +960,7 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
             P.small_rows = false;
     }
     long long work = 0;
+    std::map<const int *, int> tables;   // offsets of the chunk and word tables (cached ones) in the plan
     const int adaptive = kDefaultChunkWork;   // untuned classes: about 2^20 candidate units per queue item
     bool quorum_used = false;
     for (size_t k = 0; k < specs.size(); ++k) {
@@ -863,14 +978,26 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
         const bool tree = in.sieve_mid == 0;
         const long long seeds = (long long)in.nseed * in.W;
         const int cw = h->chunk_work_for(s.n, s.m, s.l, s.d);
-        const ChunkTable &ct = h->chunks(s.l, s.d, cw > 0 ? cw : adaptive);
-        in.cps = ct.cps;
         in.grab = h->grab_for(s.n, s.m, s.l, s.d);
+        const WordTable &wt = h->words(s.l, s.d, tree && in.grab == 1 && in.q == in.n);
+        const ChunkTable &ct = wt.words > 0 ? h->word_chunks(s.l, s.d, cw > 0 ? cw : adaptive)
+                                            : h->chunks(s.l, s.d, cw > 0 ? cw : adaptive);
+        in.cps = ct.cps;
         in.prune_rows = h->prune_rows_for(s.n, s.m, s.l, s.d);
         in.partial_rows = h->partial_rows_for(s.n, s.m, s.l, s.d);
         in.triple_rows = h->triple_rows_for(s.n, s.m, s.l, s.d);
-        in.ctab = (int)P.ctab.size();
-        P.ctab.insert(P.ctab.end(), ct.tab.begin(), ct.tab.end());
+        // one copy of a table for all the plan's instances that read it
+        const auto table = [&](const std::vector<int> &tab) {
+            const auto found = tables.find(tab.data());
+            if (found != tables.end())
+                return found->second;
+            P.ctab.resize(round_up(P.ctab.size(), 2));   // the kernel reads pairs
+            const int at = (int)P.ctab.size();
+            P.ctab.insert(P.ctab.end(), tab.begin(), tab.end());
+            return tables[tab.data()] = at;
+        };
+        in.ctab = table(ct.tab);
+        in.words = wt.words > 0 ? table(wt.tab) : -1;
         in.seq_off = (long long)P.seq_bytes;
         P.seq_bytes += round_up((size_t)s.n * s.m, 16);
         in.plane_off = (long long)P.planes;
@@ -908,7 +1035,7 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
         const long long r = seeds % B;
         const int kk = r > 0 ? (int)std::min<long long>(B / r, 16) : 0;
         if (specs.size() == 1 && in.cps == 1 && seeds > B && kk >= 2) {
-            const ChunkTable ct2 = make_chunks_k(s.l, s.d, kk);
+            const ChunkTable ct2 = make_chunks_k(s.l, s.d, kk, wt);
             const int whole = (int)(seeds - r);
             P.seg.push_back(Segment{work, (int)k, 0, whole, 0, 0, 0});
             work += whole;
@@ -1903,8 +2030,15 @@ static bool served_admit(Served *S, Request *r)
         return false;
     std::lock_guard<std::recursive_mutex> hg(h->mu);
     const int cw = h->chunk_work_for(r->n, r->m, r->l, r->d);
-    const ChunkTable &ct = h->chunks(r->l, r->d, cw > 0 ? cw : kDefaultChunkWork);
-    if ((int)ct.tab.size() > Served::kCtabMax) {
+    const int grab = h->grab_for(r->n, r->m, r->l, r->d);
+    const WordTable *wt = &h->words(r->l, r->d, grab == 1);
+    if ((int)wt->tab.size() > Served::kCtabMax / 2)
+        wt = &h->words(r->l, r->d, false);
+    const ChunkTable &ct = wt->words > 0 ? h->word_chunks(r->l, r->d, cw > 0 ? cw : kDefaultChunkWork)
+                                         : h->chunks(r->l, r->d, cw > 0 ? cw : kDefaultChunkWork);
+    const size_t ct_ints = round_up(ct.tab.size(), 2);   // the word table's pairs follow
+    const size_t ctab_ints = ct_ints + wt->tab.size();
+    if ((int)ctab_ints > Served::kCtabMax) {
         r->status = PMS_EINVAL;
         return true;
     }
@@ -1919,7 +2053,7 @@ static bool served_admit(Served *S, Request *r)
     if (r->form.planes != 0)
         r->form = SieveForm{};   // the served form solves q = n
     const bool tree = r->form.mid == 0;
-    ReqLayout L(r->n, r->m, r->W, r->raw_cap, ct.tab.size(), tree);
+    ReqLayout L(r->n, r->m, r->W, r->raw_cap, ctab_ints, tree);
     if (L.total > S->pool_bytes) {
         r->status = PMS_ENOMEM;   // can never fit
         return true;
@@ -1952,7 +2086,7 @@ static bool served_admit(Served *S, Request *r)
     in.W = r->W;
     in.NW = (r->W + 31) / 32;
     in.cps = ct.cps;
-    in.grab = h->grab_for(r->n, r->m, r->l, r->d);
+    in.grab = grab;
     in.prune_rows = h->prune_rows_for(r->n, r->m, r->l, r->d);
     in.partial_rows = h->partial_rows_for(r->n, r->m, r->l, r->d);
     in.triple_rows = h->triple_rows_for(r->n, r->m, r->l, r->d);
@@ -1965,12 +2099,14 @@ static bool served_admit(Served *S, Request *r)
     in.compat_off = (long long)((off + L.compat) / 4);
     in.rlen_off = (long long)((off + L.rowlen) / 4);
     in.ctab = (int)((off + L.ctab) / sizeof(int));
+    in.words = wt->words > 0 ? in.ctab + (int)ct_ints : -1;
     in.raw_cap = r->raw_cap;
     int *hc = S->h_ctab + (size_t)r->slot * Served::kCtabMax;
     std::memcpy(hc, ct.tab.data(), ct.tab.size() * sizeof(int));
+    std::memcpy(hc + ct_ints, wt->tab.data(), wt->tab.size() * sizeof(int));
     cudaStream_t st = S->st;
     cudaMemcpyAsync(S->pool + off + L.seqs, r->seqs.data(), r->seqs.size(), cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(S->pool + off + L.ctab, hc, ct.tab.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(S->pool + off + L.ctab, hc, ctab_ints * sizeof(int), cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(S->d_inst + r->slot, &in, sizeof(InstDev), cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(srv_rawcnt(S) + r->slot, 0, 4, st);
     cudaMemsetAsync(srv_flags(S) + r->slot, 0, 4, st);
@@ -3166,7 +3302,8 @@ extern "C" int pms_solve_device_noalloc(const uint8_t *d_seqs, int n, int m, int
     in.W = m - l + 1;
     in.NW = (in.W + 31) / 32;
     in.cps = cps;
-    in.grab = kDefaultGrab;   // the lane-asynchronous node walk, as in the other paths
+    in.grab = kDefaultGrab;   // the lane-asynchronous node walk
+    in.words = -1;
     in.prune_rows = default_prune_rows(n, d);
     {
         const int pr = default_partial_rows(n, m, l, d);

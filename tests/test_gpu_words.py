@@ -1,0 +1,41 @@
+"""The verification kernel's filter on words of nodes, and the three-string test of many nodes at
+once, against the oracle: groups of fewer than five positions, one to three groups, full words and
+words of one node, rows of one entry, in shared and in global memory, a warp's words in 8, 16 and 32
+lanes, n = 1 and 2."""
+import numpy as np
+import pytest
+
+import planted_inputs as pi
+import paper_2403_00306_gb300 as pms
+
+pytestmark = pytest.mark.gpu
+
+# (n, m, l, d)
+CASES = [(1, 12, 4, 1), (2, 30, 3, 2), (3, 25, 5, 2), (4, 40, 7, 3), (5, 33, 9, 0), (6, 60, 10, 3), (8, 60, 14, 4),
+         (20, 20, 15, 4), (12, 47, 15, 5), (64, 24, 16, 4), (6, 30, 17, 5), (10, 30, 20, 5), (5, 64, 32, 3),
+         (2, 19, 19, 6)]
+
+
+@pytest.mark.parametrize("case", CASES, ids=str)
+def test_words_match_oracle(oracle_, case):
+    n, m, l, d = case
+    for seqs in (pi.planted_instance(n, m, l, d, 3).seqs, pi.random_sequences(n, m, 31)):
+        want = oracle_.solve_packed(seqs, l, d)
+        for opts in ({}, {"smem_rows": 8}, {"triple_rows": 6}, {"triple_rows": -1}, {"chunk_work": 4096}):
+            with pms.Context(0) as c:
+                c.set_options(grab=1, **opts)
+                assert np.array_equal(c.solve(seqs, l, d), want), opts
+
+
+@pytest.mark.parametrize("case", [(20, 900, 15, 4), (20, 600, 17, 5), (12, 260, 19, 6), (20, 300, 13, 4)], ids=str)
+def test_words_and_batches_agree(case):
+    """Whole motif sets of larger instances: words of nodes against breadth-first batches of nodes."""
+    n, m, l, d = case
+    seqs = pi.planted_instance(n, m, l, d, 9).seqs
+    got = []
+    for opts in ({"grab": 1}, {"grab": 128}, {"grab": 1, "triple_rows": 19}):
+        with pms.Context(0) as c:
+            c.set_options(**opts)
+            got.append(c.solve(seqs, l, d))
+    assert len(got[0]) > 0
+    assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
