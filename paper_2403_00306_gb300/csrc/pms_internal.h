@@ -51,6 +51,8 @@ struct InstDev {
     uint32_t raw_cap;      // capacity of the raw motif buffer (power of two)
     int triple_rows;       // rows after the first whose occurrences are tested in pairs with the first
                            //   row's (three-string feasibility below a node); 0: no such test
+    int buckets;           // sieve form: offset (words) of this instance's buckets, whose keys are sorted before the
+                           //   sort kernel; -1: the sort kernel sorts them
     int words;             // offset (ints, even) in the chunk arena of this instance's table of node words: words, first
                            //   word of the second and third group, 0, then (U, mask) pairs; queue chunks are then
                            //   ranges of words. -1: ranges of nodes
@@ -151,13 +153,30 @@ size_t main_smem_bytes(bool small_rows = false);
 cudaError_t launch_sort_unique(const InstDev *inst, const int *inst_list, int nlist, uint64_t *raw, uint64_t *tmp,
                                const uint32_t *raw_count, const uint32_t *flags, StatusDev *status,
                                uint64_t *dense, uint32_t dense_cap, uint32_t *dense_total,
-                               cudaStream_t st);
+                               const uint32_t *key_count, cudaStream_t st);
+// Sorts the keys of the listed instances (in sieve form, with buckets) in raw:
+// scattered by bucket to tmp, then each bucket's keys by rank.
+cudaError_t launch_bucket_sort(const InstDev *inst, const int *list, int nlist, uint64_t *raw, uint64_t *tmp,
+                               const uint32_t *key_count, uint32_t *buckets, cudaStream_t st);
 cudaError_t init_tables();
 // Host handles of the pack and sort/unique kernels (to find their nodes in a captured graph).
 const void *pack_kernel_fn();
 const void *sort_unique_kernel_fn();
 cudaError_t launch_probe(int kind, int iters, int blocks, unsigned long long *cycles, unsigned long long *sink,
                          cudaStream_t st);
+
+// Buckets of the keys of a large answer: the first six letters (all, where a
+// motif has fewer), in key order.
+constexpr int kBucketBits = 12;
+constexpr int kBuckets = 1 << kBucketBits;
+// Words of one instance: keys per bucket and, zeroed with them, keys placed per
+// bucket; then the first key of every bucket.
+constexpr int kBucketWords = 3 * kBuckets;
+__host__ __device__ inline uint32_t bucket_of(uint64_t key, int l)
+{
+    const int low = 2 * l - kBucketBits;
+    return (uint32_t)(low > 0 ? key >> low : key);
+}
 
 // Launch configuration of a programmatic dependent launch: the kernel may be
 // scheduled before the previous kernel in the stream has completed, and
@@ -195,8 +214,9 @@ struct SieveParams {
     unsigned long long *head;     // queue head (zeroed before the launch)
     const uint2 *planes;          // instance plane_off: its window words
     uint64_t *raw;
-    uint32_t *raw_count;
-    uint32_t *flags;
+    uint32_t *raw_count;          // per instance: motifs, once per seed window near them
+    uint32_t *key_count;          // per instance: keys in raw (every motif once)
+    uint32_t *buckets;            // instance buckets: keys per bucket (see bucket_of)
 };
 
 cudaError_t sieve_init_tables();

@@ -2845,7 +2845,7 @@ __global__ void __launch_bounds__(kSortThreads)
     sort_unique_kernel(const InstDev *__restrict__ inst, const int *__restrict__ inst_list, uint64_t *raw,
                        uint64_t *tmp, const uint32_t *__restrict__ raw_count, const uint32_t *__restrict__ flags,
                        StatusDev *__restrict__ status, uint64_t *__restrict__ dense, uint32_t dense_cap,
-                       uint32_t *dense_total)
+                       uint32_t *dense_total, const uint32_t *__restrict__ key_count)
 {
     extern __shared__ __align__(16) uint64_t sk[];
     __shared__ uint32_t warp_tot[32];
@@ -2854,8 +2854,35 @@ __global__ void __launch_bounds__(kSortThreads)
     const int I = inst_list ? inst_list[blockIdx.x] : (int)blockIdx.x;
     const InstDev in = inst[I];
     const uint32_t rc = raw_count[I];
-    const uint32_t n = rc < in.raw_cap ? rc : in.raw_cap;
+    const uint32_t nk = in.sieve_mid ? key_count[I] : rc;
+    const uint32_t n = nk < in.raw_cap ? nk : in.raw_cap;
     uint64_t *a = raw + in.raw_off;
+    if (in.sieve_mid && in.buckets >= 0) {
+        // sorted and without duplicates already
+        if (threadIdx.x == 0) {
+            const uint32_t base = atomicAdd(dense_total, n);
+            s_base = base;
+            uint32_t f = flags[I];
+            if (rc > in.raw_cap || base + n > dense_cap)
+                f |= kFlagOverflow;
+            status[I] = StatusDev{rc, n, f, base};
+        }
+        __syncthreads();
+        const uint32_t room = s_base < dense_cap ? dense_cap - s_base : 0u;
+        uint64_t *to = dense + s_base;
+        const uint32_t m = min(n, room);
+        for (uint32_t i = threadIdx.x; i < m; i += 4 * blockDim.x) {
+            uint64_t v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                v[u] = i + u * blockDim.x < m ? a[i + u * blockDim.x] : 0ull;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i + u * blockDim.x < m)
+                    to[i + u * blockDim.x] = v[u];
+        }
+        return;
+    }
     uint32_t P2 = 1;
     while (P2 < n)
         P2 <<= 1;
@@ -2910,6 +2937,87 @@ __global__ void __launch_bounds__(kSortThreads)
         if (threadIdx.x == 0)
             s_run += s_total;
         __syncthreads();
+    }
+}
+
+// Large answers of the sieve form (every motif once, counted by bucket as the
+// sieve emits it), sorted by the whole grid: one CTA alone took 85 us for 5900
+// keys in the one-CTA kernel above and 8.1 ms for the 256 instances of the
+// batch (up to 600 k keys each).
+// Scatter: gridDim.x CTAs per instance; each scans the instance's counts for
+// the buckets' first places (CTA 0 stores them) and places its share of the keys.
+constexpr int kBucketThreads = 256;
+__global__ void __launch_bounds__(kBucketThreads)
+    bucket_scatter_kernel(const InstDev *__restrict__ inst, const int *__restrict__ list, const uint64_t *__restrict__ raw,
+                          uint64_t *__restrict__ tmp, const uint32_t *__restrict__ key_count, uint32_t *buckets)
+{
+    __shared__ uint32_t first[kBuckets];
+    __shared__ uint32_t warp_tot[32], total;
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int I = list[blockIdx.y];
+    const InstDev in = inst[I];
+    const uint32_t n = min(key_count[I], in.raw_cap);
+    uint32_t *count = buckets + in.buckets, *placed = count + kBuckets, *start = placed + kBuckets;
+    constexpr int kPer = kBuckets / kBucketThreads;
+    uint32_t v[kPer], sum = 0;
+#pragma unroll
+    for (int u = 0; u < kPer / 4; ++u) {
+        const uint4 q = reinterpret_cast<const uint4 *>(count)[threadIdx.x * (kPer / 4) + u];
+        v[4 * u] = q.x;
+        v[4 * u + 1] = q.y;
+        v[4 * u + 2] = q.z;
+        v[4 * u + 3] = q.w;
+        sum += q.x + q.y + q.z + q.w;
+    }
+    uint32_t at = block_exclusive_scan(sum, warp_tot, &total);
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        first[threadIdx.x * kPer + u] = at;
+        at += v[u];
+    }
+    __syncthreads();
+    if (blockIdx.x == 0)
+        for (int b = threadIdx.x; b < kBuckets; b += kBucketThreads)
+            start[b] = first[b];
+    for (uint32_t i = blockIdx.x * kBucketThreads + threadIdx.x; i < n; i += gridDim.x * kBucketThreads) {
+        const uint64_t key = raw[in.raw_off + i];
+        const uint32_t b = bucket_of(key, in.l);
+        tmp[in.raw_off + first[b] + atomicAdd(&placed[b], 1u)] = key;
+    }
+}
+
+// Rank: a warp per bucket; a key's place is the number of smaller ones (all
+// keys differ). Chance answers hold a few dozen keys a bucket.
+__global__ void __launch_bounds__(kBucketThreads)
+    bucket_rank_kernel(const InstDev *__restrict__ inst, const int *__restrict__ list, uint64_t *__restrict__ raw,
+                       const uint64_t *__restrict__ tmp, const uint32_t *__restrict__ buckets)
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const InstDev in = inst[list[blockIdx.y]];
+    const uint32_t *count = buckets + in.buckets, *start = count + 2 * kBuckets;
+    const int lane = threadIdx.x & 31;
+    for (int b = blockIdx.x * (kBucketThreads / 32) + (threadIdx.x >> 5); b < kBuckets;
+         b += gridDim.x * (kBucketThreads / 32)) {
+        const uint32_t n = count[b];
+        if (n == 0)
+            continue;
+        const uint64_t *from = tmp + in.raw_off + start[b];
+        uint64_t *to = raw + in.raw_off + start[b];
+        for (uint32_t i0 = 0; i0 < n; i0 += 32) {
+            const uint32_t i = i0 + lane;
+            const uint64_t key = i < n ? from[i] : ~0ull;
+            uint32_t rank = 0;
+            for (uint32_t j0 = 0; j0 < n; j0 += 32) {
+                const uint64_t other = j0 + lane < n ? from[j0 + lane] : ~0ull;
+                const int m = (int)min(32u, n - j0);
+                for (int j = 0; j < m; ++j)
+                    rank += __shfl_sync(kFull, other, j) < key ? 1u : 0u;
+            }
+            if (i < n)
+                to[rank] = key;
+        }
     }
 }
 
@@ -3114,7 +3222,8 @@ cudaError_t launch_pack(const InstDev *inst, int ninst, const long long *win_pre
 
 cudaError_t launch_sort_unique(const InstDev *inst, const int *inst_list, int nlist, uint64_t *raw, uint64_t *tmp,
                                const uint32_t *raw_count, const uint32_t *flags, StatusDev *status,
-                               uint64_t *dense, uint32_t dense_cap, uint32_t *dense_total, cudaStream_t st)
+                               uint64_t *dense, uint32_t dense_cap, uint32_t *dense_total, const uint32_t *key_count,
+                               cudaStream_t st)
 {
     const size_t smem = std::max<size_t>(kSortSmemKeys * sizeof(uint64_t), (2 * 32 * 256 + 256) * sizeof(uint32_t));
     static thread_local int attr_set_dev = -1;
@@ -3129,7 +3238,24 @@ cudaError_t launch_sort_unique(const InstDev *inst, const int *inst_list, int nl
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = dependent_launch(attr, nlist, kSortThreads, smem, st);
     return cudaLaunchKernelEx(&cfg, sort_unique_kernel, inst, inst_list, raw, tmp, raw_count, flags, status, dense,
-                              dense_cap, dense_total);
+                              dense_cap, dense_total, key_count);
+}
+
+cudaError_t launch_bucket_sort(const InstDev *inst, const int *list, int nlist, uint64_t *raw, uint64_t *tmp,
+                               const uint32_t *key_count, uint32_t *buckets, cudaStream_t st)
+{
+    // CTAs per instance: enough for one answer alone, few each for many
+    const int scatter = nlist >= 64 ? 4 : 32, rank = nlist >= 64 ? 32 : 512;
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = dependent_launch(attr, scatter, kBucketThreads, 0, st);
+    cfg.gridDim.y = (unsigned)nlist;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, bucket_scatter_kernel, inst, list, (const uint64_t *)raw, tmp, key_count,
+                                       buckets);
+    if (e != cudaSuccess)
+        return e;
+    cfg.gridDim.x = (unsigned)rank;
+    return cudaLaunchKernelEx(&cfg, bucket_rank_kernel, inst, list, raw, (const uint64_t *)tmp,
+                              (const uint32_t *)buckets);
 }
 
 cudaError_t launch_probe(int kind, int iters, int blocks, unsigned long long *cycles, unsigned long long *sink,

@@ -276,7 +276,8 @@ struct Served;
 // counter planes and warps per block, see launch_sieve) or the tree (mid = 0).
 struct SieveForm {
     int mid = 0, planes = 0, share = 1;
-    double us = 0;   // estimated time
+    double us = 0;       // estimated time
+    double motifs = 0;   // expected motifs of random sequences
 };
 
 struct pms_ctx {
@@ -361,6 +362,7 @@ struct pms_ctx {
             void *dense;
             uint32_t dense_cap;
             void *dense_total;
+            const void *key_count;
         } sv{};
         struct {
             const void *inst;
@@ -373,7 +375,7 @@ struct pms_ctx {
         bool input_rows = false;   // the node `pack` is that kernel (input pointer: argument 1)
         void *pack_args[7] = {};
         void *rows_args[6] = {};
-        void *sort_args[10] = {};
+        void *sort_args[11] = {};
         DBuf meta;             // this plan's descriptors (the kernels of the graph read them)
         uint64_t gen = 0;      // buffer generation the graph was captured with
         uint64_t candidates = 0;
@@ -678,11 +680,12 @@ struct Plan {
     };
     std::vector<SieveSeg> sieve_seg;
     std::vector<SieveLaunch> sieve;
+    std::vector<int> bucketed;           // instances whose answers are sorted by buckets
 };
 
 // Byte layout of the descriptor block (device d_meta, pinned h_meta).
 struct MetaLayout {
-    size_t inst, seg, win, rowp, seedp, segp, ctab, sieve, total;
+    size_t inst, seg, win, rowp, seedp, segp, ctab, sieve, bucketed, total;
     MetaLayout(const Plan &p)
     {
         size_t o = 0;
@@ -702,17 +705,20 @@ struct MetaLayout {
         o = round_up(o + p.ctab.size() * sizeof(int), 16);
         sieve = o;
         o = round_up(o + p.sieve_seg.size() * sizeof(SieveSeg), 16);
+        bucketed = o;
+        o = round_up(o + p.bucketed.size() * sizeof(int), 16);
         total = o;
     }
 };
 
 // Counters block (d_ctr): queue heads, work counters, dense_total, then per instance
-// raw_count and flags, then (items > 0) the steal cursor and the nodes claimed
-// of every queue item, for the verification kernel's work sharing.
+// raw_count, key_count and flags, then (items > 0) the steal cursor and the nodes claimed
+// of every queue item, for the verification kernel's work sharing, then the
+// buckets of large answers. All of it is cleared before a launch.
 constexpr int kMaxSieveLaunches = 7;   // q = n with 3 to 6 middle letters, the quorum form with 3 to 5
 struct CtrLayout {
-    size_t head, head_pair, head_sieve, work, dense_total, raw_count, flags, steal, claim, total;
-    CtrLayout(size_t k, size_t items = 0)
+    size_t head, head_pair, head_sieve, work, dense_total, raw_count, key_count, flags, steal, claim, buckets, total;
+    CtrLayout(size_t k, size_t items = 0, size_t bucketed = 0)
     {
         head = 0;
         head_pair = 8;
@@ -720,10 +726,12 @@ struct CtrLayout {
         work = head_sieve + 8 * kMaxSieveLaunches;
         dense_total = work + kCntNum * 8;
         raw_count = round_up(dense_total + 4, 16);
-        flags = round_up(raw_count + 4 * k, 16);
+        key_count = round_up(raw_count + 4 * k, 16);
+        flags = round_up(key_count + 4 * k, 16);
         steal = round_up(flags + 4 * k, 16);
         claim = steal + 16;
-        total = round_up(claim + 8 * items, 256);
+        buckets = round_up(claim + 8 * items, 256);
+        total = buckets + bucketed * kBucketWords * 4;
     }
 };
 
@@ -897,7 +905,7 @@ static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int
         const double us = (wide && o.share == 8 ? std::max(latency, 25.0 + marks) : latency + marks) + lookups;
         if (us < best) {
             best = us;
-            form = SieveForm{o.mid, o.planes, o.share, us};
+            form = SieveForm{o.mid, o.planes, o.share, us, motifs};
         }
     }
     return form;
@@ -946,6 +954,11 @@ static void plan_sieve(Plan &P, const std::vector<SieveForm> &form)
     }
 }
 
+// Expected motifs from which an answer is sorted by buckets: (13,4), n = 20,
+// m = 1000, 5300 of them, solve 412 -> 330 us; below about a thousand the
+// one-CTA sort takes no longer than two more launches.
+constexpr double kBucketMotifs = 1024;
+
 static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
 {
     Plan P;
@@ -975,6 +988,12 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
         in.q = (h->opt.quorum > 0 && h->opt.quorum < s.n) ? h->opt.quorum : s.n;
         in.nseed = s.n - in.q + 1;
         in.sieve_mid = form[k].mid;
+        // answers of chance motifs, which one CTA would sort for long
+        in.buckets = -1;
+        if (in.sieve_mid > 0 && form[k].motifs >= kBucketMotifs) {
+            in.buckets = (int)(P.bucketed.size() * kBucketWords);
+            P.bucketed.push_back((int)k);
+        }
         const bool tree = in.sieve_mid == 0;
         const long long seeds = (long long)in.nseed * in.W;
         const int cw = h->chunk_work_for(s.n, s.m, s.l, s.d);
@@ -1095,6 +1114,7 @@ static void fill_meta(const Plan &P, const MetaLayout &ml, char *hm)
     std::memcpy(hm + ml.segp, P.seg_pair.data(), P.seg_pair.size() * sizeof(Segment));
     std::memcpy(hm + ml.ctab, P.ctab.data(), P.ctab.size() * sizeof(int));
     std::memcpy(hm + ml.sieve, P.sieve_seg.data(), P.sieve_seg.size() * sizeof(SieveSeg));
+    std::memcpy(hm + ml.bucketed, P.bucketed.data(), P.bucketed.size() * sizeof(int));
 }
 
 // Enqueues the whole pipeline of a plan on h->stream. d_seq_src: device
@@ -1107,7 +1127,7 @@ static int enqueue_plan(pms_ctx *h, const Plan &P, const uint8_t *d_seq_src, Sta
 {
     const size_t k = P.inst.size();
     MetaLayout ml(P);
-    CtrLayout cl(k, (size_t)P.total_items);
+    CtrLayout cl(k, (size_t)P.total_items, P.bucketed.size());
     int rc;
     if ((rc = h->ensure(h->d_meta, ml.total)) || (rc = h->ensure(h->d_ctr, cl.total)) ||
         (rc = h->ensure(h->d_planes, P.planes * sizeof(uint2))) || (rc = h->ensure(h->d_raw, P.raw * 8)) ||
@@ -1200,7 +1220,8 @@ static int enqueue_plan(pms_ctx *h, const Plan &P, const uint8_t *d_seq_src, Sta
         sp.planes = mp.planes;
         sp.raw = mp.raw;
         sp.raw_count = d_rawcnt;
-        sp.flags = d_flags;
+        sp.key_count = (uint32_t *)(dc + cl.key_count);
+        sp.buckets = (uint32_t *)(dc + cl.buckets);
         if ((e = launch_sieve(sp, L.mid, L.planes, L.share, h->num_sms, st)) != cudaSuccess)
             return h->cuda_fail(e, "sieve kernel");
     }
@@ -1221,9 +1242,15 @@ static int enqueue_plan(pms_ctx *h, const Plan &P, const uint8_t *d_seq_src, Sta
             return h->cuda_fail(e, "pair kernel");
     }
     record_event(h, h->evm1, st, meta_dev != nullptr);
+    if (!P.bucketed.empty() &&
+        (e = launch_bucket_sort(d_inst, (const int *)(dm + ml.bucketed), (int)P.bucketed.size(), (uint64_t *)h->d_raw.p,
+                                (uint64_t *)h->d_tmp.p, (const uint32_t *)(dc + cl.key_count),
+                                (uint32_t *)(dc + cl.buckets), st)) != cudaSuccess)
+        return h->cuda_fail(e, "bucket sort kernels");
     if ((e = launch_sort_unique(d_inst, nullptr, (int)k, (uint64_t *)h->d_raw.p, (uint64_t *)h->d_tmp.p, d_rawcnt,
                                 d_flags, status_out,
-                                dense_out, dense_cap, (uint32_t *)(dc + cl.dense_total), st)) != cudaSuccess)
+                                dense_out, dense_cap, (uint32_t *)(dc + cl.dense_total), (const uint32_t *)(dc + cl.key_count),
+                                st)) != cudaSuccess)
         return h->cuda_fail(e, "sort/unique kernel");
     record_event(h, h->ev1, st, meta_dev != nullptr);
     return PMS_OK;
@@ -1339,6 +1366,7 @@ static void capture_graph(pms_ctx *h, const std::string &key, const Plan &P, con
                 std::memcpy(&G.sv.dense, a[7], sizeof G.sv.dense);
                 std::memcpy(&G.sv.dense_cap, a[8], sizeof G.sv.dense_cap);
                 std::memcpy(&G.sv.dense_total, a[9], sizeof G.sv.dense_total);
+                std::memcpy(&G.sv.key_count, a[10], sizeof G.sv.key_count);
             }
         }
         if (!G.pack || !G.sort)
@@ -1382,6 +1410,7 @@ static void capture_graph(pms_ctx *h, const std::string &key, const Plan &P, con
     S.sort_args[7] = &S.sv.dense;
     S.sort_args[8] = &S.sv.dense_cap;
     S.sort_args[9] = &S.sv.dense_total;
+    S.sort_args[10] = &S.sv.key_count;
 }
 
 // Enqueues a plan: a plan seen before (one instance or a batch: the same
@@ -1877,7 +1906,8 @@ struct Served {
     size_t pool_bytes = 0;
     PoolAlloc palloc;
     InstDev *d_inst = nullptr;       // [slots]
-    uint32_t *d_cnt = nullptr;       // raw_count[slots], flags[slots], dense_total[slots], zero[4], ids[slots]
+    uint32_t *d_cnt = nullptr;       // raw_count[slots], flags[slots], dense_total[slots], key_count[slots], zero[4],
+                                     // ids[slots]
     InstDev *h_inst = nullptr;       // pinned [slots]
     char *h_stage = nullptr;         // pinned [slots]: status block + inline codes of a finishing request
     static constexpr size_t kStage = sizeof(StatusDev) + kInlineKeys * 8;
@@ -1902,14 +1932,15 @@ struct Served {
     long long waves = 0, max_reqs_per_wave = 0, overlapped_waves = 0;
 };
 
-// d_cnt words: raw_count[slots], flags[slots], dense_total[slots], then an
+// d_cnt words: raw_count[slots], flags[slots], dense_total[slots], key_count[slots], then an
 // 8-word zero block (8-byte aligned; the prefix array of one-instance
 // launches), then the slot ids 0..slots-1 (instance lists of the sorts).
-static size_t srv_zero_word(int slots) { return round_up(3 * (size_t)slots, 2); }
+static size_t srv_zero_word(int slots) { return round_up(4 * (size_t)slots, 2); }
 static size_t srv_cnt_words(int slots) { return srv_zero_word(slots) + 8 + (size_t)slots; }
 static uint32_t *srv_rawcnt(Served *S) { return S->d_cnt; }
 static uint32_t *srv_flags(Served *S) { return S->d_cnt + S->slots; }
 static uint32_t *srv_dense_total(Served *S) { return S->d_cnt + 2 * S->slots; }
+static uint32_t *srv_keycnt(Served *S) { return S->d_cnt + 3 * S->slots; }
 static long long *srv_zero(Served *S) { return (long long *)(S->d_cnt + srv_zero_word(S->slots)); }
 static int *srv_ids(Served *S) { return (int *)(S->d_cnt + srv_zero_word(S->slots) + 8); }
 
@@ -2093,6 +2124,7 @@ static bool served_admit(Served *S, Request *r)
     in.q = r->n;
     in.nseed = 1;
     in.sieve_mid = r->form.mid;
+    in.buckets = -1;
     in.seq_off = (long long)(off + L.seqs);
     in.plane_off = (long long)((off + L.planes) / sizeof(uint2));
     in.raw_off = (long long)((off + L.raw) / 8);
@@ -2111,6 +2143,7 @@ static bool served_admit(Served *S, Request *r)
     cudaMemsetAsync(srv_rawcnt(S) + r->slot, 0, 4, st);
     cudaMemsetAsync(srv_flags(S) + r->slot, 0, 4, st);
     cudaMemsetAsync(srv_dense_total(S) + r->slot, 0, 4, st);
+    cudaMemsetAsync(srv_keycnt(S) + r->slot, 0, 4, st);
     const long long windows = (long long)r->n * r->W;
     launch_pack(S->d_inst + r->slot, 1, srv_zero(S), windows, (const uint8_t *)S->pool, (uint2 *)S->pool,
                 srv_flags(S) + r->slot, (int)std::max<long long>(1, std::min<long long>((windows + 255) / 256, h->num_sms * 8)),
@@ -2293,7 +2326,7 @@ static void served_loop(Served *S)
                     sp.planes = mp.planes;
                     sp.raw = mp.raw;
                     sp.raw_count = mp.raw_count;
-                    sp.flags = mp.flags;
+                    sp.key_count = srv_keycnt(S);
                     // a launch with few blocks gives each a CTA
                     const bool few = sp.total < 16ll * h->num_sms;
                     e = launch_sieve(sp, j + 3, 0, !few ? 1 : j >= 2 ? 8 : 0, h->num_sms, S->st);
@@ -2307,7 +2340,7 @@ static void served_loop(Served *S)
                                                (uint64_t *)S->pool + r->raw_cap, srv_rawcnt(S), srv_flags(S),
                                                (StatusDev *)(base + r->status_rel) - r->slot,
                                                (uint64_t *)(base + r->dense_rel), r->raw_cap,
-                                               srv_dense_total(S) + r->slot, S->st);
+                                               srv_dense_total(S) + r->slot, srv_keycnt(S), S->st);
                     if (e == cudaSuccess)
                         e = cudaMemcpyAsync(stage, base + r->status_rel, sizeof(StatusDev), cudaMemcpyDeviceToHost,
                                             S->st);
@@ -3395,7 +3428,7 @@ extern "C" int pms_solve_device_noalloc(const uint8_t *d_seqs, int n, int m, int
     const uint32_t cap = (uint32_t)std::min<size_t>(capacity, 0xffffffffu);
     if ((e = launch_sort_unique(d_inst, nullptr, 1, (uint64_t *)(base + o_raw), (uint64_t *)(base + o_tmp), d_rawcnt,
                                 d_flags, (StatusDev *)d_status, d_motifs, cap, (uint32_t *)(dc + cl.dense_total),
-                                st)) != cudaSuccess)
+                                nullptr, st)) != cudaSuccess)
         return PMS_ECUDA;
     return PMS_OK;
 }

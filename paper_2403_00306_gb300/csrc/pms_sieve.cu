@@ -273,12 +273,18 @@ __device__ __forceinline__ bool sv_occurs(const uint2 *__restrict__ win, int W, 
     return false;
 }
 
+// Where an instance's motifs go.
+struct SvOut {
+    uint64_t *raw;
+    uint32_t *raw_count, *key_count, *buckets;
+};
+
 // Up to 32 strings, one per lane (`has`): those that occur in the sequences
-// first..n-1 too are appended to the raw codes, once per window of the seed
-// sequences within d, as the tree form finds them.
+// first..n-1 too are appended to the keys. The raw count grows by the windows of
+// the seed sequences within d of them, as often as the tree form finds them.
 template <int kMid>
-__device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, uint64_t *raw, uint32_t *raw_count, uint32_t *flags,
-                                     const uint2 *__restrict__ win, bool has, uint2 c, int first, int lane)
+__device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, SvOut out, const uint2 *__restrict__ win,
+                                     bool has, uint2 c, int first, int lane)
 {
     const int n = inst->n, W = inst->W, d = inst->d, l = inst->l;
     uint32_t todo = __ballot_sync(kFull, has);
@@ -300,21 +306,17 @@ __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, uint64_t 
         if (lane == src)
             copies = k;
     }
-    int incl = copies;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o)
-            incl += y;
-    }
-    const int all = __shfl_sync(kFull, incl, 31);
-    if (all == 0)
+    const uint32_t found = __ballot_sync(kFull, copies > 0);
+    if (found == 0u)
         return;
+    const int all = __reduce_add_sync(kFull, copies);
     uint32_t base = 0;
-    if (lane == 0)
-        base = atomicAdd(raw_count, (uint32_t)all);
-    base = __shfl_sync(kFull, base, 0) + (uint32_t)(incl - copies);
-    if (copies > 0) {
+    if (lane == 0) {
+        atomicAdd(out.raw_count, (uint32_t)all);
+        base = atomicAdd(out.key_count, (uint32_t)__popc(found));
+    }
+    base = __shfl_sync(kFull, base, 0) + (uint32_t)__popc(found & ((1u << lane) - 1u));
+    if (copies > 0 && base < inst->raw_cap) {   // beyond it the raw count tells
         const int A = l - kMid - kSvSuf;
         const uint32_t mid = c.x >> 6;
         const uint32_t h = (c.y >> 16) | ((mid >> kMid) << A) | (((c.x >> 3) & 7u) << (A + kMid));
@@ -322,14 +324,15 @@ __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, uint64_t 
         uint64_t key = 0;
         for (int k = 0; k < l; ++k)
             key = (key << 2) | (uint64_t)((((h >> k) & 1u) << 1) | ((lo >> k) & 1u));
-        for (int k = 0; k < copies; ++k) {
-            const uint32_t pos = base + (uint32_t)k;
-            if (pos < inst->raw_cap)
-                raw[inst->raw_off + pos] = key;
-            else
-                atomicOr(flags, kFlagOverflow);
-        }
+        out.raw[inst->raw_off + base] = key;
+        if (inst->buckets >= 0)
+            atomicAdd(out.buckets + inst->buckets + bucket_of(key, l), 1u);
     }
+}
+
+__device__ __forceinline__ SvOut out_of(const SieveParams &p, int I)
+{
+    return SvOut{p.raw, p.raw_count + I, p.key_count + I, p.buckets};
 }
 
 // The string of bit `bit` of mark word `at` ([half][word]) of a block.
@@ -604,7 +607,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                         const bool has = v != 0u;
                         const int bit = has ? __ffs(v) - 1 : 0;
                         v &= v - 1u;
-                        sv_emit<kMid>(p.inst + blk.I, p.raw, p.raw_count + blk.I, p.flags + blk.I, blk.win, has,
+                        sv_emit<kMid>(p.inst + blk.I, out_of(p, blk.I), blk.win, has,
                                       sv_string<kMid>(blk.prefix, at, bit), i, lane);
                     }
                 }
@@ -677,7 +680,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_split_kernel(Sie
                     const bool has = v != 0u;
                     const int bit = has ? __ffs(v) - 1 : 0;
                     v &= v - 1u;
-                    sv_emit<kMid>(p.inst + blk.I, p.raw, p.raw_count + blk.I, p.flags + blk.I, blk.win, has,
+                    sv_emit<kMid>(p.inst + blk.I, out_of(p, blk.I), blk.win, has,
                                   sv_string<kMid>(blk.prefix, at, bit), in.n, lane);
                 }
             }

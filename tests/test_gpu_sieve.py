@@ -62,3 +62,29 @@ def test_sieve_and_tree_form_agree(case):
             outs.append((out.cpu().numpy(), st.cpu().numpy(), c.solve(seqs, l, d)))
     assert np.array_equal(outs[0][1], outs[1][1]) and np.array_equal(outs[0][0], outs[1][0])
     assert np.array_equal(outs[0][2], outs[1][2]) and len(outs[0][2]) > 0
+
+
+@pytest.mark.parametrize("case", [(9, 2, 12, 900, 0), (10, 3, 20, 500, 0), (11, 3, 12, 700, 0), (13, 4, 16, 900, 0),
+                                  (14, 4, 6, 900, 0), (11, 3, 14, 600, 13)], ids=str)
+def test_large_answers_sorted_by_buckets(case):
+    """Answers of a thousand to a few hundred thousand motifs (motifs of fewer and of more letters than
+    a bucket number holds), alone, in a batch and on the device entry point with too little room."""
+    import torch
+    l, d, n, m, q = case
+    seqs = pi.planted_instance(n, m, l, d, 21).seqs
+    with pms.Context(0) as c, pms.Context(0) as tree:
+        c.set_options(quorum=q)
+        tree.set_options(quorum=q, grab=1)
+        want = tree.solve(seqs, l, d)
+        assert len(want) > 1000
+        assert np.array_equal(c.solve(seqs, l, d), want)
+        for got in c.solve_batch([(seqs, l, d)] * 3):
+            assert np.array_equal(got, want)
+        out = torch.zeros(1024, dtype=torch.int64, device="cuda")
+        st = torch.zeros(4, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        c.solve_device(torch.from_numpy(seqs.copy()).cuda(), n, m, l, d, out, 1000, st)
+        torch.cuda.synchronize()
+        s = st.cpu().numpy().astype(np.uint32)
+        assert s[1] == len(want) and s[2] == 2
+        assert np.array_equal(out[:1000].cpu().numpy().astype(np.uint64), want[:1000]) and not out[1000:].any()
