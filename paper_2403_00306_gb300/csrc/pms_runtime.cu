@@ -896,12 +896,11 @@ static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int
         const double windows = o.share == 8 && !wide ? std::ceil(W / 256.0) * 256.0 : W;
         const double marks = rounds * windows * S * (o.a + o.b * words) * 1e-6;
         // every motif is looked up in the seed sequences, by as many warps as have blocks
-        const double lookups = motifs * seeds * 14e-6 * (o.share != 1 ? 1.0 : std::max(1.0, slots / blocks));
+        const double lookups = motifs * seeds * 14e-6 * (o.share == 8 ? 1.0 : std::max(1.0, slots / (o.share == 0 ? 20.0 * blocks : blocks)));
         const double latency = !single          ? 0.0
                                : !wide          ? 35.0
-                               : o.share == 8   ? 12.0 + 0.085 * W
-                               : l == 11        ? 10.0 + 0.052 * W
-                                                : 14.0 + 0.03 * W;
+                               : o.share == 8   ? 12.0 + 0.085 * W * std::max(n, 20) / 20.0
+                                                : ((n + 19) / 20) * (l == 11 ? 14.0 + 0.022 * W : 15.0 + 0.012 * W);
         const double us = (wide && o.share == 8 ? std::max(latency, 25.0 + marks) : latency + marks) + lookups;
         if (us < best) {
             best = us;

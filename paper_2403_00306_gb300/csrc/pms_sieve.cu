@@ -97,11 +97,11 @@ __host__ __device__ constexpr int sv_groups2()
 
 // Shared memory of a CTA besides its marks, which it precedes: the marks are
 // aligned to one half of a buffer.
-template <int kMid>
+template <int kMid, int kWarps = kSvWarps>
 struct SvSmem {
     uint32_t ball[4 * 64 * 2];             // g_sv_ball
     uint16_t change[sv_groups<kMid>() * 32];
-    uint32_t list[kSvWarps][64];           // windows with one change left, until 32 are there
+    uint32_t list[kWarps][64];             // windows with one change left, until 32 are there
     int first[kSvMaxShell + 2];
     long long item;                        // of the CTA, when its warps share a block
     int alive[3];                          // lanes that hold strings alive after sequence i, at i % 3
@@ -145,7 +145,8 @@ struct SvLane {
     uint32_t pair[sv_groups2<kMid>()];
     int t;                              // letters `single` changes
     int half;                           // the half of the words `single` works on first
-    __device__ __forceinline__ SvLane(const SvSmem<kMid> &sm, int lane)
+    template <class Smem>
+    __device__ __forceinline__ SvLane(const Smem &sm, int lane)
     {
         const int e0 = kBoth ? (lane & 15) : lane < 1 + 3 * kMid ? lane : lane - 16;
         half = kBoth ? lane >> 4 : 0;
@@ -165,9 +166,9 @@ struct SvLane {
 // windows in turn. marks: shared address, aligned to kHalf, so that within a
 // half a word address is an exclusive-or away from another. prefix: the
 // block's, as in a window's word.
-template <int kMid, int kShare>
+template <int kMid, int kShare, class Smem>
 __device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, int d, uint32_t prefix, uint32_t marks,
-                                        uint32_t *list, const SvSmem<kMid> &sm, const SvLane<kMid> &my, int g, int lane)
+                                        uint32_t *list, const Smem &sm, const SvLane<kMid> &my, int g, int lane)
 {
     using M = SvMarks<kMid>;
     constexpr int kStep = 32 * kShare;
@@ -366,38 +367,38 @@ __device__ __forceinline__ void share_sync()
 // Shared memory: the tables, then the buffers of marks at the next multiple of
 // kHalf of the shared address space, in which dynamic shared memory starts
 // after what the system reserves (`reserved`: 1 KB).
-template <int kMid>
+template <int kMid, int kWarps = kSvWarps>
 __host__ __device__ constexpr uint32_t sv_marks_at(uint32_t reserved)
 {
     using M = SvMarks<kMid>;
-    return (reserved + (uint32_t)sizeof(SvSmem<kMid>) + M::kHalf - 1) / M::kHalf * M::kHalf;
+    return (reserved + (uint32_t)sizeof(SvSmem<kMid, kWarps>) + M::kHalf - 1) / M::kHalf * M::kHalf;
 }
-template <int kMid>
+template <int kMid, int kWarps = kSvWarps>
 size_t sv_smem_bytes(int reserved, int buffers)
 {
-    return sv_marks_at<kMid>((uint32_t)reserved) - reserved + (size_t)buffers * SvMarks<kMid>::kBytes;
+    return sv_marks_at<kMid, kWarps>((uint32_t)reserved) - reserved + (size_t)buffers * SvMarks<kMid>::kBytes;
 }
 
 // Copies the tables to shared memory and clears the marks; returns the shared
 // address of the first buffer.
-template <int kMid>
+template <int kMid, int kWarps = kSvWarps>
 __device__ __forceinline__ uint32_t sv_setup(unsigned char *raw, int buffers)
 {
     using M = SvMarks<kMid>;
-    SvSmem<kMid> &sm = *reinterpret_cast<SvSmem<kMid> *>(raw);
+    SvSmem<kMid, kWarps> &sm = *reinterpret_cast<SvSmem<kMid, kWarps> *>(raw);
     const uint32_t raw0 = (uint32_t)__cvta_generic_to_shared(raw);
-    const uint32_t marks0 = sv_marks_at<kMid>(raw0);
+    const uint32_t marks0 = sv_marks_at<kMid, kWarps>(raw0);
     const SvTable &tab = g_sv_table[kMid - 3];
-    for (int i = threadIdx.x; i < sv_groups<kMid>() * 32; i += kSvThreads)
+    for (int i = threadIdx.x; i < sv_groups<kMid>() * 32; i += 32 * kWarps)
         sm.change[i] = tab.change[i];
-    for (int i = threadIdx.x; i < 4 * 64 * 2; i += kSvThreads)
+    for (int i = threadIdx.x; i < 4 * 64 * 2; i += 32 * kWarps)
         sm.ball[i] = (&g_sv_ball[0][0][0])[i];
     if (threadIdx.x < kSvMaxShell + 2)
         sm.first[threadIdx.x] = tab.first[threadIdx.x];
     if (threadIdx.x < 3)
         sm.alive[threadIdx.x] = 0;
     uint4 *m4 = reinterpret_cast<uint4 *>(raw + (marks0 - raw0));
-    for (int i = threadIdx.x; i < buffers * (int)(M::kBytes / 16); i += kSvThreads)
+    for (int i = threadIdx.x; i < buffers * (int)(M::kBytes / 16); i += 32 * kWarps)
         m4[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     return marks0;
@@ -623,17 +624,21 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
 }
 
 // The form for few blocks, q = n: a CTA per block, whose warps take the
-// sequences i = warp, warp + kSvWarps, ... with marks of their own, so that
-// they meet only once, to intersect what they are left with.
+// sequences i = warp, warp + kSplitWarps, ... with marks of their own, so that
+// they meet only once, to intersect what they are left with. Twenty warps: what
+// a solve waits for is one warp's sequences, and most instances have about
+// twenty (whole solves, 8 warps and 20: (9,2), n = 20, m = 600, 32.1 and 20.5 us;
+// (11,3), n = 17, m = 733, from host memory, 87 and 67 us).
+constexpr int kSplitWarps = 20;
 template <int kMid, int kMinBlocks>
-__global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_split_kernel(SieveParams p)
+__global__ void __launch_bounds__(32 * kSplitWarps, kMinBlocks) sieve_split_kernel(SieveParams p)
 {
     extern __shared__ __align__(16) unsigned char sv_raw[];
     using M = SvMarks<kMid>;
     constexpr int kPieces = 2 * M::kWords / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    SvSmem<kMid> &sm = *reinterpret_cast<SvSmem<kMid> *>(sv_raw);
-    const uint32_t marks0 = sv_setup<kMid>(sv_raw, kSvWarps);
+    SvSmem<kMid, kSplitWarps> &sm = *reinterpret_cast<SvSmem<kMid, kSplitWarps> *>(sv_raw);
+    const uint32_t marks0 = sv_setup<kMid, kSplitWarps>(sv_raw, kSplitWarps);
     const uint32_t marks = marks0 + warp * M::kBytes;
     uint32_t *all = reinterpret_cast<uint32_t *>(sv_raw + (marks0 - (uint32_t)__cvta_generic_to_shared(sv_raw)));
     uint32_t *mw = all + warp * (2 * M::kWords);
@@ -650,7 +655,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_split_kernel(Sie
 #pragma unroll
         for (int k = 0; k < kPieces; ++k)
             cur[k] = kFull;
-        for (int i = warp; i < in.n && !*(volatile int *)dead; i += kSvWarps) {
+        for (int i = warp; i < in.n && !*(volatile int *)dead; i += kSplitWarps) {
             sv_mark<kMid, 1>(blk.win + (size_t)i * in.W, in.W, in.d, blk.prefix, marks, sm.list[warp], sm, my, 0,
                              lane);
             __syncwarp();
@@ -670,11 +675,11 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_split_kernel(Sie
             mw[k * 32 + lane] = cur[k];
         __syncthreads();
         if (!*(volatile int *)dead) {
-            // mark word at: warp at / 32 % kSvWarps
-            for (int at = warp * 32 + lane; at < 2 * M::kWords; at += kSvThreads) {
+            // mark word at: warp at / 32 % kSplitWarps
+            for (int at = warp * 32 + lane; at < 2 * M::kWords; at += 32 * kSplitWarps) {
                 uint32_t v = kFull;
 #pragma unroll
-                for (int t = 0; t < kSvWarps; ++t)
+                for (int t = 0; t < kSplitWarps; ++t)
                     v &= all[t * (2 * M::kWords) + at];
                 while (__any_sync(kFull, v != 0u)) {
                     const bool has = v != 0u;
@@ -743,14 +748,15 @@ void fill_table(SvTable &t)
     }
 }
 
-cudaError_t launch_kernel(void (*kernel)(SieveParams), const SieveParams &p, long long blocks, size_t smem, cudaStream_t st)
+cudaError_t launch_kernel(void (*kernel)(SieveParams), const SieveParams &p, long long blocks, size_t smem,
+                          cudaStream_t st, int threads = kSvThreads)
 {
     const cudaError_t e =
         cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return e;
     cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = dependent_launch(attr, (int)blocks, kSvThreads, smem, st);
+    const cudaLaunchConfig_t cfg = dependent_launch(attr, (int)blocks, threads, smem, st);
     return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
@@ -767,7 +773,7 @@ template <int kMid, int kMinBlocks>
 cudaError_t launch_split(const SieveParams &p, int sms, int reserved, cudaStream_t st)
 {
     return launch_kernel(sieve_split_kernel<kMid, kMinBlocks>, p, std::min<long long>((long long)sms * kMinBlocks, p.total),
-                         sv_smem_bytes<kMid>(reserved, kSvWarps), st);
+                         sv_smem_bytes<kMid, kSplitWarps>(reserved, kSplitWarps), st, 32 * kSplitWarps);
 }
 
 }  // namespace
@@ -810,8 +816,8 @@ cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, i
     if (mid == 5)
         return share == 1 ? launch<5, 0, 1, 2>(p, sms, reserved, st) : launch<5, 0, 8, 4>(p, sms, reserved, st);
     if (mid == 4)
-        return share == 1 ? launch<4, 0, 1, 4>(p, sms, reserved, st) : launch_split<4, 5>(p, sms, reserved, st);
-    return share == 1 ? launch<3, 0, 1, 5>(p, sms, reserved, st) : launch_split<3, 5>(p, sms, reserved, st);
+        return share == 1 ? launch<4, 0, 1, 4>(p, sms, reserved, st) : launch_split<4, 2>(p, sms, reserved, st);
+    return share == 1 ? launch<3, 0, 1, 5>(p, sms, reserved, st) : launch_split<3, 2>(p, sms, reserved, st);
 }
 
 }  // namespace pms
