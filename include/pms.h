@@ -77,9 +77,10 @@ typedef struct {
     int chunk_work;        /* target work of one queue item, in candidate units */
     int grab;              /* tree-node filter: 0 = the tuned value, else 1;
                               1 = by words of up to 32 nodes, a row at a time
-                              (default; trees of more than 2^18 nodes: a
-                              lane-asynchronous walk, every lane taking one
-                              node through the rows and leaving a row at the
+                              (default; where chance occurrences are common
+                              and for trees of more than 2^18 nodes a
+                              lane-asynchronous walk: every lane takes one
+                              node through the rows and leaves a row at the
                               node's own first feasible occurrence); g > 1 =
                               breadth-first batches of up to 128 nodes that
                               shrink to g nodes as a queue item runs out
