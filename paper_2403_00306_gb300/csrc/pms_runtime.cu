@@ -899,8 +899,10 @@ static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int
         const double rounds = single && !wide && o.share == 1 ? std::ceil(blocks / slots) * slots : blocks;
         const double windows = o.share == 8 && !wide ? std::ceil(W / 256.0) * 256.0 : W;
         const double marks = rounds * windows * S * (o.a + o.b * words) * 1e-6;
-        // every motif is looked up in the seed sequences, by as many warps as have blocks
-        const double lookups = motifs * seeds * 14e-6 * (o.share == 8 ? 1.0 : std::max(1.0, slots / (o.share == 0 ? 20.0 * blocks : blocks)));
+        // every motif is looked up in the seed sequences, by as many warps as have
+        // blocks, or where a block holds many their windows are passed over once more
+        const double warps = o.share == 8 ? slots : std::min(slots, o.share == 0 ? 20.0 * blocks : blocks);
+        const double lookups = std::min(motifs * seeds * 14e-6 * slots / warps, 2.0 + marks * (n - q + 1) / S);
         const double latency = !single          ? 0.0
                                : !wide          ? 35.0
                                : o.share == 8   ? 12.0 + 0.085 * W * std::max(n, 20) / 20.0

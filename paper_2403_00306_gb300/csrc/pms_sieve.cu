@@ -88,6 +88,16 @@ __device__ SvTable g_sv_table[4];          // kMid = 3, 4, 5, 6
 // bits of the ball of radius v around last letters s, one half of the 64: [v][s][half]
 __device__ uint32_t g_sv_ball[4][64][2];
 
+// changes of t of kMid letters
+template <int kMid>
+__host__ __device__ constexpr int sv_shell(int t)
+{
+    int c = 1;
+    for (int i = 0; i < t; ++i)
+        c = c * 3 * (kMid - i) / (i + 1);
+    return c;
+}
+
 // groups of the shell of two changes: the table entries a lane keeps in registers
 template <int kMid>
 __host__ __device__ constexpr int sv_groups2()
@@ -126,6 +136,30 @@ __device__ __forceinline__ void red_or_if(bool on, uint32_t addr, uint32_t v)
                  "r"(v));
 }
 
+// What a pass over windows does with the words of their balls: mark them, or
+// count the strings that are marked already.
+struct SvMark {
+    static constexpr bool kCount = false;
+    __device__ __forceinline__ void operator()(uint32_t addr, uint32_t bits, bool = true) { red_or(addr, bits); }
+    __device__ __forceinline__ void if_(bool on, uint32_t addr, uint32_t bits) { red_or_if(on, addr, bits); }
+};
+struct SvCount {
+    static constexpr bool kCount = true;
+    uint32_t found = 0;
+    // once: not a lane that repeats another's change
+    __device__ __forceinline__ void operator()(uint32_t addr, uint32_t bits, bool once = true)
+    {
+        uint32_t v;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+        found += once ? (uint32_t)__popc(v & bits) : 0u;
+    }
+    __device__ __forceinline__ void if_(bool on, uint32_t addr, uint32_t bits)
+    {
+        if (on)
+            (*this)(addr, bits);
+    }
+};
+
 // The distance of two strings as sieve words (see sieve_word), prefix included.
 template <int kMid>
 __device__ __forceinline__ int sv_distance(uint2 a, uint2 b)
@@ -162,18 +196,20 @@ struct SvLane {
     }
 };
 
-// The windows of one sequence mark the block's words; kShare warps take 32
-// windows in turn. marks: shared address, aligned to kHalf, so that within a
+// The windows of one sequence mark the block's words (or count the strings
+// marked there, see SvCount); kShare warps take 32 windows in turn. marks: shared address, aligned to kHalf, so that within a
 // half a word address is an exclusive-or away from another. prefix: the
 // block's, as in a window's word.
-template <int kMid, int kShare, class Smem>
-__device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, int d, uint32_t prefix, uint32_t marks,
-                                        uint32_t *list, const Smem &sm, const SvLane<kMid> &my, int g, int lane)
+template <int kMid, int kShare, class Op, class Smem>
+__device__ __forceinline__ void sv_pass(Op &op, const uint2 *__restrict__ win, int W, int d, uint32_t prefix,
+                                        uint32_t marks, uint32_t *list, const Smem &sm, const SvLane<kMid> &my, int g,
+                                        int lane)
 {
     using M = SvMarks<kMid>;
     constexpr int kStep = 32 * kShare;
     constexpr bool kBoth = SvLane<kMid>::kBoth;
     const uint32_t lt = (1u << lane) - 1u;
+    const bool once1 = (kBoth ? lane & 15 : lane) <= 3 * kMid;   // `single` is no other lane's
     const uint32_t single0 = marks + my.single;
     const uint32_t *ball2 = sm.ball + (2 - my.t) * 128 + my.half;   // radius 2 or 1 of the last letters
     int n1 = 0;
@@ -187,7 +223,7 @@ __device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, in
         const int r = in ? d - __popc((y | (y >> 16)) & 0xffffu) : -1;
         // word offset in a half's marks; the last three letters choose half and bit
         const uint32_t off = (code >> 6) << 2;
-        red_or_if(r == 0, (marks + (code & 32u) * (M::kHalf / 32u)) ^ off, 1u << (code & 31u));
+        op.if_(r == 0, (marks + (code & 32u) * (M::kHalf / 32u)) ^ off, 1u << (code & 31u));
         const uint32_t one = __ballot_sync(kFull, r == 1);
         if (r == 1)
             list[n1 + __popc(one & lt)] = code;
@@ -198,13 +234,13 @@ __device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, in
             const uint32_t v = __shfl_sync(kFull, packed, __ffs(two) - 1);
             two &= two - 1u;
             const uint32_t o = v & 0xffffu, suf = (v >> 16) & 63u;
-            red_or(single0 ^ o, ball2[2 * suf]);
+            op(single0 ^ o, ball2[2 * suf], once1);
             if (!kBoth)
-                red_or((single0 + M::kHalf) ^ o, ball2[2 * suf + 1]);
+                op((single0 + M::kHalf) ^ o, ball2[2 * suf + 1], once1);
             const uint32_t wh = (marks + (suf >> 5) * M::kHalf) ^ o, bit = 1u << (suf & 31u);
 #pragma unroll
             for (int t = 0; t < sv_groups2<kMid>(); ++t)
-                red_or(wh ^ my.pair[t], bit);
+                op(wh ^ my.pair[t], bit, 32 * t + lane < sv_shell<kMid>(2));
         }
         uint32_t more = __ballot_sync(kFull, r > 2);
         while (more) {
@@ -214,18 +250,20 @@ __device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, in
             const int rr = __shfl_sync(kFull, r, src);
             const uint32_t o = v & 0xffffu, suf = (v >> 16) & 63u;
             const uint32_t *ball = sm.ball + 2 * suf;
-            red_or(single0 ^ o, ball[min(rr - my.t, 3) * 128 + my.half]);
+            op(single0 ^ o, ball[min(rr - my.t, 3) * 128 + my.half], once1);
             if (!kBoth)
-                red_or((single0 + M::kHalf) ^ o, ball[min(rr - my.t, 3) * 128 + 1]);
+                op((single0 + M::kHalf) ^ o, ball[min(rr - my.t, 3) * 128 + 1], once1);
             const int tmax = min(rr, kMid);
             const uint16_t *ch = sm.change + lane;
             for (int t = 2; t <= tmax; ++t) {
                 const int q1 = sm.first[t + 1];
+                // groups of the shell without repeated changes
+                const int whole = Op::kCount ? sm.first[t] + ((sv_shell<kMid>(t) - lane + 31) >> 5) : q1;
                 if (t == rr) {
                     const uint32_t wh = (marks + (suf >> 5) * M::kHalf) ^ o, bit = 1u << (suf & 31u);
 #pragma unroll 4
                     for (int q = sm.first[t]; q < q1; ++q)
-                        red_or(wh ^ ch[q * 32], bit);
+                        op(wh ^ ch[q * 32], bit, q < whole);
                 } else {
                     const uint32_t wa = marks ^ o;
                     const int rad = min(rr - t, 3);
@@ -233,8 +271,8 @@ __device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, in
 #pragma unroll 4
                     for (int q = sm.first[t]; q < q1; ++q) {
                         const uint32_t wc = wa ^ ch[q * 32];
-                        red_or(wc, b0);
-                        red_or(wc + M::kHalf, b1);
+                        op(wc, b0, q < whole);
+                        op(wc + M::kHalf, b1, q < whole);
                     }
                 }
             }
@@ -246,12 +284,12 @@ __device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, in
             const uint32_t v = list[lane], up = list[32 + lane];
             if (lane < n1) {
                 const uint32_t suf = v & 63u, o = (v >> 6) << 2;
-                red_or(marks ^ o, sm.ball[128 + 2 * suf]);
-                red_or((marks + M::kHalf) ^ o, sm.ball[128 + 2 * suf + 1]);
+                op(marks ^ o, sm.ball[128 + 2 * suf]);
+                op((marks + M::kHalf) ^ o, sm.ball[128 + 2 * suf + 1]);
                 const uint32_t wh = (marks + (suf >> 5) * M::kHalf) ^ o, bit = 1u << (suf & 31u);
 #pragma unroll
                 for (int e = 1; e <= 3 * kMid; ++e)
-                    red_or(wh ^ (sv_single<kMid>(e) << 2), bit);
+                    op(wh ^ (sv_single<kMid>(e) << 2), bit);
             }
             __syncwarp();
             list[lane] = up;
@@ -259,6 +297,36 @@ __device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, in
             __syncwarp();
         }
     }
+}
+
+template <int kMid, int kShare, class Smem>
+__device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, int d, uint32_t prefix, uint32_t marks,
+                                        uint32_t *list, const Smem &sm, const SvLane<kMid> &my, int g, int lane)
+{
+    SvMark op;
+    sv_pass<kMid, kShare>(op, win, W, d, prefix, marks, list, sm, my, g, lane);
+}
+
+// Strings of a block from which their windows in the seed sequences are counted
+// by a pass over those windows, as marking does, instead of string by string: a
+// string's own look at the windows costs about 8 instructions per 32 of them, the
+// pass 60 to 300 whatever the number of strings. Whole solves, us, without and
+// with it: (9,2), n = 20, m = 1200 105 and 63; (11,3), n = 20, m = 1200 147 and
+// 82; 256 mixed instances, some of 600 k motifs, 34.6 and 25.1 ms.
+constexpr int kSvCountFrom = 32;
+
+// Adds the windows of win[0..W) within d of each string marked in the block,
+// summed over the strings, to the raw count; kShare warps take part.
+template <int kMid, int kShare, class Smem>
+__device__ __noinline__ void sv_count(const uint2 *__restrict__ win, int W, int d, uint32_t prefix, uint32_t marks,
+                                      uint32_t *list, const Smem &sm, uint32_t *raw_count, int g, int lane)
+{
+    SvCount op;
+    const SvLane<kMid> my(sm, lane);
+    sv_pass<kMid, kShare>(op, win, W, d, prefix, marks, list, sm, my, g, lane);
+    const uint32_t all = __reduce_add_sync(kFull, op.found);
+    if (lane == 0 && all != 0u)
+        atomicAdd(raw_count, all);
 }
 
 // Does a window of the sequence lie within d of the string c? Warp-uniform.
@@ -282,14 +350,19 @@ struct SvOut {
 
 // Up to 32 strings, one per lane (`has`): those that occur in the sequences
 // first..n-1 too are appended to the keys. The raw count grows by the windows of
-// the seed sequences within d of them, as often as the tree form finds them.
+// the seed sequences within d of them, as often as the tree form finds them
+// (unless these are counted already).
 template <int kMid>
 __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, SvOut out, const uint2 *__restrict__ win,
-                                     bool has, uint2 c, int first, int lane)
+                                     bool has, uint2 c, int first, bool counted, int lane)
 {
     const int n = inst->n, W = inst->W, d = inst->d, l = inst->l;
     uint32_t todo = __ballot_sync(kFull, has);
     int copies = 0;
+    if (counted && first >= n) {
+        copies = has ? 1 : 0;
+        todo = 0u;
+    }
     while (todo) {
         const int src = __ffs(todo) - 1;
         todo &= todo - 1u;
@@ -313,7 +386,8 @@ __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, SvOut out
     const int all = __reduce_add_sync(kFull, copies);
     uint32_t base = 0;
     if (lane == 0) {
-        atomicAdd(out.raw_count, (uint32_t)all);
+        if (!counted)
+            atomicAdd(out.raw_count, (uint32_t)all);
         base = atomicAdd(out.key_count, (uint32_t)__popc(found));
     }
     base = __shfl_sync(kFull, base, 0) + (uint32_t)__popc(found & ((1u << lane) - 1u));
@@ -487,7 +561,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
         const InstDev &in = blk.in;
         // what is left of the block's strings goes back to its marks
         uint32_t left = 0;   // != 0: this thread holds some
-        int i = 0;
+        int i = 0, holding = 0;   // holding: threads that do, of the block
         if constexpr (kPlanes == 0) {
             uint32_t cur[kPieces];
 #pragma unroll
@@ -539,6 +613,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                         *(volatile int *)&sm.alive[(i + 1) % 3] = 0;
                 }
                 ++i;
+                holding = lanes;
                 if (lanes <= kSvLookupLanes)
                     break;
             }
@@ -587,11 +662,19 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                     break;
                 }
             }
+            holding = kShare == 1 ? __popc(__ballot_sync(kFull, left != 0u)) : __syncthreads_count(left != 0u);
             if (__any_sync(kFull, left != 0u)) {
 #pragma unroll
                 for (int k = 0; k < kPieces; ++k)
                     mw[at_of(k)] = sv_above<kPlanes, kPieces>(cnt, k, in.q - 1);
             }
+        }
+        const bool counted = i == in.n && holding >= kSvCountFrom / 2;
+        if (counted) {   // the windows of s_1..s_{n-q+1} are contiguous
+            share_sync<kShare>();
+            sv_count<kMid, kShare>(blk.win, in.nseed * in.W, in.d, blk.prefix, marks, sm.list[warp], sm,
+                                   p.raw_count + blk.I, g, lane);
+            share_sync<kShare>();
         }
         // the strings of a warp's threads, the pieces of one thread at a time
         uint32_t holders = __ballot_sync(kFull, left != 0u);
@@ -609,7 +692,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                         const int bit = has ? __ffs(v) - 1 : 0;
                         v &= v - 1u;
                         sv_emit<kMid>(p.inst + blk.I, out_of(p, blk.I), blk.win, has,
-                                      sv_string<kMid>(blk.prefix, at, bit), i, lane);
+                                      sv_string<kMid>(blk.prefix, at, bit), i, counted, lane);
                     }
                 }
             }
@@ -647,7 +730,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps, kMinBlocks) sieve_split_kern
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the packed windows are complete and visible
     for (long long it = blockIdx.x; it < p.total; it += gridDim.x) {
         if (threadIdx.x == 0)
-            *dead = 0;
+            sm.alive[0] = sm.alive[1] = 0;
         __syncthreads();
         SvBlock blk(p, it, kMid);
         const InstDev &in = blk.in;
@@ -676,17 +759,32 @@ __global__ void __launch_bounds__(32 * kSplitWarps, kMinBlocks) sieve_split_kern
         __syncthreads();
         if (!*(volatile int *)dead) {
             // mark word at: warp at / 32 % kSplitWarps
+            int strings = 0;
             for (int at = warp * 32 + lane; at < 2 * M::kWords; at += 32 * kSplitWarps) {
                 uint32_t v = kFull;
 #pragma unroll
                 for (int t = 0; t < kSplitWarps; ++t)
                     v &= all[t * (2 * M::kWords) + at];
+                all[at] = v;
+                strings += __popc(v);
+            }
+            strings = __reduce_add_sync(kFull, strings);
+            if (lane == 0 && strings > 0)
+                atomicAdd(&sm.alive[1], strings);
+            __syncthreads();
+            const bool counted = *(volatile int *)&sm.alive[1] >= kSvCountFrom;
+            if (counted) {
+                sv_count<kMid, kSplitWarps>(blk.win, in.nseed * in.W, in.d, blk.prefix, marks0, sm.list[warp], sm,
+                                            p.raw_count + blk.I, warp, lane);
+            }
+            for (int at = warp * 32 + lane; at < 2 * M::kWords; at += 32 * kSplitWarps) {
+                uint32_t v = all[at];
                 while (__any_sync(kFull, v != 0u)) {
                     const bool has = v != 0u;
                     const int bit = has ? __ffs(v) - 1 : 0;
                     v &= v - 1u;
                     sv_emit<kMid>(p.inst + blk.I, out_of(p, blk.I), blk.win, has,
-                                  sv_string<kMid>(blk.prefix, at, bit), in.n, lane);
+                                  sv_string<kMid>(blk.prefix, at, bit), in.n, counted, lane);
                 }
             }
         }
