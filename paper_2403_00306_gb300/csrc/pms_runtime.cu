@@ -851,9 +851,7 @@ static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int
 {
     const double W = m - l + 1, E = expected_near(m, l, d), p = 1.0 - std::exp(-E);
     const double seeds = W * (n - q + 1);
-    // short motifs that most sequences hold: the answer is a good part of all
-    // 4^l strings, and writing it is what takes the time
-    if (n < 2 || (l == 8 && E > 1.0))
+    if (n < 2)
         return SieveForm{};
     const double per_candidate =
         q == n ? 4000e-6 * E * E * E / (1.0 + E / 0.15) : 390e-6 * E * E * E / (E + 0.02) * (1.0 + 3.0 * (n - q));
