@@ -1925,12 +1925,20 @@ struct Served {
     char *d_ring = nullptr;
     char *h_ring = nullptr;          // pinned
     size_t ring_stride = 0;
+    // after the ring: the steal cursor (16 bytes) and the claim counters of one
+    // wave's items, so that CTAs that ran out of items join others'. One wave
+    // runs at a time (stream order). None under a small memory budget; a wave
+    // of more items runs without.
+    static constexpr int kClaimItems = 1 << 16;
+    char *d_claim = nullptr;
+    size_t ring_bytes = 0;           // of the allocation, claim counters included
     cudaEvent_t ring_ev[kRing] = {};
     int ring_pos = 0;
     uint32_t *d_scratch = nullptr;
     size_t scratch_bytes = 0;
     long long rows_cap = 0;
-    int blocks = 0;
+    int blocks = 0;        // CTAs the row scratch has room for
+    int occ[2] = {1, 1};   // CTAs per SM of the verification kernel and of its small-rows form
     std::vector<cudaEvent_t> wave_ev;   // in-flight waves
     std::string fatal;
     long long waves = 0, max_reqs_per_wave = 0, overlapped_waves = 0;
@@ -1972,7 +1980,13 @@ static int served_start(pms_ctx *h)
     S->d_inst = (InstDev *)h->dev_alloc(S->slots * sizeof(InstDev));
     S->d_cnt = (uint32_t *)h->dev_alloc(cnt_words * 4);
     S->ring_stride = round_up(Served::kRingSegs + (size_t)S->slots * (sizeof(Segment) + sizeof(SieveSeg)), 256);
-    S->d_ring = (char *)h->dev_alloc(S->ring_stride * Served::kRing);
+    S->ring_bytes = S->ring_stride * Served::kRing;
+    const bool claims = h->budget == 0 || h->budget - h->used >= ((size_t)256 << 20);
+    if (claims)
+        S->ring_bytes += 16 + 8 * (size_t)Served::kClaimItems;
+    S->d_ring = (char *)h->dev_alloc(S->ring_bytes);
+    if (claims && S->d_ring)
+        S->d_claim = S->d_ring + S->ring_stride * Served::kRing;
     bool ok = S->pool && S->d_inst && S->d_cnt && S->d_ring;
     if (ok)
         ok = cudaHostAlloc((void **)&S->h_inst, S->slots * sizeof(InstDev), cudaHostAllocDefault) == cudaSuccess &&
@@ -1985,7 +1999,7 @@ static int served_start(pms_ctx *h)
         h->dev_free(S->pool, pool);
         h->dev_free(S->d_inst, S->slots * sizeof(InstDev));
         h->dev_free(S->d_cnt, cnt_words * 4);
-        h->dev_free(S->d_ring, S->ring_stride * Served::kRing);
+        h->dev_free(S->d_ring, S->ring_bytes);
         if (S->h_inst)
             cudaFreeHost(S->h_inst);
         if (S->h_ctab)
@@ -2008,10 +2022,12 @@ static int served_start(pms_ctx *h)
         cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     for (int i = S->slots - 1; i >= 0; --i)
         S->free_slots.push_back(i);
-    int occ = std::max(1, h->occ[0]);
-    if (h->opt.ctas_per_sm > 0)
-        occ = std::min(occ, h->opt.ctas_per_sm);
-    S->blocks = h->num_sms * occ;
+    for (int f = 0; f < 2; ++f) {
+        S->occ[f] = std::max(1, f ? h->occ_small[0] : h->occ[0]);
+        if (h->opt.ctas_per_sm > 0)
+            S->occ[f] = std::min(S->occ[f], h->opt.ctas_per_sm);
+    }
+    S->blocks = h->num_sms * std::max(S->occ[0], S->occ[1]);
     h->served = S.release();
     h->served->th = std::thread(served_loop, h->served);
     return PMS_OK;
@@ -2040,7 +2056,7 @@ static void served_stop(pms_ctx *h)
     h->dev_free(S->pool, S->pool_bytes);
     h->dev_free(S->d_inst, S->slots * sizeof(InstDev));
     h->dev_free(S->d_cnt, cnt_words * 4);
-    h->dev_free(S->d_ring, S->ring_stride * Served::kRing);
+    h->dev_free(S->d_ring, S->ring_bytes);
     if (S->d_scratch)
         h->dev_free(S->d_scratch, S->scratch_bytes);
     cudaFreeHost(S->h_inst);
@@ -2237,6 +2253,7 @@ static void served_loop(Served *S)
             long long items = 0;
             double units = 0;
             long long need_rows = 0;
+            bool small = S->occ[1] > S->occ[0];   // the small-rows form, by the rule of make_plan
             for (Request *r : S->active) {
                 if (r->state != 1 || r->chunks_next >= r->chunks_total)
                     continue;
@@ -2259,6 +2276,8 @@ static void served_loop(Served *S)
                 items += take;
                 units += take * r->units_per_chunk;
                 need_rows = std::max<long long>(need_rows, (long long)round_up((size_t)(r->n - 1) * (r->W + 3), 4));
+                if (expected_seed_rows(r->n, r->m, r->l, r->d) > kSmallFormRows)
+                    small = false;
                 if (r->chunks_next >= r->chunks_total)
                     finishing.push_back(r);
             }
@@ -2278,7 +2297,8 @@ static void served_loop(Served *S)
                         S->d_scratch = (uint32_t *)h->dev_alloc(S->scratch_bytes);
                         if (S->d_scratch)
                             break;
-                        S->blocks /= 2;
+                        const int least = h->num_sms * std::min(S->occ[0], S->occ[1]);
+                        S->blocks = S->blocks > least ? least : S->blocks / 2;
                     }
                     if (!S->d_scratch) {
                         served_fail_all(S, "served form: no memory for the row scratch");
@@ -2314,10 +2334,21 @@ static void served_loop(Served *S)
                 mp.flags = srv_flags(S);
                 mp.scratch = S->d_scratch;
                 mp.rows_cap = (int)S->rows_cap;
-                mp.smem_rows_cap = h->opt.smem_rows > 0 ? std::min(h->opt.smem_rows, kRowSmemCap) : kRowSmemCap;
+                const int rows_cap_smem = small ? kRowSmemCapSmall : kRowSmemCap;
+                mp.smem_rows_cap = h->opt.smem_rows > 0 ? std::min(h->opt.smem_rows, rows_cap_smem) : rows_cap_smem;
                 mp.counters = nullptr;
+                long long ctas = std::min<long long>(S->blocks, (long long)h->num_sms * S->occ[small]);
+                if (S->d_claim && items <= Served::kClaimItems) {
+                    mp.steal_state = (unsigned int *)S->d_claim;
+                    mp.item_claim = (int *)(S->d_claim + 16);
+                    ctas = std::min(ctas, 2 * items);
+                    if (e == cudaSuccess && items > 0)
+                        e = cudaMemsetAsync(S->d_claim, 0, 16 + 8 * (size_t)items, S->st);
+                } else {
+                    ctas = std::min(ctas, items);
+                }
                 if (e == cudaSuccess && items > 0)
-                    e = launch_main(mp, (int)std::min<long long>(S->blocks, items), false, S->st);
+                    e = launch_main(mp, (int)ctas, false, S->st, small);
                 for (int j = 0; j < 4 && e == cudaSuccess; ++j) {
                     if (sieve_segs[j].empty())
                         continue;
