@@ -57,9 +57,15 @@ constexpr uint32_t kFull = 0xffffffffu;
 constexpr int kSvWarps = 8;
 constexpr int kSvThreads = kSvWarps * 32;
 constexpr int kSvMaxShell = 6;             // changed middle letters, at most kMid
-// Lanes that still hold strings, at or below which a block looks its strings up
-// in the remaining sequences instead of marking them.
-constexpr int kSvLookupLanes = 2;
+// Threads that still hold strings, at or below which a block looks its strings up
+// in the remaining sequences instead of marking them. A CTA that shares six
+// letters waits for the warp with the most strings. Solves, us, at 0, 2, 6 and 12:
+// (17,5), n = 20, m = 1200 4303, 4102, 4214 and 4627 (4326 before the look-ups had
+// four loads in flight); five letters at 2, 12 and
+// 24: (13,4), n = 20, m = 600 162, 150 and 152; a warp per block, 256 mixed
+// instances, 2 and 5: 24.4 and 24.0 ms.
+template <int kMid, int kShare>
+constexpr int kSvLookupLanes = kMid == 6 ? 2 : kShare == 1 ? 5 : 12;
 
 // Index change of one changed letter: number e = 1 + 3 p + v changes position
 // p by v + 1 (exclusive-or of the 2-bit code); e = 0 is no change.
@@ -333,9 +339,13 @@ __device__ __noinline__ void sv_count(const uint2 *__restrict__ win, int W, int 
 template <int kMid>
 __device__ __forceinline__ bool sv_occurs(const uint2 *__restrict__ win, int W, int d, uint2 c, int lane)
 {
-    for (int w0 = 0; w0 < W; w0 += 32) {
-        const int w = w0 + lane;
-        const bool hit = w < W && sv_distance<kMid>(__ldg(win + w), c) <= d;
+    for (int w0 = 0; w0 < W; w0 += 128) {   // four loads in flight
+        bool hit = false;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int w = min(w0 + 32 * k + lane, W - 1);   // the last window again
+            hit |= sv_distance<kMid>(__ldg(win + w), c) <= d;
+        }
         if (__any_sync(kFull, hit))
             return true;
     }
@@ -614,7 +624,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                 }
                 ++i;
                 holding = lanes;
-                if (lanes <= kSvLookupLanes)
+                if (lanes <= kSvLookupLanes<kMid, kShare>)
                     break;
             }
             if (kBuf > 1)
