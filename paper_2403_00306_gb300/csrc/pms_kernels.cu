@@ -17,7 +17,8 @@
 //     it mismatches w wherever w agrees with x, and off P it mismatches w
 //     wherever x does. A node with an empty reduced row has no motif among
 //     its 3^|P| leaves (the branch-and-bound of qPMSPrune, applied per node);
-//     each lane walks one node through the rows with this bound;
+//     up to 32 nodes are filtered at once as the bits of a word, or, where
+//     most nodes pass, a lane walks one node through the rows;
 //   * below a surviving node, partial candidates (letters fixed above the
 //     three lowest changed positions) are tested with the exact bound over
 //     their leaves, or the 81 leaves of a 4-position node are handled as a
@@ -864,7 +865,8 @@ __device__ __forceinline__ int filter_subsets(const WarpCtx &c, int N)
     return N;
 }
 
-// The walk of single nodes, for trees of too many nodes for a word table.
+// The walk of single nodes, where most nodes pass a row and for trees of too
+// many nodes for a word table.
 // Lane-asynchronous node filter of a chunk: every lane holds one tree node P
 // and its position in the rows (row rank r, entry quad e4); each step a lane
 // tests the next 4 * kWalkQuads entries of its own row with the bound popc(D_w ^ P) <= d.
@@ -1962,14 +1964,18 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
                 walk_init(c);
                 for (;;) {
                     bool fin;
-                    int qn = in.words >= 0
+                    const int qn = in.words >= 0
                                        ? word_run<kCount>(c, p.ctab + in.words, g0, g1, cs, ctr, base, exh, fin)
                                        : walk_run<kCount>(c, tab, g0, g1, cs, ctr, base, exh, fin);
                     uint32_t *queue = wsm[warp].subs + 64;
-                    if (in.triple_rows > 0 && qn >= kPairMin && in.n > 2)
-                        qn = pair_filter<kCount>(c, queue, qn);
-                    for (int i = 0; i < qn; ++i)
-                        expand_subset<kCount>(c, queue[i]);
+                    // the walk returns up to 63 nodes, the word filter 32
+                    for (int q0 = 0; q0 < qn; q0 += 32) {
+                        int k = min(32, qn - q0);
+                        if (in.triple_rows > 0 && k >= kPairMin && in.n > 2)
+                            k = pair_filter<kCount>(c, queue + q0, k);
+                        for (int i = 0; i < k; ++i)
+                            expand_subset<kCount>(c, queue[q0 + i]);
+                    }
                     __syncwarp();
                     if (fin)
                         break;

@@ -842,10 +842,10 @@ static double expected_seed_rows(int n, int m, int l, int d)
 //     words of a block that a window marks on average; S = n, or less where a
 //     block's strings run out sooner. With few blocks, one block's latency counts.
 //     Measured (estimated), us, by middle letters:
-//     5: (15,4) m = 600 199 (184), m = 1000 337 (349); (13,4) m = 600 174 (151);
+//     5: (15,4) m = 600 199 (184), m = 1000 337 (349); (13,4) m = 600 150 (151);
 //        (17,5) m = 1200 5429 (5470); (16,5) m = 600 1183 (1130)
-//     6: (17,5) m = 1200 4326 (4990); (15,4) m = 1200 392 (377); (16,4) 655 (690);
-//        (19,6) m = 1200 58900 (58000, the tree 110800)
+//     6: (17,5) m = 1200 4102 (4990); (15,4) m = 1200 392 (377); (16,4) 655 (690);
+//        (19,6) m = 1200 55600 (58000, the tree 110800)
 // `single`: the only instance of its launch.
 static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int q, bool single)
 {
