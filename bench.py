@@ -60,7 +60,7 @@ NCU_TRAFFIC = {
     "pms_kernels.cu": {"sha256": "74f437207a783ca1+69100b3a5b5aee1d",
                        "plain9_2": 1.099520e6, "plain15_4": 1.066240e6,
                        "plain17_5": 1.102336e6, "plain19_6": 1.618432e6},
-    "pms_sigma.cu": {"sha256": "f08996edcfffd0da+69100b3a5b5aee1d", "protein9_4": 4.6230528e7},
+    "pms_sigma_sieve.cu": {"sha256": ""},
 }
 
 def source_sha(name: str) -> str:
@@ -191,6 +191,17 @@ def n_ball(l: int, d: int, sigma: int = 4) -> int:
 
 
 # ------------------------------------------------------------------ CPU baseline (oracle)
+
+# comparisons of the sieve's rooflines: it marks balls and compares no l-mers, and the count
+# mode is the tree form's, so its work is stated as what the task cannot do without
+SIEVE_BASIS = "every seed with every other window, one comparison per tree node of a seed"
+SIEVE_LD = ((9, 2),)   # plain configurations that the library solves in the sieve form; quorums too
+
+
+def least_comparisons(n: int, m: int, l: int, d: int, q: int = 0) -> float:
+    W = m - l + 1
+    return W * (n - q + 1 if q else 1) * ((n - 1) * W + sum(math.comb(l, k) for k in range(d + 1)))
+
 
 def _oracle():
     import oracle
@@ -341,12 +352,13 @@ class Peaks:
         # 4 integer issue slots per comparison (2 LOP3, POPC, IMNMX) on 128 lanes per SM
         self.peak_int4 = self.sms * 128 * self.fmax / 4.0
 
-    def roofline(self, cmp_per_launch: float, ms: float, kernel: str, traffic, share: float) -> dict:
+    def roofline(self, cmp_per_launch: float, ms: float, kernel: str, traffic, share: float,
+                 basis: str = "the kernel's own comparisons (count mode)") -> dict:
         achieved = cmp_per_launch / (ms / 1000.0) if ms > 0 else float("nan")
         return {"bound": "alu", "achieved": achieved / 1e12, "peak": self.peak_popc / 1e12, "unit": "Tcmp/s",
                 "frac": achieved / self.peak_popc, "frac_popc": achieved / self.peak_popc,
                 "frac_int4": achieved / self.peak_int4, "peak_int4": self.peak_int4 / 1e12,
-                "traffic": traffic, "kernel": kernel, "cmp_per_launch": cmp_per_launch,
+                "traffic": traffic, "kernel": kernel, "cmp_per_launch": cmp_per_launch, "cmp_basis": basis,
                 "verify_ms_per_launch": ms,
                 "peak_basis": f"one POPC per comparison: {self.popc:.2f} POPC/clk/SM (measured probe) x {self.sms} "
                               f"SMs x {self.fmax/1e6:.0f} MHz (of measured); frac_int4 against {self.sms} SMs x "
@@ -442,6 +454,7 @@ def measure_plain(pms, torch, dev, stream, peaks, l, d, K, Wm, rank, dist, q: in
         tested += s["candidates_tested"]
     cctx.close()
     verify_avg_ms = statistics.mean(verify_ms)
+    sieve = bool(q) or (l, d) in SIEVE_LD
 
     # e2e through the host-buffer C-ABI call: the inputs cross from pinned host
     # memory (read there by the packing kernel) and the status block and codes
@@ -469,17 +482,20 @@ def measure_plain(pms, torch, dev, stream, peaks, l, d, K, Wm, rank, dist, q: in
         # the second pass over the same steps, graphs with the device-time events inside
         "kernel_timing_pass": {"ms_per_step": timed_step_ms, "verify_ms": statistics.mean(verify_ms),
                                "graph": "pms_options.graph = 1 (event nodes around each kernel)"},
-        # candidates generated and compared explicitly against occurrences (count mode)
-        "candidate_checks_per_s": tested_total / (total_ms / 1000.0),
-        "candidates_tested_per_step": tested / K,
+        "form": "sieve" if sieve else "tree",
+        # candidates generated and compared explicitly against occurrences (count mode; none in the sieve form)
+        "candidate_checks_per_s": None if sieve else tested_total / (total_ms / 1000.0),
+        "candidates_tested_per_step": None if sieve else tested / K,
         # the searched space W * |B(x, d)| per solve, for scale (not checks)
         "search_space_per_s": solves * W * (n - q + 1 if q else 1) * n_ball(l, d) / (total_ms / 1000.0),
-        "roofline": peaks.roofline(cmp_total / K, verify_avg_ms, "main_kernel (verification)",
-                                   measured_traffic("pms_kernels.cu", f"quorum{l}_{d}_q{q}" if q else f"plain{l}_{d}"),
+        "roofline": peaks.roofline(least_comparisons(n, m, l, d, q), verify_avg_ms, "sieve_kernel", None,
+                                   verify_avg_ms / timed_step_ms, SIEVE_BASIS) if sieve else
+                    peaks.roofline(cmp_total / K, verify_avg_ms, "main_kernel (verification)",
+                                   measured_traffic("pms_kernels.cu", f"plain{l}_{d}"),
                                    verify_avg_ms / timed_step_ms),
         "e2e": {"value": solves / (e2e_total / 1000.0), "unit": "solves/s", "h2d_bytes_per_step": n * m,
                 "d2h_bytes_per_step": 16 + 8 * e2e_codes / K, "ms_per_step": e2e_total / K},
-        "gpu_launches": 3 * K,   # packing + compatibility masks, verification, sort/unique
+        "gpu_launches": 3 * K,   # packing (+ compatibility masks), verification or sieve, sort/unique
     }
 
 
@@ -581,8 +597,8 @@ def bench_sigma(args, ws, rank, local, dist, l, d) -> dict:
                    "timing": "CUDA events on the library stream from the packing kernel to the sort kernel"},
         "candidate_checks_per_s": sum(tested) / (sum(kern_ms) / 1000.0),
         "search_space_per_s": solves * W * n_ball(l, d, 20) / (total_ms / 1000.0),
-        "roofline": peaks.roofline(statistics.mean(cmps), verify_avg, "sigma_main_kernel (search)",
-                                   measured_traffic("pms_sigma.cu", f"protein{l}_{d}"),
+        "roofline": peaks.roofline(statistics.mean(cmps), verify_avg, "sigma_sieve_kernel (search)",
+                                   measured_traffic("pms_sigma_sieve.cu", f"protein{l}_{d}"),
                                    verify_avg / (total_ms / K)),
         # up: the letters; down: the 112-byte counter block and the motifs' letters
         "e2e": {"value": solves / (e2e_total / 1000.0), "unit": "solves/s", "h2d_bytes_per_step": n * m,
@@ -632,12 +648,6 @@ def measure_batch(pms, torch, dev, peaks, args, rank, dist, steps: int = 3) -> d
             tk += ctx.stats()["ms_kernel"]
         one_wall.append(tw)
         one_kern.append(tk)
-    # verification-kernel work (count mode, untimed)
-    cctx = pms.Context(dev.index)
-    cctx.set_options(count_work=1)
-    cctx.solve_batch(batch)
-    cs = cctx.stats()
-    cctx.close()
     ctx.close()
     ok = all(not isinstance(r, Exception) for r in res)
     kern_ms = statistics.mean(kern)
@@ -657,12 +667,12 @@ def measure_batch(pms, torch, dev, peaks, args, rank, dist, steps: int = 3) -> d
                            "timing": "sum of the device times of 256 pms_solve calls",
                            "e2e_value": 256 / statistics.mean(one_wall)},
             "verify_ms": ver_ms, "share_verify": ver_ms / kern_ms,
-            "other_kernels_ms": kern_ms - ver_ms,   # packing, compatibility masks, sort/unique
+            "other_kernels_ms": kern_ms - ver_ms,   # packing, compatibility masks, sorts
             "graph_replays_after_timed_steps": replays,
-            "candidate_checks_per_s": cs["candidates_tested"] / (kern_ms / 1000.0),
-            "roofline": peaks.roofline(cs["cmp_reduce"] + cs["cmp_verify"], ver_ms, "main_kernel (verification)",
-                                       None, ver_ms / kern_ms),
-            "all_ok": ok, "autotune_s": t_tune, "gpu_launches": 4 * steps, "clocks": clk.summary()}
+            "roofline": peaks.roofline(sum(least_comparisons(i.n, i.m, i.l, i.d) for i in insts), ver_ms,
+                                       "sieve_kernel and main_kernel", None, ver_ms / kern_ms, SIEVE_BASIS),
+            # packing, masks, verification, the sieve with 4, 5 and 6 middle letters, the bucket sort's two, sort/unique
+            "all_ok": ok, "autotune_s": t_tune, "gpu_launches": 9 * steps, "clocks": clk.summary()}
 
 
 def measure_serve(pms, torch, dev, args, rank, dist, tune: bool = True) -> dict:
@@ -747,7 +757,7 @@ def measure_serve(pms, torch, dev, args, rank, dist, tune: bool = True) -> dict:
             "e2e": {"value": solves / span_max, "unit": "solves/s",
                     "h2d_bytes_per_step": int(statistics.mean(i.n * i.m for _, i in reqs)),
                     "d2h_bytes_per_step": 16 + 512 * 8},
-            "gpu_launches": 3 * count + int(st["serve_waves"]), "clocks": clk.summary()}
+            "gpu_launches": 2 * count + int(st["serve_waves"]), "clocks": clk.summary()}
 
 
 def bench_onehot(args, ws, rank, local, dist) -> dict:
