@@ -52,15 +52,14 @@ QUORUM_WORKLOADS = {"quorum15_4_q10": (15, 4, 10)}
 PROTEIN_WORKLOADS = {f"protein{l}_{d}": (l, d) for (l, d) in pi.PROTEIN_LD}
 L2_FLUSH_BYTES = 512 << 20
 
-# DRAM bytes (read + write) per launch of each search kernel from one-pass ncu
+# DRAM bytes (read + write) per launch of each search kernel from ncu
 # captures (dram__bytes_read.sum + dram__bytes_write.sum, profiles/*.md), valid
 # only for the sources they were taken on (sha256 prefix of the kernel file and
 # the shared header); otherwise the bench reports null.
 NCU_TRAFFIC = {
-    "pms_kernels.cu": {"sha256": "74f437207a783ca1+69100b3a5b5aee1d",
-                       "plain9_2": 1.099520e6, "plain15_4": 1.066240e6,
-                       "plain17_5": 1.102336e6, "plain19_6": 1.618432e6},
-    "pms_sigma_sieve.cu": {"sha256": ""},
+    "pms_kernels.cu": {"sha256": "d8a342c03baae39c+72e22c8f1ad63e07",
+                       "plain15_4": 1.076480e6, "plain17_5": 1.103104e6, "plain19_6": 1.375744e6},
+    "pms_sigma_sieve.cu": {"sha256": "2b5fcea7bedb5186+72e22c8f1ad63e07", "protein9_4": 4.10624e5},
 }
 
 def source_sha(name: str) -> str:
