@@ -884,27 +884,37 @@ cudaError_t launch_split(const SieveParams &p, int sms, int reserved, cudaStream
                          sv_smem_bytes<kMid, kSplitWarps>(reserved, kSplitWarps), st, 32 * kSplitWarps);
 }
 
+// The tables as they are uploaded. Made once, by whichever thread creates the first
+// context, and only read after that: contexts may be created by several threads at a
+// time, and an upload beside another context's running kernel writes the same bytes.
+struct SvTables {
+    SvTable t[4];
+    uint32_t ball[4][64][2] = {};
+    SvTables()
+    {
+        fill_table<3>(t[0]);
+        fill_table<4>(t[1]);
+        fill_table<5>(t[2]);
+        fill_table<6>(t[3]);
+        for (int v = 0; v < 4; ++v)
+            for (int s = 0; s < 64; ++s)
+                for (int u = 0; u < 64; ++u) {
+                    const int x = s ^ u, diff = (x | (x >> 3)) & 7;
+                    if ((diff & 1) + ((diff >> 1) & 1) + (diff >> 2) <= v)
+                        ball[v][s][u >> 5] |= 1u << (u & 31);
+                }
+    }
+};
+
 }  // namespace
 
 cudaError_t sieve_init_tables()
 {
-    static SvTable t[4];
-    fill_table<3>(t[0]);
-    fill_table<4>(t[1]);
-    fill_table<5>(t[2]);
-    fill_table<6>(t[3]);
-    uint32_t ball[4][64][2] = {};
-    for (int v = 0; v < 4; ++v)
-        for (int s = 0; s < 64; ++s)
-            for (int u = 0; u < 64; ++u) {
-                const int x = s ^ u, diff = (x | (x >> 3)) & 7;
-                if ((diff & 1) + ((diff >> 1) & 1) + (diff >> 2) <= v)
-                    ball[v][s][u >> 5] |= 1u << (u & 31);
-            }
-    const cudaError_t e = cudaMemcpyToSymbol(g_sv_table, t, sizeof t);
+    static const SvTables tables;
+    const cudaError_t e = cudaMemcpyToSymbol(g_sv_table, tables.t, sizeof tables.t);
     if (e != cudaSuccess)
         return e;
-    return cudaMemcpyToSymbol(g_sv_ball, ball, sizeof ball);
+    return cudaMemcpyToSymbol(g_sv_ball, tables.ball, sizeof tables.ball);
 }
 
 cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, int sms, cudaStream_t st)
