@@ -748,7 +748,10 @@ __global__ void __launch_bounds__(32 * kSplitWarps, kMinBlocks) sieve_split_kern
 #pragma unroll
         for (int k = 0; k < kPieces; ++k)
             cur[k] = kFull;
-        for (int i = warp; i < in.n && !*(volatile int *)dead; i += kSplitWarps) {
+        for (int i = warp; i < in.n; i += kSplitWarps) {
+            // another warp may set the flag at any time: the lanes decide together, as the marks need them all
+            if (__any_sync(kFull, *(volatile int *)dead))
+                break;
             sv_mark<kMid, 1>(blk.win + (size_t)i * in.W, in.W, in.d, blk.prefix, marks, sm.list[warp], sm, my, 0,
                              lane);
             __syncwarp();

@@ -88,3 +88,14 @@ def test_large_answers_sorted_by_buckets(case):
         s = st.cpu().numpy().astype(np.uint32)
         assert s[1] == len(want) and s[2] == 2
         assert np.array_equal(out[:1000].cpu().numpy().astype(np.uint64), want[:1000]) and not out[1000:].any()
+
+
+@pytest.mark.parametrize("case", [(45, 300, 9, 1), (64, 120, 10, 2), (50, 500, 11, 2)], ids=str)
+def test_blocks_that_end_in_any_warp(oracle_, case):
+    """A CTA per block, a sequence per warp: blocks that run out of strings in different warps, often."""
+    n, m, l, d = case
+    seqs = pi.planted_instance(n, m, l, d, 17).seqs
+    want = oracle_.solve_packed(seqs, l, d)
+    with pms.Context(0) as c:
+        for _ in range(20):
+            assert np.array_equal(c.solve(seqs, l, d), want)
