@@ -959,7 +959,12 @@ static void plan_sieve(Plan &P, const std::vector<SieveForm> &form)
 
 // Expected motifs from which an answer is sorted by buckets: (13,4), n = 20,
 // m = 1000, 5300 of them, solve 412 -> 330 us; below about a thousand the
-// one-CTA sort takes no longer than two more launches.
+// one-CTA sort takes no longer than two more launches. At most kMaxBucketed
+// instances of a launch have buckets: so many answers keep every SM busy with a
+// CTA each, and a grid's second dimension holds 65535 CTAs. Nor has one whose
+// buckets (48 KB) take more memory than the masks that the tree form would hold
+// for it, so that a memory budget goes as far as in that form.
+constexpr size_t kMaxBucketed = 4096;
 constexpr double kBucketMotifs = 1024;
 
 static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
@@ -991,14 +996,15 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
         in.q = (h->opt.quorum > 0 && h->opt.quorum < s.n) ? h->opt.quorum : s.n;
         in.nseed = s.n - in.q + 1;
         in.sieve_mid = form[k].mid;
+        const long long seeds = (long long)in.nseed * in.W;
         // answers of chance motifs, which one CTA would sort for long
         in.buckets = -1;
-        if (in.sieve_mid > 0 && form[k].motifs >= kBucketMotifs) {
+        if (in.sieve_mid > 0 && form[k].motifs >= kBucketMotifs && P.bucketed.size() < kMaxBucketed &&
+            (size_t)seeds * (s.n - 1) * (in.NW + 1) >= kBucketWords) {
             in.buckets = (int)(P.bucketed.size() * kBucketWords);
             P.bucketed.push_back((int)k);
         }
         const bool tree = in.sieve_mid == 0;
-        const long long seeds = (long long)in.nseed * in.W;
         const int cw = h->chunk_work_for(s.n, s.m, s.l, s.d);
         in.grab = h->grab_for(s.n, s.m, s.l, s.d);
         const WordTable &wt = h->words(s.l, s.d, tree && in.grab == 1 && in.q == in.n,

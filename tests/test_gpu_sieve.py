@@ -99,3 +99,18 @@ def test_blocks_that_end_in_any_warp(oracle_, case):
     with pms.Context(0) as c:
         for _ in range(20):
             assert np.array_equal(c.solve(seqs, l, d), want)
+
+
+# the first: more dense instances than a grid has rows; the second: more than have buckets in one launch
+@pytest.mark.parametrize("case", [(66000, 2, 40, 6, 2, 8192), (4200, 3, 456, 7, 2, 131072)], ids=str)
+def test_batch_of_many_dense_instances(oracle_, case):
+    """Batches whose instances have thousands of motifs each; 33 different instances among them."""
+    count, n, m, l, d, cap = case
+    kinds = [pi.random_sequences(n, m, 500 + k) for k in range(33)]
+    want = [oracle_.solve_packed(s, l, d) for s in kinds]
+    assert min(len(w) for w in want) > 1000
+    with pms.Context(0) as c:
+        c.set_options(max_motifs=cap)
+        got = c.solve_batch([(kinds[k % 33], l, d) for k in range(count)])
+    assert len(got) == count
+    assert all(np.array_equal(g, want[k % 33]) for k, g in enumerate(got))
