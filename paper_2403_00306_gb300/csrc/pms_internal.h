@@ -26,6 +26,9 @@ constexpr int kRowSmemCapSmall = 1280;  // the same in the 4-CTAs-per-SM form of
 // Flags reported per instance.
 constexpr uint32_t kFlagInvalidByte = 1u;
 constexpr uint32_t kFlagOverflow = 2u;
+// Between kernels only, never in a status:
+constexpr uint32_t kFlagSkewed = 1u << 30;   // a large answer that the sort kernel sorts after all (bucket_scatter_kernel)
+constexpr uint32_t kFlagInternal = kFlagSkewed;
 
 // One instance as the kernels see it. Offsets index the arenas below.
 struct InstDev {
@@ -155,9 +158,10 @@ cudaError_t launch_sort_unique(const InstDev *inst, const int *inst_list, int nl
                                uint64_t *dense, uint32_t dense_cap, uint32_t *dense_total,
                                const uint32_t *key_count, cudaStream_t st);
 // Sorts the keys of the listed instances (in sieve form, with buckets) in raw:
-// scattered by bucket to tmp, then each bucket's keys by rank.
+// scattered by bucket to tmp, then each bucket's keys by rank; those with too full
+// a bucket are left to the sort kernel (kFlagSkewed).
 cudaError_t launch_bucket_sort(const InstDev *inst, const int *list, int nlist, uint64_t *raw, uint64_t *tmp,
-                               const uint32_t *key_count, uint32_t *buckets, cudaStream_t st);
+                               const uint32_t *key_count, uint32_t *buckets, uint32_t *flags, cudaStream_t st);
 cudaError_t init_tables();
 // Host handles of the pack and sort/unique kernels (to find their nodes in a captured graph).
 const void *pack_kernel_fn();

@@ -2863,12 +2863,12 @@ __global__ void __launch_bounds__(kSortThreads)
     const uint32_t nk = in.sieve_mid ? key_count[I] : rc;
     const uint32_t n = nk < in.raw_cap ? nk : in.raw_cap;
     uint64_t *a = raw + in.raw_off;
-    if (in.sieve_mid && in.buckets >= 0) {
+    if (in.sieve_mid && in.buckets >= 0 && !(flags[I] & kFlagSkewed)) {
         // sorted and without duplicates already
         if (threadIdx.x == 0) {
             const uint32_t base = atomicAdd(dense_total, n);
             s_base = base;
-            uint32_t f = flags[I];
+            uint32_t f = flags[I] & ~kFlagInternal;
             if (rc > in.raw_cap || base + n > dense_cap)
                 f |= kFlagOverflow;
             status[I] = StatusDev{rc, n, f, base};
@@ -2926,7 +2926,7 @@ __global__ void __launch_bounds__(kSortThreads)
         const uint32_t base = atomicAdd(dense_total, s_total);
         s_base = base;
         s_run = 0;
-        uint32_t f = flags[I];
+        uint32_t f = flags[I] & ~kFlagInternal;
         if (rc > in.raw_cap || base + s_total > dense_cap)
             f |= kFlagOverflow;
         status[I] = StatusDev{rc, s_total, f, base};
@@ -2952,13 +2952,23 @@ __global__ void __launch_bounds__(kSortThreads)
 // batch (up to 600 k keys each).
 // Scatter: gridDim.x CTAs per instance; each scans the instance's counts for
 // the buckets' first places (CTA 0 stores them) and places its share of the keys.
+// A bucket is ranked by one warp, key by key: 0.8 ns times its keys squared (largest
+// bucket 7,491: 42.6 ms). Where letters are far from uniform the motifs crowd into few
+// buckets, and the radix sort, 9 ns a key whatever they are, ends sooner once the largest
+// bucket's square exceeds about 11 times the keys. Sorting, ms, by buckets and by radix:
+// (13,4), n = 20, m = 1000, letters drawn 0.25 each 0.019 and 0.103 (5,714 keys);
+// 0.35/0.15/0.15/0.35 42.6 and 27.9 (3.0 M keys, square 18.6 times them); 0.8/0.1/0.05/0.05
+// 169 and 22.3 (2.5 M, 85 times); (11,3), n = 12, m = 700, 0.8/0.1/0.05/0.05 0.82 and
+// 1.16 (158 k, 6.6 times); (14,4), n = 6, m = 900, the same letters 1785 and 46 (5.1 M, 426 times).
 constexpr int kBucketThreads = 256;
+constexpr unsigned long long kBucketSkew = 10;
 __global__ void __launch_bounds__(kBucketThreads)
     bucket_scatter_kernel(const InstDev *__restrict__ inst, const int *__restrict__ list, const uint64_t *__restrict__ raw,
-                          uint64_t *__restrict__ tmp, const uint32_t *__restrict__ key_count, uint32_t *buckets)
+                          uint64_t *__restrict__ tmp, const uint32_t *__restrict__ key_count, uint32_t *buckets,
+                          uint32_t *flags)
 {
     __shared__ uint32_t first[kBuckets];
-    __shared__ uint32_t warp_tot[32], total;
+    __shared__ uint32_t warp_tot[32], total, most;
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int I = list[blockIdx.y];
@@ -2966,7 +2976,9 @@ __global__ void __launch_bounds__(kBucketThreads)
     const uint32_t n = min(key_count[I], in.raw_cap);
     uint32_t *count = buckets + in.buckets, *placed = count + kBuckets, *start = placed + kBuckets;
     constexpr int kPer = kBuckets / kBucketThreads;
-    uint32_t v[kPer], sum = 0;
+    uint32_t v[kPer], sum = 0, full = 0;
+    if (threadIdx.x == 0)
+        most = 0;
 #pragma unroll
     for (int u = 0; u < kPer / 4; ++u) {
         const uint4 q = reinterpret_cast<const uint4 *>(count)[threadIdx.x * (kPer / 4) + u];
@@ -2975,14 +2987,23 @@ __global__ void __launch_bounds__(kBucketThreads)
         v[4 * u + 2] = q.z;
         v[4 * u + 3] = q.w;
         sum += q.x + q.y + q.z + q.w;
+        full = max(max(full, max(q.x, q.y)), max(q.z, q.w));
     }
     uint32_t at = block_exclusive_scan(sum, warp_tot, &total);
+    full = __reduce_max_sync(kFull, full);
+    if ((threadIdx.x & 31) == 0)
+        atomicMax(&most, full);
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
         first[threadIdx.x * kPer + u] = at;
         at += v[u];
     }
     __syncthreads();
+    if ((unsigned long long)most * most > kBucketSkew * n) {
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            atomicOr(&flags[I], kFlagSkewed);
+        return;
+    }
     if (blockIdx.x == 0)
         for (int b = threadIdx.x; b < kBuckets; b += kBucketThreads)
             start[b] = first[b];
@@ -2994,13 +3015,16 @@ __global__ void __launch_bounds__(kBucketThreads)
 }
 
 // Rank: a warp per bucket; a key's place is the number of smaller ones (all
-// keys differ). Chance answers hold a few dozen keys a bucket.
+// keys differ). Answers over uniform letters hold a few to a few hundred keys a bucket.
 __global__ void __launch_bounds__(kBucketThreads)
     bucket_rank_kernel(const InstDev *__restrict__ inst, const int *__restrict__ list, uint64_t *__restrict__ raw,
-                       const uint64_t *__restrict__ tmp, const uint32_t *__restrict__ buckets)
+                       const uint64_t *__restrict__ tmp, const uint32_t *__restrict__ buckets,
+                       const uint32_t *__restrict__ flags)
 {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (flags[list[blockIdx.y]] & kFlagSkewed)
+        return;
     const InstDev in = inst[list[blockIdx.y]];
     const uint32_t *count = buckets + in.buckets, *start = count + 2 * kBuckets;
     const int lane = threadIdx.x & 31;
@@ -3248,7 +3272,7 @@ cudaError_t launch_sort_unique(const InstDev *inst, const int *inst_list, int nl
 }
 
 cudaError_t launch_bucket_sort(const InstDev *inst, const int *list, int nlist, uint64_t *raw, uint64_t *tmp,
-                               const uint32_t *key_count, uint32_t *buckets, cudaStream_t st)
+                               const uint32_t *key_count, uint32_t *buckets, uint32_t *flags, cudaStream_t st)
 {
     // CTAs per instance: enough for one answer alone, few each for many
     const int scatter = nlist >= 64 ? 4 : 32, rank = nlist >= 64 ? 32 : 512;
@@ -3256,12 +3280,12 @@ cudaError_t launch_bucket_sort(const InstDev *inst, const int *list, int nlist, 
     cudaLaunchConfig_t cfg = dependent_launch(attr, scatter, kBucketThreads, 0, st);
     cfg.gridDim.y = (unsigned)nlist;
     cudaError_t e = cudaLaunchKernelEx(&cfg, bucket_scatter_kernel, inst, list, (const uint64_t *)raw, tmp, key_count,
-                                       buckets);
+                                       buckets, flags);
     if (e != cudaSuccess)
         return e;
     cfg.gridDim.x = (unsigned)rank;
     return cudaLaunchKernelEx(&cfg, bucket_rank_kernel, inst, list, raw, (const uint64_t *)tmp,
-                              (const uint32_t *)buckets);
+                              (const uint32_t *)buckets, (const uint32_t *)flags);
 }
 
 cudaError_t launch_probe(int kind, int iters, int blocks, unsigned long long *cycles, unsigned long long *sink,

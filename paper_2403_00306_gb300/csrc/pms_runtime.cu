@@ -1255,7 +1255,7 @@ static int enqueue_plan(pms_ctx *h, const Plan &P, const uint8_t *d_seq_src, Sta
     if (!P.bucketed.empty() &&
         (e = launch_bucket_sort(d_inst, (const int *)(dm + ml.bucketed), (int)P.bucketed.size(), (uint64_t *)h->d_raw.p,
                                 (uint64_t *)h->d_tmp.p, (const uint32_t *)(dc + cl.key_count),
-                                (uint32_t *)(dc + cl.buckets), st)) != cudaSuccess)
+                                (uint32_t *)(dc + cl.buckets), d_flags, st)) != cudaSuccess)
         return h->cuda_fail(e, "bucket sort kernels");
     if ((e = launch_sort_unique(d_inst, nullptr, (int)k, (uint64_t *)h->d_raw.p, (uint64_t *)h->d_tmp.p, d_rawcnt,
                                 d_flags, status_out,

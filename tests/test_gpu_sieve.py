@@ -114,3 +114,48 @@ def test_batch_of_many_dense_instances(oracle_, case):
         got = c.solve_batch([(kinds[k % 33], l, d) for k in range(count)])
     assert len(got) == count
     assert all(np.array_equal(g, want[k % 33]) for k, g in enumerate(got))
+
+
+def _skewed(n, m, p, seed):
+    """Sequences whose letters are drawn with the probabilities p."""
+    return np.frombuffer(b"ACGT", dtype=np.uint8)[np.random.default_rng(seed).choice(4, size=(n, m), p=p)]
+
+
+# letters far from uniform: the motifs crowd into few buckets. The first answer's largest bucket is
+# within what is ranked bucket by bucket, the second's is not
+@pytest.mark.parametrize("p", [(0.8, 0.1, 0.05, 0.05), (0.955, 0.015, 0.015, 0.015)], ids=str)
+def test_skewed_letters_match_oracle(oracle_, p):
+    seqs = _skewed(12, 700, p, 5)
+    want = oracle_.solve_packed(seqs, 11, 3, cap=1 << 26)
+    assert len(want) > 8192
+    with pms.Context(0) as c:
+        for _ in range(3):   # kernel by kernel, captured, replayed
+            assert np.array_equal(c.solve(seqs, 11, 3), want)
+        for got in c.solve_batch([(seqs, 11, 3)] * 3):
+            assert np.array_equal(got, want)
+
+
+def test_skewed_letters_in_a_large_answer():
+    """Five million motifs, 46,000 of them in the fullest bucket (one warp would rank it for 1.8 s); the
+    answer is in order, and strings near the sequences are in it exactly if every sequence has them."""
+    seqs = _skewed(6, 900, (0.8, 0.1, 0.05, 0.05), 5)
+    l, d = 14, 4
+    with pms.Context(0) as c:
+        c.set_options(graph=-1)
+        got = c.solve(seqs, l, d)
+        assert c.stats()["ms_kernel"] < 400
+    assert len(got) > 1 << 22 and np.all(got[1:] > got[:-1])
+    code = np.searchsorted(np.frombuffer(b"ACGT", dtype=np.uint8), seqs)
+    windows = np.lib.stride_tricks.sliding_window_view(code, l, axis=1)
+    place = 4 ** np.arange(l - 1, -1, -1)
+    rng, inside = np.random.default_rng(6), 0
+    for _ in range(2000):
+        s = windows[rng.integers(6), rng.integers(windows.shape[1])].copy()
+        at = rng.permutation(l)[:rng.integers(d + 3)]
+        s[at] = rng.integers(0, 4, len(at))
+        want = bool(((windows != s).sum(axis=2) <= d).any(axis=1).all())
+        key = np.uint64(s @ place)
+        i = np.searchsorted(got, key)
+        assert (i < len(got) and got[i] == key) == want
+        inside += want
+    assert 100 < inside < 1900
