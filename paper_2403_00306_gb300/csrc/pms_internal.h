@@ -28,7 +28,8 @@ constexpr uint32_t kFlagInvalidByte = 1u;
 constexpr uint32_t kFlagOverflow = 2u;
 // Between kernels only, never in a status:
 constexpr uint32_t kFlagSkewed = 1u << 30;   // a large answer that the sort kernel sorts after all (bucket_scatter_kernel)
-constexpr uint32_t kFlagInternal = kFlagSkewed;
+constexpr uint32_t kFlagRawBeyond = 1u << 31;   // sieve form: the raw count does not fit 32 bits
+constexpr uint32_t kFlagInternal = kFlagSkewed | kFlagRawBeyond;
 
 // One instance as the kernels see it. Offsets index the arenas below.
 struct InstDev {
@@ -219,6 +220,7 @@ struct SieveParams {
     const uint2 *planes;          // instance plane_off: its window words
     uint64_t *raw;
     uint32_t *raw_count;          // per instance: motifs, once per seed window near them
+    uint32_t *flags;              // per instance: kFlagRawBeyond
     uint32_t *key_count;          // per instance: keys in raw (every motif once)
     uint32_t *buckets;            // instance buckets: keys per bucket (see bucket_of)
 };

@@ -2859,9 +2859,10 @@ __global__ void __launch_bounds__(kSortThreads)
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the producing kernel has completed
     const int I = inst_list ? inst_list[blockIdx.x] : (int)blockIdx.x;
     const InstDev in = inst[I];
-    const uint32_t rc = raw_count[I];
+    const uint32_t rc = (flags[I] & kFlagRawBeyond) ? 0xffffffffu : raw_count[I];
     const uint32_t nk = in.sieve_mid ? key_count[I] : rc;
     const uint32_t n = nk < in.raw_cap ? nk : in.raw_cap;
+    const bool over = rc > in.raw_cap || nk > in.raw_cap;
     uint64_t *a = raw + in.raw_off;
     if (in.sieve_mid && in.buckets >= 0 && !(flags[I] & kFlagSkewed)) {
         // sorted and without duplicates already
@@ -2869,7 +2870,7 @@ __global__ void __launch_bounds__(kSortThreads)
             const uint32_t base = atomicAdd(dense_total, n);
             s_base = base;
             uint32_t f = flags[I] & ~kFlagInternal;
-            if (rc > in.raw_cap || base + n > dense_cap)
+            if (over || base + n > dense_cap)
                 f |= kFlagOverflow;
             status[I] = StatusDev{rc, n, f, base};
         }
@@ -2927,7 +2928,7 @@ __global__ void __launch_bounds__(kSortThreads)
         s_base = base;
         s_run = 0;
         uint32_t f = flags[I] & ~kFlagInternal;
-        if (rc > in.raw_cap || base + s_total > dense_cap)
+        if (over || base + s_total > dense_cap)
             f |= kFlagOverflow;
         status[I] = StatusDev{rc, s_total, f, base};
     }

@@ -1230,6 +1230,7 @@ static int enqueue_plan(pms_ctx *h, const Plan &P, const uint8_t *d_seq_src, Sta
         sp.planes = mp.planes;
         sp.raw = mp.raw;
         sp.raw_count = d_rawcnt;
+        sp.flags = d_flags;
         sp.key_count = (uint32_t *)(dc + cl.key_count);
         sp.buckets = (uint32_t *)(dc + cl.buckets);
         if ((e = launch_sieve(sp, L.mid, L.planes, L.share, h->num_sms, st)) != cudaSuccess)
@@ -1667,14 +1668,20 @@ static int solve_specs(pms_ctx *h, std::vector<InstSpec> specs, std::vector<Inst
         for (size_t j = 0; j < sub.size(); ++j) {
             const int idx = todo[j];
             const uint32_t cap = P.inst[j].raw_cap;
-            const bool overflow = sd[j].raw_count > cap;
-            if (overflow && !(sd[j].flags & kFlagInvalidByte) && !h->opt.max_motifs && cap < (1u << 26)) {
-                specs[idx].raw_cap = pow2_at_least(std::max<size_t>((size_t)cap * 8, (size_t)sd[j].raw_count * 2));
+            const bool overflow = sd[j].raw_count > cap, invalid = sd[j].flags & kFlagInvalidByte;
+            // the sieve stores a motif once, however often it counts: its answer is whole
+            // while the buffer has room left, or has room for every string
+            const bool sieve = P.inst[j].sieve_mid > 0;
+            const size_t strings = sieve ? (size_t)1 << (2 * sub[j].l) : 0;
+            const bool whole = sieve && !h->opt.max_motifs && (sd[j].unique_count < cap || cap >= strings);
+            if (overflow && !whole && !invalid && !h->opt.max_motifs && cap < (1u << 26)) {
+                const size_t want = std::max<size_t>((size_t)cap * 8, (size_t)sd[j].raw_count * 2);
+                specs[idx].raw_cap = pow2_at_least(sieve ? std::min(want, strings) : want);
                 again.push_back(idx);
                 continue;
             }
             InstOut &o = out[idx];
-            o.status = status_code(sd[j]);
+            o.status = whole && !invalid ? PMS_OK : status_code(sd[j]);
             o.raw_count = sd[j].raw_count;
             o.codes.assign(dense + sd[j].dense_off, dense + sd[j].dense_off + sd[j].unique_count);
         }
@@ -2367,6 +2374,7 @@ static void served_loop(Served *S)
                     sp.planes = mp.planes;
                     sp.raw = mp.raw;
                     sp.raw_count = mp.raw_count;
+                    sp.flags = mp.flags;
                     sp.key_count = srv_keycnt(S);
                     // a launch with few blocks gives each a CTA
                     const bool few = sp.total < 16ll * h->num_sms;

@@ -151,7 +151,7 @@ struct SvMark {
 };
 struct SvCount {
     static constexpr bool kCount = true;
-    uint32_t found = 0;
+    unsigned long long found = 0;
     // once: not a lane that repeats another's change
     __device__ __forceinline__ void operator()(uint32_t addr, uint32_t bits, bool once = true)
     {
@@ -321,18 +321,37 @@ __device__ __forceinline__ void sv_mark(const uint2 *__restrict__ win, int W, in
 // 82; 256 mixed instances, some of 600 k motifs, 34.6 and 25.1 ms.
 constexpr int kSvCountFrom = 32;
 
+// Where an instance's motifs go.
+struct SvOut {
+    uint64_t *raw;
+    uint32_t *raw_count, *key_count, *buckets, *flags;
+};
+
+// Adds to an instance's raw count (one lane). The count has 32 bits, and dense
+// answers over long sequences exceed them: the flag says so from then on.
+__device__ __forceinline__ void sv_raw_add(SvOut out, unsigned long long v)
+{
+    const uint32_t add = (uint32_t)min(v, 0xffffffffull);
+    const uint32_t was = atomicAdd(out.raw_count, add);
+    if (add != v || was + add < was)
+        atomicOr(out.flags, kFlagRawBeyond);
+}
+
 // Adds the windows of win[0..W) within d of each string marked in the block,
 // summed over the strings, to the raw count; kShare warps take part.
 template <int kMid, int kShare, class Smem>
 __device__ __noinline__ void sv_count(const uint2 *__restrict__ win, int W, int d, uint32_t prefix, uint32_t marks,
-                                      uint32_t *list, const Smem &sm, uint32_t *raw_count, int g, int lane)
+                                      uint32_t *list, const Smem &sm, SvOut out, int g, int lane)
 {
     SvCount op;
     const SvLane<kMid> my(sm, lane);
     sv_pass<kMid, kShare>(op, win, W, d, prefix, marks, list, sm, my, g, lane);
-    const uint32_t all = __reduce_add_sync(kFull, op.found);
-    if (lane == 0 && all != 0u)
-        atomicAdd(raw_count, all);
+    unsigned long long all = op.found;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        all += __shfl_xor_sync(kFull, all, o);
+    if (lane == 0 && all != 0ull)
+        sv_raw_add(out, all);
 }
 
 // Does a window of the sequence lie within d of the string c? Warp-uniform.
@@ -351,12 +370,6 @@ __device__ __forceinline__ bool sv_occurs(const uint2 *__restrict__ win, int W, 
     }
     return false;
 }
-
-// Where an instance's motifs go.
-struct SvOut {
-    uint64_t *raw;
-    uint32_t *raw_count, *key_count, *buckets;
-};
 
 // Up to 32 strings, one per lane (`has`): those that occur in the sequences
 // first..n-1 too are appended to the keys. The raw count grows by the windows of
@@ -397,7 +410,7 @@ __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, SvOut out
     uint32_t base = 0;
     if (lane == 0) {
         if (!counted)
-            atomicAdd(out.raw_count, (uint32_t)all);
+            sv_raw_add(out, (unsigned long long)all);
         base = atomicAdd(out.key_count, (uint32_t)__popc(found));
     }
     base = __shfl_sync(kFull, base, 0) + (uint32_t)__popc(found & ((1u << lane) - 1u));
@@ -417,7 +430,7 @@ __device__ __noinline__ void sv_emit(const InstDev *__restrict__ inst, SvOut out
 
 __device__ __forceinline__ SvOut out_of(const SieveParams &p, int I)
 {
-    return SvOut{p.raw, p.raw_count + I, p.key_count + I, p.buckets};
+    return SvOut{p.raw, p.raw_count + I, p.key_count + I, p.buckets, p.flags + I};
 }
 
 // The string of bit `bit` of mark word `at` ([half][word]) of a block.
@@ -683,7 +696,7 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
         if (counted) {   // the windows of s_1..s_{n-q+1} are contiguous
             share_sync<kShare>();
             sv_count<kMid, kShare>(blk.win, in.nseed * in.W, in.d, blk.prefix, marks, sm.list[warp], sm,
-                                   p.raw_count + blk.I, g, lane);
+                                   out_of(p, blk.I), g, lane);
             share_sync<kShare>();
         }
         // the strings of a warp's threads, the pieces of one thread at a time
@@ -788,7 +801,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps, kMinBlocks) sieve_split_kern
             const bool counted = *(volatile int *)&sm.alive[1] >= kSvCountFrom;
             if (counted) {
                 sv_count<kMid, kSplitWarps>(blk.win, in.nseed * in.W, in.d, blk.prefix, marks0, sm.list[warp], sm,
-                                            p.raw_count + blk.I, warp, lane);
+                                            out_of(p, blk.I), warp, lane);
             }
             for (int at = warp * 32 + lane; at < 2 * M::kWords; at += 32 * kSplitWarps) {
                 uint32_t v = all[at];

@@ -159,3 +159,23 @@ def test_skewed_letters_in_a_large_answer():
         assert (i < len(got) and got[i] == key) == want
         inside += want
     assert 100 < inside < 1900
+
+
+def test_raw_count_beyond_32_bits():
+    """Every one of the 4^10 strings is a motif, and each is near some 4,100 of the 52,428 seed windows:
+    the raw count is 52428 |B(10,5)| = 2^32 + 39320."""
+    import torch
+    n, m, l, d = 2, 52437, 10, 5
+    seqs = pi.random_sequences(n, m, 8)
+    with pms.Context(0) as c:
+        assert np.array_equal(c.solve(seqs, l, d), np.arange(4 ** l, dtype=np.uint64))
+        out = torch.zeros(4 ** l, dtype=torch.int64, device="cuda")
+        st = torch.zeros(4, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        c.solve_device(torch.from_numpy(seqs.copy()).cuda(), n, m, l, d, out, 4 ** l, st)
+        torch.cuda.synchronize()
+        assert list(st.cpu().numpy().astype(np.uint32)[:3]) == [0xffffffff, 4 ** l, 2]
+        c.set_options(max_motifs=1 << 16)   # above what the count's low 32 bits say
+        with pytest.raises(pms.PMSError) as e:
+            c.solve(seqs, l, d)
+        assert e.value.code == pms.PMS_ETOOMANY
