@@ -204,9 +204,9 @@ inline cudaLaunchConfig_t dependent_launch(cudaLaunchAttribute *attr, int blocks
 
 // ---------------------------------------------------------------- the sieve form (pms_sieve.cu)
 
-// The blocks of one instance in a sieve launch, from global item work_lo on.
+// Blocks of one instance in a sieve launch: from block block_lo on, as global items from work_lo on.
 struct SieveSeg {
-    long long work_lo;
+    long long work_lo, block_lo;
     int inst;
     int pad;
 };

@@ -950,7 +950,7 @@ static void plan_sieve(Plan &P, const std::vector<SieveForm> &form)
         });
         Plan::SieveLaunch L{f[0], f[1], form[list[0]].share, P.sieve_seg.size(), (int)list.size(), 0};
         for (int k : list) {
-            P.sieve_seg.push_back(SieveSeg{L.total, k, 0});
+            P.sieve_seg.push_back(SieveSeg{L.total, 0, k, 0});
             L.total += 1ll << (2 * (P.inst[k].l - f[0] - kSvSuf));
         }
         P.sieve.push_back(L);
@@ -1833,7 +1833,7 @@ struct Request {
     size_t dense_rel = 0, status_rel = 0;   // offsets in the arena
     long long chunks_total = 0, chunks_next = 0;
     double units_per_chunk = 1.0;
-    SieveForm form;                // mid > 0: sieve form, run whole by one wave
+    SieveForm form;                // mid > 0: sieve form, its chunks are blocks
     cudaEvent_t done_ev = nullptr;
     int status = PMS_OK;
     std::vector<uint64_t> codes;
@@ -2138,8 +2138,8 @@ static bool served_admit(Served *S, Request *r)
         units += (double)binom(r->l, i) * (std::pow(3.0, i) + kNodeUnits);
     r->units_per_chunk = std::max(1.0, units / ct.cps);
     if (!tree) {
-        r->chunks_total = 1;
-        r->units_per_chunk = r->form.us * kUnitsPerUs;
+        r->chunks_total = 1ll << (2 * (r->l - r->form.mid - kSvSuf));   // blocks
+        r->units_per_chunk = std::max(1e-3, r->form.us * kUnitsPerUs / (double)r->chunks_total);
     }
     InstDev &in = S->h_inst[r->slot];
     in = InstDev{};
@@ -2273,17 +2273,21 @@ static void served_loop(Served *S)
                 if (units >= wave_units || (int)reqs >= S->slots)
                     break;
                 ++reqs;
-                if (r->form.mid > 0) {
+                const bool sieve = r->form.mid > 0;
+                long long take = (long long)std::ceil((wave_units - units) / r->units_per_chunk);
+                // a sieve's share of a wave keeps every SM busy
+                take = std::max<long long>(sieve ? 16ll * h->num_sms : 1, take);
+                take = std::min(take, r->chunks_total - r->chunks_next);
+                if (sieve) {
                     const int j = r->form.mid - 3;
-                    sieve_segs[j].push_back(SieveSeg{sieve_blocks[j], r->slot, 0});
-                    sieve_blocks[j] += 1ll << (2 * (r->l - r->form.mid - kSvSuf));
-                    r->chunks_next = r->chunks_total;
-                    units += r->units_per_chunk;
-                    finishing.push_back(r);
+                    sieve_segs[j].push_back(SieveSeg{sieve_blocks[j], r->chunks_next, r->slot, 0});
+                    sieve_blocks[j] += take;
+                    r->chunks_next += take;
+                    units += take * r->units_per_chunk;
+                    if (r->chunks_next >= r->chunks_total)
+                        finishing.push_back(r);
                     continue;
                 }
-                long long take = (long long)std::ceil((wave_units - units) / r->units_per_chunk);
-                take = std::max<long long>(1, std::min(take, r->chunks_total - r->chunks_next));
                 segs.push_back(Segment{items, r->slot, (int)r->chunks_next, (int)(r->chunks_next + take), 0});
                 r->chunks_next += take;
                 items += take;

@@ -519,7 +519,8 @@ struct SvBlock {
         }
         I = p.seg[lo].inst;
         in = p.inst[I];
-        const uint32_t b = (uint32_t)(it - p.seg[lo].work_lo);   // the prefix letters' planes, hi above lo
+        // the prefix letters' planes, hi above lo
+        const uint32_t b = (uint32_t)(it - p.seg[lo].work_lo + p.seg[lo].block_lo);
         const int A = in.l - mid_letters - kSvSuf;
         prefix = (b & ((1u << A) - 1u)) | ((b >> A) << 16);
         win = p.planes + in.plane_off;

@@ -88,3 +88,21 @@ def test_memory_budget_enforced():
         c.solve(inst.seqs, 15, 4)
     assert e.value.code == pms.PMS_ENOMEM
     c.close()
+
+
+def test_served_sieve_requests_are_divided():
+    """Requests whose strings are sieved in blocks give way to others like those searched seed by seed:
+    with short waves a heavy one takes many, and small ones among them share those."""
+    heavy = [pi.planted_instance(20, 1200, 17, 5, 3), pi.planted_instance(20, 1200, 15, 4, 4)]
+    small = [pi.planted_instance(20, 300 + 17 * k, 13, 4, 50 + k) for k in range(6)]
+    reqs = small[:3] + heavy + small[3:]
+    with pms.Context(0) as plain, pms.Context(0) as ctx:
+        alone = [plain.solve(r.seqs, r.l, r.d) for r in reqs]
+        ctx.set_options(serve_wave_items=1)
+        for _ in range(2):
+            tickets = [ctx.submit(r.seqs, r.l, r.d) for r in reqs]
+            for r, t, want in zip(reqs, tickets, alone):
+                assert np.array_equal(ctx.wait(t, 60000), want), (r.l, r.d, r.m)
+                ctx.release(t)
+        # 65,536 blocks of (17,5), a wave's share being those of 16 warps a multiprocessor
+        assert ctx.stats()["serve_waves"] >= 2 * 20
