@@ -73,7 +73,7 @@ typedef struct {
  * count_work, smem_rows, seed_mode, partial_rows or triple_rows selects the
  * tree form, which these fields describe. */
 typedef struct {
-    int ctas_per_sm;       /* resident CTAs of the verification kernel per SM */
+    int ctas_per_sm;       /* resident CTAs of the verification (or sieve) kernel per SM */
     int chunk_work;        /* target work of one queue item, in candidate units */
     int grab;              /* tree-node filter: 0 = the tuned value, else 1;
                               1 = by words of up to 32 nodes, a row at a time

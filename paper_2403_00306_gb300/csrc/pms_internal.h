@@ -230,7 +230,8 @@ cudaError_t sieve_init_tables();
 // the quorum form (5 with mid 4 or 5, 7 with mid 3), 0 for q = n. share (q = n):
 // 1 a warp per block; 8 a CTA per block, its warps split every sequence's
 // windows (mid 5, 6); 0 a CTA per block, its warps split the sequences (mid 3, 4).
-cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, int sms, cudaStream_t st);
+// per_sm: CTAs per SM at most, 0: as many as fit.
+cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, int sms, int per_sm, cudaStream_t st);
 
 // ---------------------------------------------------------------- general alphabets (pms_sigma.cu)
 //

@@ -1233,7 +1233,7 @@ static int enqueue_plan(pms_ctx *h, const Plan &P, const uint8_t *d_seq_src, Sta
         sp.flags = d_flags;
         sp.key_count = (uint32_t *)(dc + cl.key_count);
         sp.buckets = (uint32_t *)(dc + cl.buckets);
-        if ((e = launch_sieve(sp, L.mid, L.planes, L.share, h->num_sms, st)) != cudaSuccess)
+        if ((e = launch_sieve(sp, L.mid, L.planes, L.share, h->num_sms, h->opt.ctas_per_sm, st)) != cudaSuccess)
             return h->cuda_fail(e, "sieve kernel");
     }
     if (P.pair_mode && P.total_pair_items > 0) {
@@ -1952,6 +1952,7 @@ struct Served {
     long long rows_cap = 0;
     int blocks = 0;        // CTAs the row scratch has room for
     int occ[2] = {1, 1};   // CTAs per SM of the verification kernel and of its small-rows form
+    int per_sm = 0;        // pms_options.ctas_per_sm
     std::vector<cudaEvent_t> wave_ev;   // in-flight waves
     std::string fatal;
     long long waves = 0, max_reqs_per_wave = 0, overlapped_waves = 0;
@@ -2035,6 +2036,7 @@ static int served_start(pms_ctx *h)
         cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     for (int i = S->slots - 1; i >= 0; --i)
         S->free_slots.push_back(i);
+    S->per_sm = h->opt.ctas_per_sm;
     for (int f = 0; f < 2; ++f) {
         S->occ[f] = std::max(1, f ? h->occ_small[0] : h->occ[0]);
         if (h->opt.ctas_per_sm > 0)
@@ -2382,7 +2384,8 @@ static void served_loop(Served *S)
                     sp.key_count = srv_keycnt(S);
                     // a launch with few blocks gives each a CTA
                     const bool few = sp.total < 16ll * h->num_sms;
-                    e = launch_sieve(sp, j + 3, 0, !few ? 1 : j >= 2 ? 8 : 0, h->num_sms, S->st);
+                    e = launch_sieve(sp, j + 3, 0, !few ? 1 : j >= 2 ? 8 : 0, h->num_sms, S->per_sm,
+                                     S->st);
                 }
                 cudaEventRecord(S->ring_ev[rp], S->st);
                 for (Request *r : finishing) {

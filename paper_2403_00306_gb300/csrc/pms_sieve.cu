@@ -886,18 +886,19 @@ cudaError_t launch_kernel(void (*kernel)(SieveParams), const SieveParams &p, lon
 }
 
 template <int kMid, int kPlanes, int kShare, int kMinBlocks>
-cudaError_t launch(const SieveParams &p, int sms, int reserved, cudaStream_t st)
+cudaError_t launch(const SieveParams &p, int sms, int per_sm, int reserved, cudaStream_t st)
 {
     const long long teams = kSvWarps / kShare;
     return launch_kernel(sieve_kernel<kMid, kPlanes, kShare, kMinBlocks>, p,
-                         std::min<long long>((long long)sms * kMinBlocks, (p.total + teams - 1) / teams),
+                         std::min<long long>((long long)sms * std::min(kMinBlocks, per_sm), (p.total + teams - 1) / teams),
                          sv_smem_bytes<kMid>(reserved, sv_buffers<kMid, kPlanes, kShare>()), st);
 }
 
 template <int kMid, int kMinBlocks>
-cudaError_t launch_split(const SieveParams &p, int sms, int reserved, cudaStream_t st)
+cudaError_t launch_split(const SieveParams &p, int sms, int per_sm, int reserved, cudaStream_t st)
 {
-    return launch_kernel(sieve_split_kernel<kMid, kMinBlocks>, p, std::min<long long>((long long)sms * kMinBlocks, p.total),
+    return launch_kernel(sieve_split_kernel<kMid, kMinBlocks>, p,
+                         std::min<long long>((long long)sms * std::min(kMinBlocks, per_sm), p.total),
                          sv_smem_bytes<kMid, kSplitWarps>(reserved, kSplitWarps), st, 32 * kSplitWarps);
 }
 
@@ -934,7 +935,7 @@ cudaError_t sieve_init_tables()
     return cudaMemcpyToSymbol(g_sv_ball, tables.ball, sizeof tables.ball);
 }
 
-cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, int sms, cudaStream_t st)
+cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, int sms, int per_sm, cudaStream_t st)
 {
     int dev = 0, reserved = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -942,17 +943,19 @@ cudaError_t launch_sieve(const SieveParams &p, int mid, int planes, int share, i
         e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     if (e != cudaSuccess)
         return e;
+    if (per_sm <= 0)
+        per_sm = 1 << 16;
     if (planes > 0)
-        return mid == 5   ? launch<5, 5, 8, 3>(p, sms, reserved, st)
-               : mid == 4 ? launch<4, 5, 1, 2>(p, sms, reserved, st)
-                          : launch<3, 7, 1, 3>(p, sms, reserved, st);
+        return mid == 5   ? launch<5, 5, 8, 3>(p, sms, per_sm, reserved, st)
+               : mid == 4 ? launch<4, 5, 1, 2>(p, sms, per_sm, reserved, st)
+                          : launch<3, 7, 1, 3>(p, sms, per_sm, reserved, st);
     if (mid == 6)
-        return launch<6, 0, 8, 4>(p, sms, reserved, st);
+        return launch<6, 0, 8, 4>(p, sms, per_sm, reserved, st);
     if (mid == 5)
-        return share == 1 ? launch<5, 0, 1, 2>(p, sms, reserved, st) : launch<5, 0, 8, 4>(p, sms, reserved, st);
+        return share == 1 ? launch<5, 0, 1, 2>(p, sms, per_sm, reserved, st) : launch<5, 0, 8, 4>(p, sms, per_sm, reserved, st);
     if (mid == 4)
-        return share == 1 ? launch<4, 0, 1, 4>(p, sms, reserved, st) : launch_split<4, 2>(p, sms, reserved, st);
-    return share == 1 ? launch<3, 0, 1, 5>(p, sms, reserved, st) : launch_split<3, 2>(p, sms, reserved, st);
+        return share == 1 ? launch<4, 0, 1, 4>(p, sms, per_sm, reserved, st) : launch_split<4, 2>(p, sms, per_sm, reserved, st);
+    return share == 1 ? launch<3, 0, 1, 5>(p, sms, per_sm, reserved, st) : launch_split<3, 2>(p, sms, per_sm, reserved, st);
 }
 
 }  // namespace pms

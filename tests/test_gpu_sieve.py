@@ -179,3 +179,22 @@ def test_raw_count_beyond_32_bits():
         with pytest.raises(pms.PMSError) as e:
             c.solve(seqs, l, d)
         assert e.value.code == pms.PMS_ETOOMANY
+
+
+@pytest.mark.parametrize("case", [(20, 1000, 13, 4), (20, 800, 15, 4), (20, 600, 11, 3)], ids=str)
+def test_ctas_per_sm_bounds_the_sieve(case):
+    """One CTA per multiprocessor: the same motifs, later (but in the form for few blocks, whose 256 CTAs
+    are hardly more than one for each)."""
+    n, m, l, d = case
+    seqs = pi.planted_instance(n, m, l, d, 3).seqs
+    got, ms = [], []
+    for per_sm in (0, 1):
+        with pms.Context(0) as c:
+            c.set_options(ctas_per_sm=per_sm, graph=-1)
+            times = []
+            for _ in range(5):
+                got.append(c.solve(seqs, l, d))
+                times.append(c.stats()["ms_verify"])
+            ms.append(min(times))
+    assert all(np.array_equal(g, got[0]) for g in got)
+    assert l == 11 or ms[1] > 1.2 * ms[0]
