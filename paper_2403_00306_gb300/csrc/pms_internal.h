@@ -62,6 +62,7 @@ struct InstDev {
                            //   ranges of words. -1: ranges of nodes
     int sieve_mid;         // sieve form: middle letters of a block (pms_sieve.cu); its window words are
                            //   then stored in place of the planes. 0: the tree form
+    int pad;               // 0: the bytes are part of a captured graph's key
 };
 
 // A contiguous range of queue items: chunks [chunk_lo, chunk_hi) of instance

@@ -22,6 +22,7 @@
 #include <string>
 #include <thread>
 #include <tuple>
+#include <type_traits>
 #include <unordered_map>
 #include <vector>
 
@@ -1434,7 +1435,10 @@ static int enqueue_plan_graph(pms_ctx *h, const Plan &P, const uint8_t *d_seq_sr
     if (h->opt.graph < 0 || count_mode)
         return enqueue_plan(h, P, d_seq_src, status_out, dense_out, dense_cap, count_mode);
     MetaLayout ml(P);
-    // key: options, the verification kernel's grid, the descriptors
+    // key: options, the verification kernel's grid, the descriptors, byte by byte, so these have no padding
+    static_assert(std::has_unique_object_representations_v<InstDev> &&
+                  std::has_unique_object_representations_v<Segment> &&
+                  std::has_unique_object_representations_v<SieveSeg>);
     std::string key((const char *)&h->opt, sizeof h->opt);
     const int blocks = plan_blocks(h, P, count_mode);
     key.append((const char *)&blocks, sizeof blocks);
