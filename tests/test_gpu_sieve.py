@@ -198,3 +198,46 @@ def test_ctas_per_sm_bounds_the_sieve(case):
             ms.append(min(times))
     assert all(np.array_equal(g, got[0]) for g in got)
     assert l == 11 or ms[1] > 1.2 * ms[0]
+
+
+# (n, m, l, d, q, alone) by the form that the runtime takes for them on 152 multiprocessors (test_sieve_forms_host.py
+# holds it to that): middle letters, counter planes, warps per block. Windows a sequence at and around the
+# multiples of 32 and 256, one window, numbers of sequences around a CTA's warps and what the planes count
+# up to, quorums of one, of about half and of all but one.
+FORMS = {
+    (3, 0, 0): [(2, 10, 6, 1, 2, 1), (3, 8, 8, 1, 3, 1), (7, 36, 6, 2, 7, 1), (8, 39, 8, 3, 8, 1), (20, 41, 9, 2, 20, 1),
+                (31, 72, 9, 3, 31, 1), (21, 74, 10, 4, 21, 1)],
+    (3, 0, 1): [(21, 10, 6, 2, 21, 0), (2, 260, 6, 1, 2, 0), (3, 38, 8, 3, 3, 0), (9, 41, 10, 3, 9, 0),
+                (20, 607, 8, 1, 20, 0), (31, 72, 10, 4, 31, 0)],
+    (4, 0, 0): [(2, 11, 11, 2, 2, 1), (3, 15, 11, 3, 3, 1), (7, 41, 11, 4, 7, 1), (8, 42, 11, 5, 8, 1), (9, 43, 11, 2, 9, 1),
+                (33, 75, 11, 2, 33, 1)],
+    (4, 0, 1): [(3, 11, 11, 6, 3, 0), (2, 15, 11, 5, 2, 0), (8, 41, 11, 4, 8, 0), (9, 43, 12, 4, 9, 0), (20, 44, 12, 5, 20, 0),
+                (31, 75, 11, 3, 31, 0)],
+    (5, 0, 1): [(8, 18, 14, 6, 8, 0), (7, 77, 13, 4, 7, 0), (3, 45, 14, 5, 3, 1), (9, 45, 13, 5, 9, 0), (21, 270, 14, 4, 21, 0),
+                (31, 114, 15, 5, 31, 1), (33, 76, 13, 4, 33, 0)],
+    (5, 0, 8): [(2, 12, 12, 1, 2, 1), (7, 17, 13, 2, 7, 1), (9, 44, 12, 3, 9, 1), (3, 43, 13, 4, 3, 1), (8, 43, 12, 4, 8, 1),
+                (21, 76, 12, 5, 21, 1), (31, 75, 13, 5, 31, 1)],
+    (6, 0, 8): [(2, 268, 14, 1, 2, 1), (3, 269, 14, 4, 3, 0), (7, 413, 14, 1, 7, 1), (20, 268, 14, 1, 20, 1)],
+    (3, 7, 1): [(20, 6, 6, 3, 19, 0), (3, 10, 6, 4, 2, 1), (64, 30, 6, 1, 1, 0), (64, 73, 8, 2, 63, 0), (63, 71, 8, 2, 31, 0),
+                (9, 134, 6, 2, 4, 0), (32, 262, 8, 1, 16, 0), (33, 70, 11, 3, 30, 0), (31, 69, 6, 2, 1, 1)],
+    (4, 5, 1): [(8, 17, 13, 5, 7, 0), (20, 12, 12, 5, 18, 0), (9, 76, 12, 3, 4, 0), (31, 20, 12, 4, 30, 0),
+                (21, 44, 12, 4, 10, 1), (31, 76, 14, 4, 15, 1), (20, 77, 14, 5, 10, 0)],
+    (5, 5, 8): [(9, 267, 13, 3, 7, 1), (7, 268, 13, 4, 6, 1), (31, 613, 14, 3, 15, 1), (21, 312, 13, 3, 10, 0),
+                (31, 400, 13, 3, 30, 1), (20, 269, 14, 5, 19, 1)],
+}
+
+
+@pytest.mark.parametrize("form,case", [(f, c) for f in FORMS for c in FORMS[f]], ids=str)
+def test_every_form_at_its_edges(oracle_, form, case):
+    """Each kernel of the sieve: against the oracle where that is quick, and against the tree form."""
+    n, m, l, d, q, alone = case
+    seqs = pi.planted_instance(n, m, l, d, 13).seqs
+    with pms.Context(0) as c, pms.Context(0) as tree:
+        c.set_options(quorum=q)
+        tree.set_options(quorum=q, grab=1)
+        want = tree.solve(seqs, l, d)
+        assert len(want) > 0
+        if l <= 11:
+            assert np.array_equal(want, oracle_.solve_quorum(seqs, l, d, q, cap=1 << 24))
+        for got in [c.solve(seqs, l, d)] if alone else c.solve_batch([(seqs, l, d)] * 3):
+            assert np.array_equal(got, want)
