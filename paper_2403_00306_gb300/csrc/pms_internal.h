@@ -148,7 +148,7 @@ const void *compat_rows_kernel_fn();
 // small_rows: the form with kRowSmemCapSmall row entries in shared memory and
 // 4 resident CTAs per SM (for instances whose seeds have few feasible
 // occurrences); otherwise kRowSmemCap entries and 3 CTAs per SM.
-cudaError_t launch_main(const MainParams &p, int blocks, bool count_mode, cudaStream_t st, bool small_rows = false);
+cudaError_t launch_main(const MainParams &p, int blocks, bool count_mode, cudaStream_t st, bool small_rows, bool words);
 cudaError_t launch_pairs(const MainParams &p, int blocks, bool count_mode, cudaStream_t st);
 cudaError_t pairs_occupancy(int *blocks_per_sm, bool count_mode);
 cudaError_t launch_classify(const InstDev *inst, int ninst, const long long *seed_prefix, long long total_seeds,

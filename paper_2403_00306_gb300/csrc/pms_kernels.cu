@@ -1800,7 +1800,12 @@ __device__ __forceinline__ void build_rows(const MainParams &p, const InstDev &i
 
 // kRowsCap: row entries held in shared memory; kMinBlocks: resident CTAs per
 // SM the register allocation is bounded for (3 with 2560 entries, 4 with 1280).
-template <bool kCount, int kRowsCap, int kMinBlocks>
+// kWords: some instance has a table of node words. Launches without one take a
+// kernel of their own, with fewer spills and without the three-string test of many
+// nodes, which costs where most nodes pass. Walk, us, in the kernel of both and in
+// its own: (13,4), n = 20, m = 300 576 and 539, m = 600 1734 and 1686; (15,5), m = 300
+// 3426 and 3150; (14,4), m = 1200 3387 and 3279; (17,6), m = 300 19746 and 18522.
+template <bool kCount, int kRowsCap, int kMinBlocks, bool kWords>
 __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1826,6 +1831,8 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
         cs.feasible = 0;
         cs.table = -1;
     }
+    if constexpr (!kWords)
+        load_table(cs, 0, 0);
     // launched as a programmatic dependent of the previous kernel: nothing
     // above reads its output; wait here until it has completed and its
     // writes are visible (without the launch attribute this returns at once)
@@ -1881,9 +1888,10 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
         }
         const bool rebuild = (I != cs.cached_inst) || (seed != cs.cached_seed);
         const int table = in.words >= 0 ? in.d + 1 : 0;
-        const bool reload = cs.table != table;
-        if (reload)
-            load_table(cs, table, in.d);
+        if constexpr (kWords) {
+            if (cs.table != table)
+                load_table(cs, table, in.d);
+        }
         if (rebuild) {
             build_rows(p, in, seed, cs, smem_D, smem_HL, glob_D, glob_HL, warp, lane, kCount ? cnt : nullptr,
                        reinterpret_cast<uint32_t *>(smem_raw));
@@ -1892,7 +1900,8 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
                 cs.cached_seed = seed;
             }
         }
-        __syncthreads();   // every thread has compared cs.table
+        if constexpr (kWords)
+            __syncthreads();   // every thread has compared cs.table
         if (threadIdx.x == 0) {
             cs.table = table;
             cs.next = g0;
@@ -1964,17 +1973,24 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
                 walk_init(c);
                 for (;;) {
                     bool fin;
-                    const int qn = in.words >= 0
-                                       ? word_run<kCount>(c, p.ctab + in.words, g0, g1, cs, ctr, base, exh, fin)
-                                       : walk_run<kCount>(c, tab, g0, g1, cs, ctr, base, exh, fin);
-                    uint32_t *queue = wsm[warp].subs + 64;
-                    // the walk returns up to 63 nodes, the word filter 32
-                    for (int q0 = 0; q0 < qn; q0 += 32) {
-                        int k = min(32, qn - q0);
-                        if (in.triple_rows > 0 && k >= kPairMin && in.n > 2)
-                            k = pair_filter<kCount>(c, queue + q0, k);
-                        for (int i = 0; i < k; ++i)
-                            expand_subset<kCount>(c, queue[q0 + i]);
+                    if constexpr (kWords) {
+                        const int qn = in.words >= 0
+                                           ? word_run<kCount>(c, p.ctab + in.words, g0, g1, cs, ctr, base, exh, fin)
+                                           : walk_run<kCount>(c, tab, g0, g1, cs, ctr, base, exh, fin);
+                        uint32_t *queue = wsm[warp].subs + 64;
+                        // the walk returns up to 63 nodes, the word filter 32
+                        for (int q0 = 0; q0 < qn; q0 += 32) {
+                            int k = min(32, qn - q0);
+                            if (in.triple_rows > 0 && k >= kPairMin && in.n > 2)
+                                k = pair_filter<kCount>(c, queue + q0, k);
+                            for (int i = 0; i < k; ++i)
+                                expand_subset<kCount>(c, queue[q0 + i]);
+                        }
+                    } else {
+                        const int qn = walk_run<kCount>(c, tab, g0, g1, cs, ctr, base, exh, fin);
+                        const uint32_t *queue = wsm[warp].subs + 64;
+                        for (int i = 0; i < qn; ++i)
+                            expand_subset<kCount>(c, queue[i]);
                     }
                     __syncwarp();
                     if (fin)
@@ -3138,15 +3154,26 @@ size_t main_smem_bytes(bool small_rows)
 
 namespace {
 
+template <bool kCount, int kRowsCap, int kMinBlocks, bool kWords>
+cudaError_t occupancy_of(int *blocks_per_sm, size_t smem)
+{
+    const auto kernel = main_kernel<kCount, kRowsCap, kMinBlocks, kWords>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess)
+        return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, kMainThreads, smem);
+}
+
+// of the kernels with and without words, which are bounded for the same number
 template <bool kCount, int kRowsCap, int kMinBlocks>
 cudaError_t occupancy_of(int *blocks_per_sm, size_t smem)
 {
-    cudaError_t e = cudaFuncSetAttribute(main_kernel<kCount, kRowsCap, kMinBlocks>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess)
-        return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_kernel<kCount, kRowsCap, kMinBlocks>,
-                                                         kMainThreads, smem);
+    int words = 0;
+    cudaError_t e = occupancy_of<kCount, kRowsCap, kMinBlocks, true>(&words, smem);
+    if (e == cudaSuccess)
+        e = occupancy_of<kCount, kRowsCap, kMinBlocks, false>(blocks_per_sm, smem);
+    *blocks_per_sm = std::min(*blocks_per_sm, words);
+    return e;
 }
 
 }  // namespace
@@ -3161,19 +3188,20 @@ cudaError_t main_occupancy(int *blocks_per_sm, bool count_mode, bool small_rows)
                       : occupancy_of<false, kRowSmemCap, kMinBlocksLarge>(blocks_per_sm, smem);
 }
 
-cudaError_t launch_main(const MainParams &p, int blocks, bool count_mode, cudaStream_t st, bool small_rows)
+cudaError_t launch_main(const MainParams &p, int blocks, bool count_mode, cudaStream_t st, bool small_rows, bool words)
 {
     const size_t smem = main_smem_bytes(small_rows);
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = dependent_launch(attr, blocks, kMainThreads, smem, st);
-    if (small_rows) {
-        if (count_mode)
-            return cudaLaunchKernelEx(&cfg, main_kernel<true, kRowSmemCapSmall, kMinBlocksSmall>, p);
-        return cudaLaunchKernelEx(&cfg, main_kernel<false, kRowSmemCapSmall, kMinBlocksSmall>, p);
-    }
-    if (count_mode)
-        return cudaLaunchKernelEx(&cfg, main_kernel<true, kRowSmemCap, kMinBlocksLarge>, p);
-    return cudaLaunchKernelEx(&cfg, main_kernel<false, kRowSmemCap, kMinBlocksLarge>, p);
+    const auto of = [&](auto with, auto without) { return cudaLaunchKernelEx(&cfg, words ? with : without, p); };
+    constexpr int kSmall = kRowSmemCapSmall, kLarge = kRowSmemCap;
+    if (small_rows)
+        return count_mode ? of(main_kernel<true, kSmall, kMinBlocksSmall, true>, main_kernel<true, kSmall, kMinBlocksSmall, false>)
+                          : of(main_kernel<false, kSmall, kMinBlocksSmall, true>,
+                               main_kernel<false, kSmall, kMinBlocksSmall, false>);
+    return count_mode ? of(main_kernel<true, kLarge, kMinBlocksLarge, true>, main_kernel<true, kLarge, kMinBlocksLarge, false>)
+                      : of(main_kernel<false, kLarge, kMinBlocksLarge, true>,
+                           main_kernel<false, kLarge, kMinBlocksLarge, false>);
 }
 
 cudaError_t launch_compat(const InstDev *inst, int ninst, const long long *row_prefix, long long total_rows,

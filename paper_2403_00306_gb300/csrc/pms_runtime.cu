@@ -568,14 +568,17 @@ struct pms_ctx {
 
     // The word table of (l, d), without words where the node walk is taken: by
     // other node filters, quorums, trees of more than kMaxWordNodes nodes and
-    // where most nodes pass a row (near: expected_near), so that the walk's exit at
+    // where so many nodes pass a row (near: expected_near) that the walk's exit at
     // a row's first hit saves more than a word does. Tree form, us, walk and words:
-    // (12,3) E = 0.23 107 and 125, E = 0.47 478 and 734; (13,4) E = 0.19 370 and
-    // 300; (15,4) E = 0.07 113 and 86.
+    // (12,3) E = 0.15 65 and 61, E = 0.19 85 and 87, E = 0.47 468 and 731; (13,4)
+    // E = 0.14 162 and 148, E = 0.19 322 and 365; (14,4) E = 0.20 744 and 698, E = 0.41
+    // 3279 and 3659; (15,5) E = 0.15 1281 and 1132, E = 0.23 3150 and 3568; (16,5) E = 0.17
+    // 5670 and 4925, E = 0.25 14698 and 16348; (17,6) E = 0.12 5046 and 5164, E = 0.18 18522
+    // and 20808; (18,6) E = 0.14 49731 and 54076; (15,4) E = 0.07 117 and 93.
     const WordTable &words(int l, int d, bool walk, double near)
     {
         static const WordTable none;
-        if (!walk || near >= 0.2)
+        if (!walk || near >= (l <= 13 ? 0.16 : d >= 6 ? 0.11 : 0.2))
             return none;
         const auto key = std::make_pair(l, d);
         auto it = word_cache.find(key);
@@ -664,6 +667,7 @@ struct Plan {
     std::vector<long long> win_prefix;
     std::vector<long long> row_prefix;   // compatibility rows: sum of W * (n - 1)
     bool small_rows = false;             // verification kernel in its small-rows form (4 CTAs per SM)
+    bool words = false;                  // an instance in tree form has a table of node words
     std::vector<long long> seed_prefix;  // seeds: sum of W
     std::vector<Segment> seg_pair;       // pair-form queue (blocks of 64 windows of s_2 per seed)
     long long total_pair_items = 0;
@@ -1028,6 +1032,7 @@ static Plan make_plan(pms_ctx *h, const std::vector<InstSpec> &specs)
         };
         in.ctab = table(ct.tab);
         in.words = wt.words > 0 ? table(wt.tab) : -1;
+        P.words |= in.words >= 0;
         in.seq_off = (long long)P.seq_bytes;
         P.seq_bytes += round_up((size_t)s.n * s.m, 16);
         in.plane_off = (long long)P.planes;
@@ -1218,7 +1223,7 @@ static int enqueue_plan(pms_ctx *h, const Plan &P, const uint8_t *d_seq_src, Sta
     mp.item_claim = (int *)(dc + cl.claim);
     mp.steal_state = (unsigned int *)(dc + cl.steal);
     record_event(h, h->evm0, st, meta_dev != nullptr);
-    if (P.total_items > 0 && (e = launch_main(mp, blocks, count_mode, st, P.small_rows)) != cudaSuccess)
+    if (P.total_items > 0 && (e = launch_main(mp, blocks, count_mode, st, P.small_rows, P.words)) != cudaSuccess)
         return h->cuda_fail(e, "verification kernel");
     for (size_t j = 0; j < P.sieve.size(); ++j) {
         const Plan::SieveLaunch &L = P.sieve[j];
@@ -2273,6 +2278,7 @@ static void served_loop(Served *S)
             double units = 0;
             long long need_rows = 0;
             bool small = S->occ[1] > S->occ[0];   // the small-rows form, by the rule of make_plan
+            bool words = false;
             for (Request *r : S->active) {
                 if (r->state != 1 || r->chunks_next >= r->chunks_total)
                     continue;
@@ -2295,6 +2301,7 @@ static void served_loop(Served *S)
                     continue;
                 }
                 segs.push_back(Segment{items, r->slot, (int)r->chunks_next, (int)(r->chunks_next + take), 0});
+                words |= S->h_inst[r->slot].words >= 0;
                 r->chunks_next += take;
                 items += take;
                 units += take * r->units_per_chunk;
@@ -2371,7 +2378,7 @@ static void served_loop(Served *S)
                     ctas = std::min(ctas, items);
                 }
                 if (e == cudaSuccess && items > 0)
-                    e = launch_main(mp, (int)ctas, false, S->st, small);
+                    e = launch_main(mp, (int)ctas, false, S->st, small, words);
                 for (int j = 0; j < 4 && e == cudaSuccess; ++j) {
                     if (sieve_segs[j].empty())
                         continue;
@@ -3483,7 +3490,7 @@ extern "C" int pms_solve_device_noalloc(const uint8_t *d_seqs, int n, int m, int
     mp.rows_cap = (int)rows_cap;
     mp.smem_rows_cap = kRowSmemCap;
     mp.counters = (unsigned long long *)(dc + cl.work);
-    if ((e = launch_main(mp, blocks, false, st)) != cudaSuccess)
+    if ((e = launch_main(mp, blocks, false, st, false, false)) != cudaSuccess)
         return PMS_ECUDA;
     const uint32_t cap = (uint32_t)std::min<size_t>(capacity, 0xffffffffu);
     if ((e = launch_sort_unique(d_inst, nullptr, 1, (uint64_t *)(base + o_raw), (uint64_t *)(base + o_tmp), d_rawcnt,

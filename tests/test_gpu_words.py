@@ -39,3 +39,16 @@ def test_words_and_batches_agree(case):
             got.append(c.solve(seqs, l, d))
     assert len(got[0]) > 0
     assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
+
+
+def test_walk_and_words_in_one_launch(oracle_):
+    """Batches in tree form of instances with words of nodes ((15,4), (17,5)), of instances whose nodes are
+    walked one by one ((9,2), (13,4), (12,3)) and of both."""
+    words = [(pi.planted_instance(8, 60, 15, 4, 3).seqs, 15, 4), (pi.planted_instance(6, 30, 17, 5, 4).seqs, 17, 5)]
+    walk = [(pi.planted_instance(5, 400, 9, 2, 5).seqs, 9, 2), (pi.planted_instance(10, 220, 13, 4, 6).seqs, 13, 4),
+            (pi.planted_instance(6, 500, 12, 3, 7).seqs, 12, 3)]
+    with pms.Context(0) as c:
+        c.set_options(grab=1)
+        for batch in (words, walk, [walk[0], words[0], walk[1], words[1], walk[2], words[0]]):
+            for (seqs, l, d), got in zip(batch, c.solve_batch(batch)):
+                assert np.array_equal(got, oracle_.solve_packed(seqs, l, d)), (l, d)
