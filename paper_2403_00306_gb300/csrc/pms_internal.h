@@ -296,6 +296,7 @@ struct SigmaSieve {
     int warp_words;     // map words of a warp
     int map_words;      // map words of a CTA
     int row_bytes;      // shared or scratch bytes of a row
+    int shares;         // warps that share the windows of a sequence
 };
 constexpr int kSsMaskWords = 2048;             // row masks of one seed kept in shared memory
 constexpr int kSsSmemMax = 200 * 1024;         // dynamic shared memory of a CTA at most

@@ -399,11 +399,16 @@ __device__ __forceinline__ uint32_t ss_unrank(int r, int l)
 // seed. Rows: a pass over every window sets a mask bit for those within 2d (kept
 // in shared memory where it has room) and counts them per sequence, a second
 // stores their masks and letters, in shared memory where they fit.
-template <int kQuads, int kMinBlocks>
+//
+// kSplit: several warps share the windows of a sequence, in groups of 128. With few
+// sequences a seed's rows would otherwise wait for one warp each: (9,1), 20 letters,
+// n = 2, m = 8000, whole solves, 760 us without and 235 us with it. A kernel of its
+// own, as the shares' bookkeeping costs the others 2 % ((9,4), n = 20, 2.55 and 2.60 ms).
+template <int kQuads, int kMinBlocks, bool kSplit>
 __global__ void __launch_bounds__(kSsThreads, kMinBlocks) sigma_sieve_kernel(SigmaParams p, SigmaSieve q)
 {
     extern __shared__ __align__(16) unsigned char ss_raw[];
-    __shared__ int s_cnt[kNMax], s_off[kNMax + 1], s_order[kNMax];
+    __shared__ int s_cnt[kNMax], s_off[kNMax + 1], s_order[kNMax], s_part[kNMax];
     __shared__ int s_item, s_next, s_skip;
     __shared__ unsigned long long s_ct[kSgCntNum];
     // the warps' maps, their lists (the masks of a seed's rows while these are collected), the rows
@@ -419,6 +424,11 @@ __global__ void __launch_bounds__(kSsThreads, kMinBlocks) sigma_sieve_kernel(Sig
     const int NWm = (p.W + 31) / 32;
     const bool masks = p.n * NWm <= kSsMaskWords;
     const size_t NW = (size_t)p.n * p.W;
+    // warps that share a sequence, and the first group of 32 windows of the u-th of them
+    auto shares = [&] { return kSplit ? q.shares : 1; };
+    auto first_of = [&](int u) { return kSplit ? min(4 * (u * ((NWm + 3) / 4) / q.shares), NWm) : u * NWm; };
+    if (tid == 0)
+        s_cnt[0] = 0;
     for (;;) {
         if (tid == 0)
             s_item = (int)atomicAdd(p.head, 1u);
@@ -440,28 +450,37 @@ __global__ void __launch_bounds__(kSsThreads, kMinBlocks) sigma_sieve_kernel(Sig
                     mm |= x[g] ^ __ldg(at + g * NW);
             return mm;
         };
-        for (int i = warp; i < p.n; i += kSsWarps) {
+        for (int t = warp; t < (p.n - 1) * shares(); t += kSsWarps) {
+            const int i = 1 + t / shares(), part_of = t % shares();
+            const int c1 = first_of(part_of + 1);
             int cnt = 0;
-            if (i != 0)
-                for (int c0 = 0; c0 < NWm; c0 += 4) {
-                    // four groups of 32 windows, their loads in flight together
-                    uint32_t mm[4];
+            for (int c0 = first_of(part_of); c0 < c1; c0 += 4) {
+                // four groups of 32 windows, their loads in flight together
+                uint32_t mm[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        mm[u] = differs(i, min(32 * (c0 + u) + lane, p.W - 1));
+                for (int u = 0; u < 4; ++u)
+                    mm[u] = differs(i, min(32 * (c0 + u) + lane, p.W - 1));
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const uint32_t bal =
-                            __ballot_sync(kFull, 32 * (c0 + u) + lane < p.W && __popc(mm[u]) <= 2 * p.d);
-                        if (masks && lane == 0 && c0 + u < NWm)
-                            s_mask[i * NWm + c0 + u] = bal;
-                        cnt += __popc(bal);
-                    }
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t bal = __ballot_sync(kFull, 32 * (c0 + u) + lane < p.W && __popc(mm[u]) <= 2 * p.d);
+                    if (masks && lane == 0 && c0 + u < NWm)
+                        s_mask[i * NWm + c0 + u] = bal;
+                    cnt += __popc(bal);
                 }
+            }
             if (lane == 0)
-                s_cnt[i] = cnt;
+                (shares() > 1 ? s_part[t] : s_cnt[i]) = cnt;
         }
         __syncthreads();
+        if (shares() > 1) {
+            if (tid >= 1 && tid < p.n) {
+                int cnt = 0;
+                for (int u = 0; u < shares(); ++u)
+                    cnt += s_part[(tid - 1) * shares() + u];
+                s_cnt[tid] = cnt;
+            }
+            __syncthreads();
+        }
         if (tid == 0) {
             int o = 0, empty = 0;
             for (int i = 0; i < p.n; ++i) {
@@ -495,10 +514,14 @@ __global__ void __launch_bounds__(kSsThreads, kMinBlocks) sigma_sieve_kernel(Sig
                 L = reinterpret_cast<unsigned long long *>(base);   // scratch_rows is even
                 D = joint ? nullptr : base + 2 * (size_t)p.scratch_rows;
             }
-            for (int i = 1 + warp; i < p.n; i += kSsWarps) {
+            for (int t = warp; t < (p.n - 1) * shares(); t += kSsWarps) {
+                const int i = 1 + t / shares(), part_of = t % shares();
+                const int c1 = first_of(part_of + 1);
                 int e = s_off[i];
+                for (int u = 0; u < part_of; ++u)
+                    e += s_part[t - part_of + u];
 #pragma unroll 2
-                for (int c = 0; c < NWm; ++c) {
+                for (int c = first_of(part_of); c < c1; ++c) {
                     const int w = 32 * c + lane;
                     uint32_t bal;
                     if (masks)
@@ -561,7 +584,9 @@ using SsKernel = void (*)(SigmaParams, SigmaSieve);
 // 16 words a lane hold up to 22 letters (484 words); 32 letters need 32.
 SsKernel ss_kernel(const SigmaSieve &q)
 {
-    return q.warp_words <= 512 ? sigma_sieve_kernel<4, 3> : sigma_sieve_kernel<8, 2>;
+    if (q.shares > 1)
+        return q.warp_words <= 512 ? sigma_sieve_kernel<4, 3, true> : sigma_sieve_kernel<8, 2, true>;
+    return q.warp_words <= 512 ? sigma_sieve_kernel<4, 3, false> : sigma_sieve_kernel<8, 2, false>;
 }
 
 }  // namespace
@@ -573,6 +598,7 @@ bool sigma_sieve_plan(int n, int l, int d, int b, int sigma, SigmaSieve *q)
     q->warp_words = sigma * sigma <= 512 ? 512 : 1024;
     q->map_words = kSsWarps * q->warp_words;
     q->row_bytes = (b + 1) * l <= 64 ? 8 : 12;
+    q->shares = std::max(1, kSsWarps / (n - 1));
     return true;
 }
 
@@ -588,7 +614,8 @@ cudaError_t sigma_sieve_init()
         for (int k = 0; k <= 4; ++k)
             binom[a][k] = k == 0 ? 1u : a == 0 ? 0u : binom[a - 1][k - 1] + binom[a - 1][k];
     cudaError_t e = cudaMemcpyToSymbol(g_ss_binom, binom, sizeof binom);
-    for (const SsKernel f : {(SsKernel)sigma_sieve_kernel<4, 3>, (SsKernel)sigma_sieve_kernel<8, 2>})
+    for (const SsKernel f : {(SsKernel)sigma_sieve_kernel<4, 3, false>, (SsKernel)sigma_sieve_kernel<8, 2, false>,
+                             (SsKernel)sigma_sieve_kernel<4, 3, true>, (SsKernel)sigma_sieve_kernel<8, 2, true>})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute((const void *)f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSsSmemMax);
     return e;

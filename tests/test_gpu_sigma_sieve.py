@@ -30,3 +30,22 @@ def test_matches_oracle(oracle_, case):
         assert np.array_equal(got, want), (len(got), len(want))
         c.set_options(ctas_per_sm=1, smem_rows=8)    # few CTAs, rows in global scratch
         assert np.array_equal(c.solve_sigma(inst.seqs, l, d, alphabet), want)
+
+
+# few sequences, whose windows several warps share (W around multiples of 128 and of their shares)
+FEW = [(4, 7, 4, 2, 300), (4, 6, 2, 3, 270), (3, 8, 3, 5, 135), (32, 4, 2, 2, 50),
+       (23, 5, 2, 2, 70), (20, 6, 1, 4, 700), (4, 9, 2, 2, 1300), (20, 6, 2, 9, 260), (20, 9, 1, 2, 2100), (4, 8, 3, 4, 519),
+       (4, 6, 4, 8, 133), (5, 6, 0, 2, 1029), (20, 6, 3, 3, 8)]
+
+
+@pytest.mark.parametrize("case", FEW, ids=str)
+def test_few_sequences_match_oracle(oracle_, case):
+    sigma, l, d, n, m = case
+    alphabet = ALPHABET[:sigma]
+    inst = pi.planted_instance_sigma(n, m, l, d, 6, alphabet)
+    want = oracle_.sigma_solve(inst.seqs, l, d, alphabet)
+    with pms.Context(0) as c:
+        c.set_options(max_motifs=1 << 22)
+        assert np.array_equal(c.solve_sigma(inst.seqs, l, d, alphabet), want)
+        c.set_options(max_motifs=1 << 22, ctas_per_sm=1, smem_rows=8)
+        assert np.array_equal(c.solve_sigma(inst.seqs, l, d, alphabet), want)
