@@ -32,14 +32,15 @@ def test_matches_oracle(oracle_, case):
         assert np.array_equal(c.solve_sigma(inst.seqs, l, d, alphabet), want)
 
 
-# few sequences, whose windows several warps share (W around multiples of 128 and of their shares)
-FEW = [(4, 7, 4, 2, 300), (4, 6, 2, 3, 270), (3, 8, 3, 5, 135), (32, 4, 2, 2, 50),
+# few sequences, whose windows several warps share (W around multiples of 128 and of their shares), and answers
+# of many strings a node
+FEW = [(20, 4, 2, 2, 140), (20, 5, 3, 2, 14), (4, 7, 4, 2, 300), (4, 6, 2, 3, 270), (3, 8, 3, 5, 135), (32, 4, 2, 2, 50),
        (23, 5, 2, 2, 70), (20, 6, 1, 4, 700), (4, 9, 2, 2, 1300), (20, 6, 2, 9, 260), (20, 9, 1, 2, 2100), (4, 8, 3, 4, 519),
-       (4, 6, 4, 8, 133), (5, 6, 0, 2, 1029), (20, 6, 3, 3, 8)]
+       (20, 7, 4, 2, 9), (4, 6, 4, 8, 133), (5, 6, 0, 2, 1029), (20, 6, 3, 3, 8)]
 
 
 @pytest.mark.parametrize("case", FEW, ids=str)
-def test_few_sequences_match_oracle(oracle_, case):
+def test_few_sequences_and_dense_answers_match_oracle(oracle_, case):
     sigma, l, d, n, m = case
     alphabet = ALPHABET[:sigma]
     inst = pi.planted_instance_sigma(n, m, l, d, 6, alphabet)
