@@ -2935,42 +2935,14 @@ int pms_kernel_binary_version(int device, int *version)
     return PMS_OK;
 }
 
-// General alphabets (qPMS-Sigma). Host input, one seed per queue item of the
-// search kernel; the raw key buffer grows once if the first pass overflows it.
-int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_t *seqs, int n, int m, int l, int d,
-                    int q, const uint8_t **motifs, size_t *count)
+// pms_solve_sigma on checked arguments. Host input, one seed per queue item of the
+// search kernel; the raw key buffer grows once if the first pass overflows it. *tuples: take the
+// sieve over a node's tuples of letters where there is one; then, whether it was taken.
+static int solve_sigma(pms_ctx *h, const SigmaMap &map, const SigmaMap &letters, int sigma, const uint8_t *seqs, int n,
+                       int m, int l, int d, int qe, const uint8_t **motifs, size_t *count, double t0, bool *tuples)
 {
-    if (!h)
-        return PMS_EINVAL;
-    std::lock_guard<std::recursive_mutex> g(h->mu);
-    const double t0 = now_ms();
-    h->err.clear();
-    if (!alphabet || !seqs || !motifs || !count)
-        return h->fail(PMS_EINVAL, "null argument");
-    *motifs = nullptr;
-    *count = 0;
-    if (sigma < 2 || sigma > 32)
-        return h->fail(PMS_EINVAL, "sigma = %d outside [2, 32]", sigma);
-    SigmaMap map, letters;
-    memset(map.v, 0xFF, sizeof map.v);
-    memset(letters.v, 0, sizeof letters.v);
-    for (int a = 0; a < sigma; ++a) {
-        if (map.v[alphabet[a]] != 0xFF)
-            return h->fail(PMS_EINVAL, "letter 0x%02x repeated in the alphabet", alphabet[a]);
-        map.v[alphabet[a]] = (uint8_t)a;
-        letters.v[a] = alphabet[a];
-    }
     int rc;
-    if ((rc = check_params(h, n, m, l, d)))
-        return rc;
-    if (d > kSigMaxD)
-        return h->fail(PMS_EINVAL, "d = %d above %d", d, kSigMaxD);
-    if (q < 0 || q > n)
-        return h->fail(PMS_EINVAL, "q = %d outside [0, n]", q);
     const size_t nm = (size_t)n * m;
-    for (size_t i = 0; i < nm; ++i)
-        if (map.v[seqs[i]] == 0xFF)
-            return h->fail(PMS_EINVAL, "byte %zu (0x%02x) is not a letter of the alphabet", i, seqs[i]);
     cudaSetDevice(h->device);
     cudaError_t e;
     if (!h->sigma_ready) {
@@ -2979,7 +2951,6 @@ int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_
             return h->cuda_fail(e, "general-alphabet tables");
         h->sigma_ready = true;
     }
-    const int qe = q == 0 ? n : q;
     const int b = sigma_planes(sigma), W = m - l + 1;
     long long nodes = 0;
     for (int k = 0; k <= d; ++k)
@@ -2998,7 +2969,8 @@ int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_
     const bool large = p_row * max_rows > 0.8 * sigma_smem_rows(b, l, false);
     // the sieve form of a node's letters, and room for about every seed's rows
     SigmaSieve sieve{};
-    const bool sieved = qe == n && sigma_sieve_plan(n, l, d, b, sigma, &sieve);
+    const bool sieved = *tuples && qe == n && sigma_sieve_plan(n, l, d, b, sigma, &sieve);
+    *tuples = sieved;
     int smem_rows = sigma_smem_rows(b, l, large);
     if (sieved) {
         const int most = (int)((kSsSmemMax - sigma_sieve_smem(sieve, 0)) / sieve.row_bytes);
@@ -3182,6 +3154,59 @@ int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_
         return h->fail(PMS_ETOOMANY, "%llu motifs (with duplicates) exceed the capacity; raise max_motifs", raw);
     }
     return PMS_OK;
+}
+
+// General alphabets (qPMS-Sigma).
+int pms_solve_sigma(pms_ctx *h, const uint8_t *alphabet, int sigma, const uint8_t *seqs, int n, int m, int l, int d,
+                    int q, const uint8_t **motifs, size_t *count)
+{
+    if (!h)
+        return PMS_EINVAL;
+    std::lock_guard<std::recursive_mutex> g(h->mu);
+    const double t0 = now_ms();
+    h->err.clear();
+    if (!alphabet || !seqs || !motifs || !count)
+        return h->fail(PMS_EINVAL, "null argument");
+    *motifs = nullptr;
+    *count = 0;
+    if (sigma < 2 || sigma > 32)
+        return h->fail(PMS_EINVAL, "sigma = %d outside [2, 32]", sigma);
+    SigmaMap map, letters;
+    memset(map.v, 0xFF, sizeof map.v);
+    memset(letters.v, 0, sizeof letters.v);
+    for (int a = 0; a < sigma; ++a) {
+        if (map.v[alphabet[a]] != 0xFF)
+            return h->fail(PMS_EINVAL, "letter 0x%02x repeated in the alphabet", alphabet[a]);
+        map.v[alphabet[a]] = (uint8_t)a;
+        letters.v[a] = alphabet[a];
+    }
+    int rc;
+    if ((rc = check_params(h, n, m, l, d)))
+        return rc;
+    if (d > kSigMaxD)
+        return h->fail(PMS_EINVAL, "d = %d above %d", d, kSigMaxD);
+    if (q < 0 || q > n)
+        return h->fail(PMS_EINVAL, "q = %d outside [0, n]", q);
+    const size_t nm = (size_t)n * m;
+    for (size_t i = 0; i < nm; ++i)
+        if (map.v[seqs[i]] == 0xFF)
+            return h->fail(PMS_EINVAL, "byte %zu (0x%02x) is not a letter of the alphabet", i, seqs[i]);
+    const int qe = q == 0 ? n : q;
+    bool tuples = true;
+    rc = solve_sigma(h, map, letters, sigma, seqs, n, m, l, d, qe, motifs, count, t0, &tuples);
+    if (rc == PMS_ENOMEM && tuples && h->budget) {
+        // the tuples' buffers (packed letters, more rows in global memory) do not fit the
+        // memory budget: depth first, which needs less
+        cudaStreamSynchronize(h->stream);
+        for (pms_ctx::DBuf *buf : {&h->d_sg_letters, &h->d_sg_scratch}) {
+            h->dev_free(buf->p, buf->cap);
+            *buf = pms_ctx::DBuf{};
+        }
+        h->err.clear();
+        tuples = false;
+        rc = solve_sigma(h, map, letters, sigma, seqs, n, m, l, d, qe, motifs, count, t0, &tuples);
+    }
+    return rc;
 }
 
 void pms_destroy(pms_ctx *h)

@@ -50,3 +50,26 @@ def test_few_sequences_and_dense_answers_match_oracle(oracle_, case):
         assert np.array_equal(c.solve_sigma(inst.seqs, l, d, alphabet), want)
         c.set_options(max_motifs=1 << 22, ctas_per_sm=1, smem_rows=8)
         assert np.array_equal(c.solve_sigma(inst.seqs, l, d, alphabet), want)
+
+
+def test_memory_budget_that_holds_the_depth_first_form():
+    """A budget that a quorum of n - 1 (searched depth first) just fits also does for q = n: its own buffers
+    (packed letters, and rows in global memory, more than fit on chip here) are not asked for then."""
+    seqs = pi.planted_instance_sigma(3, 500, 9, 2, 4).seqs
+    with pms.Context(0) as c:
+        want = c.solve_sigma(seqs, 9, 2)
+    def fits(budget, q):
+        with pms.Context(0, mem_budget_bytes=budget) as c:
+            try:
+                got = c.solve_sigma(seqs, 9, 2, q=q)
+            except pms.PMSError as e:
+                assert e.code == pms.PMS_ENOMEM
+                return None
+            return got
+    lo, hi = 1 << 20, 1 << 26
+    assert fits(lo, 2) is None and fits(hi, 2) is not None
+    while hi - lo > 4096:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if fits(mid, 2) is not None else (mid, hi)
+    got = fits(hi, 0)
+    assert got is not None and np.array_equal(got, want)
