@@ -508,6 +508,7 @@ struct pms_ctx {
     };
     std::map<std::tuple<int, int, int, int>, Tuning> tuned;
     bool tuning_tree = false;   // the autotuner is timing the tree form
+    bool walk_only = false;     // no tables of node words (see run_planned)
     // sieve_form's estimates by (n, m, l, d, q, single), at most kMaxForms of them
     static constexpr size_t kMaxForms = 1024;
     mutable std::map<std::tuple<int, int, int, int, int, bool>, SieveForm> forms;
@@ -578,7 +579,7 @@ struct pms_ctx {
     const WordTable &words(int l, int d, bool walk, double near)
     {
         static const WordTable none;
-        if (!walk || near >= (l <= 13 ? 0.16 : d >= 6 ? 0.11 : 0.2))
+        if (!walk || walk_only || near >= (l <= 13 ? 0.16 : d >= 6 ? 0.11 : 0.2))
             return none;
         const auto key = std::make_pair(l, d);
         auto it = word_cache.find(key);
@@ -1498,6 +1499,29 @@ static int enqueue_plan_graph(pms_ctx *h, const Plan &P, const uint8_t *d_seq_sr
     return PMS_OK;
 }
 
+// Plans the instances and runs the plan (run: Plan -> code). Where a memory budget
+// refuses a plan with tables of node words (up to 128 KB each), it is made without,
+// and what the first plan sized otherwise is given back before.
+template <class Run>
+static int run_planned(pms_ctx *h, const std::vector<InstSpec> &specs, const Run &run)
+{
+    const Plan P = make_plan(h, specs);
+    const int rc = run(P);
+    if (rc != PMS_ENOMEM || !P.words || !h->budget)
+        return rc;
+    h->err.clear();
+    cudaStreamSynchronize(h->stream);
+    for (pms_ctx::DBuf *buf : {&h->d_meta, &h->d_ctr, &h->d_scratch}) {
+        h->dev_free(buf->p, buf->cap);
+        *buf = pms_ctx::DBuf{};
+    }
+    ++h->buf_gen;   // captured graphs that use them are stale
+    h->walk_only = true;
+    const Plan walk = make_plan(h, specs);
+    h->walk_only = false;
+    return run(walk);
+}
+
 // Records what the host knows of the last solve; device times and counters
 // are read by collect_stats once its events have completed.
 static void begin_stats(pms_ctx *h, const Plan &P, bool count_mode, double t0)
@@ -1665,9 +1689,15 @@ static int solve_specs(pms_ctx *h, std::vector<InstSpec> specs, std::vector<Inst
         std::vector<InstSpec> sub;
         for (int i : todo)
             sub.push_back(specs[i]);
-        Plan P = make_plan(h, sub);
-        candidates += P.candidates;
-        int rc = run_host_plan(h, P, sub, t0);
+        std::vector<InstDev> insts;
+        const int rc = run_planned(h, sub, [&](const Plan &P) {
+            const int e = run_host_plan(h, P, sub, t0);
+            if (e == PMS_OK) {
+                candidates += P.candidates;
+                insts = P.inst;
+            }
+            return e;
+        });
         if (rc)
             return rc;
         const StatusDev *sd = (const StatusDev *)h->h_result;
@@ -1676,11 +1706,11 @@ static int solve_specs(pms_ctx *h, std::vector<InstSpec> specs, std::vector<Inst
         std::vector<int> again;
         for (size_t j = 0; j < sub.size(); ++j) {
             const int idx = todo[j];
-            const uint32_t cap = P.inst[j].raw_cap;
+            const uint32_t cap = insts[j].raw_cap;
             const bool overflow = sd[j].raw_count > cap, invalid = sd[j].flags & kFlagInvalidByte;
             // the sieve stores a motif once, however often it counts: its answer is whole
             // while the buffer has room left, or has room for every string
-            const bool sieve = P.inst[j].sieve_mid > 0;
+            const bool sieve = insts[j].sieve_mid > 0;
             const size_t strings = sieve ? (size_t)1 << (2 * sub[j].l) : 0;
             const bool whole = sieve && !h->opt.max_motifs && (sd[j].unique_count < cap || cap >= strings);
             if (overflow && !whole && !invalid && !h->opt.max_motifs && cap < (1u << 26)) {
@@ -2106,13 +2136,29 @@ static bool served_admit(Served *S, Request *r)
     std::lock_guard<std::recursive_mutex> hg(h->mu);
     const int cw = h->chunk_work_for(r->n, r->m, r->l, r->d);
     const int grab = h->grab_for(r->n, r->m, r->l, r->d);
-    const WordTable *wt = &h->words(r->l, r->d, grab == 1, expected_near(r->m, r->l, r->d));
-    if ((int)wt->tab.size() > Served::kCtabMax / 2)
-        wt = &h->words(r->l, r->d, false, 0.0);
-    const ChunkTable &ct = wt->words > 0 ? h->word_chunks(r->l, r->d, cw > 0 ? cw : kDefaultChunkWork)
-                                         : h->chunks(r->l, r->d, cw > 0 ? cw : kDefaultChunkWork);
-    const size_t ct_ints = round_up(ct.tab.size(), 2);   // the word table's pairs follow
-    const size_t ctab_ints = ct_ints + wt->tab.size();
+    InstSpec spec{r->n, r->m, r->l, r->d, nullptr};
+    r->raw_cap = default_cap(h, spec, true);
+    // the stream's requests share the device, so the form is the one for a launch of many
+    r->form = sieve_form(h, r->n, r->m, r->l, r->d, false);
+    if (r->form.planes != 0)
+        r->form = SieveForm{};   // the served form solves q = n
+    const bool tree = r->form.mid == 0;
+    const WordTable *wt;
+    const ChunkTable *chunks;
+    size_t ct_ints, ctab_ints;
+    auto tables = [&](bool words) {
+        wt = &h->words(r->l, r->d, words, expected_near(r->m, r->l, r->d));
+        chunks = wt->words > 0 ? &h->word_chunks(r->l, r->d, cw > 0 ? cw : kDefaultChunkWork)
+                               : &h->chunks(r->l, r->d, cw > 0 ? cw : kDefaultChunkWork);
+        ct_ints = round_up(chunks->tab.size(), 2);   // the word table's pairs follow
+        ctab_ints = ct_ints + wt->tab.size();
+        return ReqLayout(r->n, r->m, r->W, r->raw_cap, ctab_ints, tree);
+    };
+    ReqLayout L = tables(tree && grab == 1);
+    // words only where their table fits what the walk's request does
+    if (wt->words > 0 && (wt->tab.size() > Served::kCtabMax / 2 || ctab_ints > Served::kCtabMax || L.total > S->pool_bytes))
+        L = tables(false);
+    const ChunkTable &ct = *chunks;
     if ((int)ctab_ints > Served::kCtabMax) {
         r->status = PMS_EINVAL;
         return true;
@@ -2121,14 +2167,6 @@ static bool served_admit(Served *S, Request *r)
         r->status = PMS_ECUDA;
         return true;
     }
-    InstSpec spec{r->n, r->m, r->l, r->d, nullptr};
-    r->raw_cap = default_cap(h, spec, true);
-    // the stream's requests share the device, so the form is the one for a launch of many
-    r->form = sieve_form(h, r->n, r->m, r->l, r->d, false);
-    if (r->form.planes != 0)
-        r->form = SieveForm{};   // the served form solves q = n
-    const bool tree = r->form.mid == 0;
-    ReqLayout L(r->n, r->m, r->W, r->raw_cap, ctab_ints, tree);
     if (L.total > S->pool_bytes) {
         r->status = PMS_ENOMEM;   // can never fit
         return true;
@@ -2608,12 +2646,14 @@ int pms_solve_device(pms_ctx *h, const uint8_t *d_seqs, int n, int m, int l, int
     std::vector<InstSpec> specs{InstSpec{n, m, l, d, nullptr}};
     if ((rc = autotune_missing(h, specs)))
         return rc;
-    Plan P = make_plan(h, specs);
     const uint32_t cap = (uint32_t)std::min<size_t>(capacity, 0xffffffffu);
-    if ((rc = enqueue_plan_graph(h, P, d_seqs, (StatusDev *)d_status, d_motifs, cap, h->opt.count_work != 0)))
-        return rc;
-    begin_stats(h, P, h->opt.count_work != 0, t0);
-    return PMS_OK;
+    const bool count = h->opt.count_work != 0;
+    return run_planned(h, specs, [&](const Plan &P) {
+        const int e = enqueue_plan_graph(h, P, d_seqs, (StatusDev *)d_status, d_motifs, cap, count);
+        if (e == PMS_OK)
+            begin_stats(h, P, count, t0);
+        return e;
+    });
 }
 
 int pms_solve_batch(pms_ctx *h, const pms_instance *inst, int k, pms_result *out)

@@ -52,3 +52,26 @@ def test_walk_and_words_in_one_launch(oracle_):
         for batch in (words, walk, [walk[0], words[0], walk[1], words[1], walk[2], words[0]]):
             for (seqs, l, d), got in zip(batch, c.solve_batch(batch)):
                 assert np.array_equal(got, oracle_.solve_packed(seqs, l, d)), (l, d)
+
+
+def test_memory_budget_that_holds_the_walk(oracle_):
+    """A budget that the batches of nodes just fit also does for the default filter: its table of words,
+    24 KB here, is left out then."""
+    seqs = pi.planted_instance(6, 26, 19, 6, 4).seqs
+    want = oracle_.solve_packed(seqs, 19, 6)
+
+    def fits(budget, **opts):
+        with pms.Context(0, mem_budget_bytes=budget) as c:
+            c.set_options(max_motifs=1 << 12, **opts)
+            try:
+                return c.solve(seqs, 19, 6)
+            except pms.PMSError as e:
+                assert e.code == pms.PMS_ENOMEM
+    lo, hi = 1 << 12, 1 << 24
+    assert fits(lo, grab=32) is None and fits(hi, grab=32) is not None
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if fits(mid, grab=32) is not None else (mid, hi)
+    for opts in ({"grab": 32}, {"grab": 1}):
+        got = fits(hi, **opts)
+        assert got is not None and np.array_equal(got, want), opts
