@@ -700,15 +700,17 @@ __global__ void __launch_bounds__(kSvThreads, kMinBlocks) sieve_kernel(SievePara
                                    out_of(p, blk.I), g, lane);
             share_sync<kShare>();
         }
-        // the strings of a warp's threads, the pieces of one thread at a time
+        // the strings of a warp's threads: of many threads, a string of each at a time; of few,
+        // the pieces of one thread at a time
         uint32_t holders = __ballot_sync(kFull, left != 0u);
         if (holders) {
             __syncwarp();
+            const bool many = __popc(holders) > kPieces / 4;
             while (holders) {
-                const int who = __ffs(holders) - 1;
-                holders &= holders - 1u;
-                for (int k0 = 0; k0 < kPieces; k0 += 32) {
-                    const int k = k0 + lane;
+                const int who = many ? lane : __ffs(holders) - 1;
+                holders = many ? 0u : holders & (holders - 1u);
+                for (int k0 = 0; k0 < kPieces; k0 += many ? 1 : 32) {
+                    const int k = many ? k0 : k0 + lane;
                     const int at = ((k / kVec) * (32 * kShare) + g * 32 + who) * kVec + k % kVec;
                     uint32_t v = k < kPieces ? mw[at] : 0u;
                     while (__any_sync(kFull, v != 0u)) {
