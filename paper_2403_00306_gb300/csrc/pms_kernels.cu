@@ -74,6 +74,7 @@ struct __align__(16) CtaSmem {
         uint32_t near[32][32];
     };
     int table;               // which: 0 the binomials, d + 1 the filter's
+    int dense;               // the seed itself occurs in every sequence
     int row_len[kNMax];      // indexed by sequence
     int row_off[kNMax];      // indexed by sequence: first entry of its row (multiple of 4)
     int row_order[kNMax];    // sequences 1..n-1, smallest row first
@@ -1089,6 +1090,15 @@ __device__ __forceinline__ int walk_run(const WarpCtx &c, const int *tab, int g0
 // eighth of a share 83 and 609; claims of 4 words 97 and 650.
 constexpr unsigned int kLaneNodes = 8;
 constexpr int kMinWords = 8;
+// Words claimed at a time at a seed that itself occurs in every sequence: where sequences
+// repeat themselves all nodes of such seeds pass, their leaves take the time, and a claim of
+// eight words of (15,4), 112 nodes, is more than the item's other warps wait for. And the nodes
+// that an unclaimed word counts for where CTAs look for an item to join. Repetitive sequences,
+// us, walk, words without either, with the hint, with both: (14,4), n = 5, m = 144 1327, 3690,
+// 2685 and 1754; (15,4), n = 20, m = 130 1908, 3791, 3807 and 2155; (16,4), n = 45, m = 244 6976,
+// 14518, 14425 and 7771.
+constexpr int kDenseWords = 2;
+constexpr int kWordHint = 2;
 
 // Appends each lane's nodes (bits of `alive` around U) to q[0..32) in lane order
 // until it is full; returns how many there are in all. `alive` keeps the rest.
@@ -1124,14 +1134,17 @@ __device__ __forceinline__ int word_run(const WarpCtx &c, const int *wtab, int g
     int sh = (int)gs[c.lane];
     finished = false;
     while (!__any_sync(kFull, alive != 0u)) {
-        // claims of an eighth of a warp's share, so that the item's warps end together
+        // claims of an eighth of a warp's share, so that the item's warps end together; of
+        // trees of few words a part for each warp ((14,2), 21 words, repetitive sequences: 252
+        // and 202 us)
         const int nw = (int)(blockDim.x >> 5);
-        const int want = min(32, max(kMinWords, (g1 - g0 + 8 * nw - 1) / (8 * nw)));
+        const int least = min(kMinWords, (wtab[0] + nw - 1) / nw);
+        const int want = cs.dense ? kDenseWords : min(32, max(least, (g1 - g0 + 8 * nw - 1) / (8 * nw)));
         int start = 0;
         if (c.lane == 0) {
             start = claim_base + atomicAdd(claim_ctr, want);
             if (items_out) {
-                claim_ctr[1] = max(0, g1 - (start + want));
+                claim_ctr[1] = kWordHint * max(0, g1 - (start + want));
                 if (start < g1 && start + want >= g1)
                     atomicAdd(items_out, 1u);
             }
@@ -1300,8 +1313,8 @@ __device__ __forceinline__ int pair_filter(const WarpCtx &c, uint32_t *queue, in
     const bool tested = live && ku <= kPairList;   // a longer list: the node passes
     uint32_t us = tested ? (1u << ku) - 1u : 1u;   // the u still possible
     for (int r = 1; r < R; ++r) {
-        const uint32_t left = __ballot_sync(kFull, live);
-        if (__popc(left) <= kPairFew)
+        // a lane whose list is too long tests nothing
+        if (__popc(__ballot_sync(kFull, tested && live)) <= kPairFew)
             break;
         unsigned long long wlo, whi;
         const int offr = c.cs->row_off[c.cs->row_order[r]];
@@ -1893,6 +1906,8 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
                 load_table(cs, table, in.d);
         }
         if (rebuild) {
+            if (kWords && threadIdx.x == 0)
+                cs.dense = 1;
             build_rows(p, in, seed, cs, smem_D, smem_HL, glob_D, glob_HL, warp, lane, kCount ? cnt : nullptr,
                        reinterpret_cast<uint32_t *>(smem_raw));
             if (threadIdx.x == 0) {
@@ -1900,8 +1915,21 @@ __global__ void __launch_bounds__(kMainThreads, kMinBlocks) main_kernel(MainPara
                 cs.cached_seed = seed;
             }
         }
-        if constexpr (kWords)
+        if constexpr (kWords) {
+            if (rebuild && cs.feasible) {
+                const uint4 *D4 = reinterpret_cast<const uint4 *>(cs.rows_in_smem != 0 ? smem_D : glob_D);
+                for (int r = warp; r < in.n - 1 && __any_sync(kFull, *(volatile int *)&cs.dense); r += kMainWarps) {
+                    bool near = false;
+                    for (int e4 = lane; e4 < cs.rank_len4[r]; e4 += 32) {
+                        const uint4 v = D4[cs.rank_off4[r] + e4];
+                        near |= min(min(__popc(v.x), __popc(v.y)), min(__popc(v.z), __popc(v.w))) <= in.d;
+                    }
+                    if (!__any_sync(kFull, near) && lane == 0)
+                        cs.dense = 0;
+                }
+            }
             __syncthreads();   // every thread has compared cs.table
+        }
         if (threadIdx.x == 0) {
             cs.table = table;
             cs.next = g0;

@@ -568,7 +568,9 @@ struct pms_ctx {
     }
 
     // The word table of (l, d), without words where the node walk is taken: by
-    // other node filters, quorums, trees of more than kMaxWordNodes nodes and
+    // other node filters, quorums, trees of more than kMaxWordNodes nodes, trees of so few
+    // (d <= 1) that one round of lanes holds them (repetitive sequences, walk and words:
+    // (13,1), n = 30, m = 1627 2.8 and 4.0 ms; random ones: (13,1), m = 600 54 and 50 us) and
     // where so many nodes pass a row (near: expected_near) that the walk's exit at
     // a row's first hit saves more than a word does. Tree form, us, walk and words:
     // (12,3) E = 0.15 65 and 61, E = 0.19 85 and 87, E = 0.47 468 and 731; (13,4)
@@ -579,7 +581,7 @@ struct pms_ctx {
     const WordTable &words(int l, int d, bool walk, double near)
     {
         static const WordTable none;
-        if (!walk || walk_only || near >= (l <= 13 ? 0.16 : d >= 6 ? 0.11 : 0.2))
+        if (!walk || walk_only || d <= 1 || near >= (l <= 13 ? 0.16 : d >= 6 ? 0.11 : 0.2))
             return none;
         const auto key = std::make_pair(l, d);
         auto it = word_cache.find(key);

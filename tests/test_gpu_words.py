@@ -75,3 +75,19 @@ def test_memory_budget_that_holds_the_walk(oracle_):
     for opts in ({"grab": 32}, {"grab": 1}):
         got = fits(hi, **opts)
         assert got is not None and np.array_equal(got, want), opts
+
+
+@pytest.mark.parametrize("case", [(5, 144, 14, 4), (4, 60, 12, 3), (6, 90, 15, 3), (12, 200, 10, 2), (8, 150, 13, 1)], ids=str)
+def test_repetitive_sequences_match_oracle(oracle_, case):
+    """Runs of one letter and repeats of seven: seeds that occur in every sequence, all of whose nodes pass."""
+    n, m, l, d = case
+    runs = pi.planted_instance(n, m, l, d, 23).seqs.copy()
+    runs[:, m // 4:m // 2] = ord("A")
+    repeats = pi.random_sequences(n, m, 24).copy()
+    repeats[:, m // 3:2 * m // 3] = np.resize(np.frombuffer(b"GATTACA", dtype=np.uint8), 2 * m // 3 - m // 3)
+    for seqs in (runs, repeats):
+        want = oracle_.solve_packed(seqs, l, d)
+        with pms.Context(0) as c:
+            c.set_options(grab=1)
+            assert np.array_equal(c.solve(seqs, l, d), want)
+            assert np.array_equal(c.solve_batch([(seqs, l, d)] * 2)[1], want)
