@@ -913,7 +913,10 @@ static SieveForm estimate_form(const pms_ctx *h, int n, int m, int l, int d, int
                                : !wide          ? 35.0
                                : o.share == 8   ? 12.0 + 0.085 * W * std::max(n, 20) / 20.0
                                                 : ((n + 19) / 20) * (l == 11 ? 14.0 + 0.022 * W : 15.0 + 0.012 * W);
-        const double us = (wide && o.share == 8 ? std::max(latency, 25.0 + marks) : latency + marks) + lookups;
+        // a quorum's block with the most hits goes through all sequences, 32 windows after another
+        const double serial = single && !all && o.share == 1 ? 22.0 + 0.0073 * n * W : 0.0;
+        const double us =
+            (wide && o.share == 8 ? std::max(latency, 25.0 + marks) : std::max(latency + marks, serial)) + lookups;
         if (us < best) {
             best = us;
             form = SieveForm{o.mid, o.planes, o.share, us, motifs};
