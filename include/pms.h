@@ -62,7 +62,7 @@ typedef struct {
 typedef struct {
     int status;             /* PMS_OK or a negative code for this instance */
     const uint64_t *motifs; /* sorted unique motif codes */
-    size_t count;           /* number of motifs (raw count on PMS_ETOOMANY) */
+    size_t count;           /* number of motifs (raw count, at most 2^32 - 1, on PMS_ETOOMANY) */
 } pms_result;
 
 /* Tunables. Zero in any field selects the default (or the tuned value).

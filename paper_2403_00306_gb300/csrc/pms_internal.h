@@ -81,7 +81,7 @@ struct Segment {
 
 // Per-instance status written by the sort/unique kernel.
 struct StatusDev {
-    uint32_t raw_count;    // motifs emitted, duplicates included
+    uint32_t raw_count;    // motifs emitted, duplicates included (2^32 - 1: that many or more)
     uint32_t unique_count; // motifs after sort/unique (written to the dense output)
     uint32_t flags;
     uint32_t dense_off;    // first code of this instance in the dense output
@@ -147,7 +147,8 @@ cudaError_t launch_compat_rows(const InstDev *inst, int n, long long seeds, cons
 const void *compat_rows_kernel_fn();
 // small_rows: the form with kRowSmemCapSmall row entries in shared memory and
 // 4 resident CTAs per SM (for instances whose seeds have few feasible
-// occurrences); otherwise kRowSmemCap entries and 3 CTAs per SM.
+// occurrences); otherwise kRowSmemCap entries and 3 CTAs per SM. words: some
+// instance has a table of node words.
 cudaError_t launch_main(const MainParams &p, int blocks, bool count_mode, cudaStream_t st, bool small_rows, bool words);
 cudaError_t launch_pairs(const MainParams &p, int blocks, bool count_mode, cudaStream_t st);
 cudaError_t pairs_occupancy(int *blocks_per_sm, bool count_mode);

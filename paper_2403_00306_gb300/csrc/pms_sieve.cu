@@ -41,7 +41,7 @@
 // instructions that sort 32 windows by the changes they have left; larger
 // blocks pay them less often. (17,5), n = 20, m = 1200: 5 middle letters and a
 // warp per block 5429 us, 6 letters and a CTA per block 4326 us (now 4102; the tree
-// 11089 us); (15,4) 449 and 392 us (1046 us). With six letters 32 KB of marks
+// 7747 us); (15,4) 449 and 392 us (668 us). With six letters 32 KB of marks
 // serve a CTA of eight warps, and what is lost is their wait for the slowest
 // (5.8 of 14 cycles per instruction), so few windows favour the warp per block.
 #include "pms_sieve.cuh"
